@@ -38,11 +38,11 @@ static void free_all(Context& c)
                     c.ray_mem[0], c.ray_mem[1], c.info, c.ccell, c.cslot, c.newid,
                     c.ent_id, c.ent_src, c.ent_cell, c.sorted_src, c.pj, c.k2, c.kappa, c.raycell, c.ecap, c.cnt, c.off, c.off2,
                     c.overlist, c.biglist, c.scan_tmp, c.dudt_buf, c.dvdt_buf, c.ctl,
-                    c.budget, c.partials, c.flag_dev, c.spec_buf};
+                    c.budget, c.partials, c.flag_dev, c.spec_buf, c.launch_cols};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int f = 0; f < NFIELD; ++f) {
-        if (c.field[f]) cudaFree(c.field[f]);
+        if (f == 0 && c.field[f]) cudaFree(c.field[f]);   // one allocation
         if (c.smooth[f]) cudaFree(c.smooth[f]);
         if (c.nar32[f]) cudaFree(c.nar32[f]);
         if (c.sm32[f]) cudaFree(c.sm32[f]);
@@ -379,8 +379,14 @@ int gwam_init(gwam_ctx** out, const gwam_grid* grid, const gwam_params* params, 
             }
             dalloc(c, c.rho_inv32, ncell);
         }
+        // the projected fields in one allocation, each on a 16-byte boundary (cleared as one range)
+        {
+            size_t at[NFIELD + 1] = {};
+            for (int f = 0; f < NFIELD; ++f) at[f + 1] = at[f] + ((size_t)c.field_len(f) + 1) / 2 * 2;
+            dalloc(c, c.field[0], at[NFIELD]);
+            for (int f = 1; f < NFIELD; ++f) c.field[f] = c.field[0] + at[f];
+        }
         for (int f = 0; f < NFIELD; ++f) {
-            dalloc(c, c.field[f], (size_t)c.field_len(f));
             dalloc(c, c.smooth[f], (size_t)c.field_len(f));
             GWAM_CUDA(cudaMemsetAsync(c.field[f], 0, sizeof(double) * (size_t)c.field_len(f), c.stream));
             GWAM_CUDA(cudaMemsetAsync(c.smooth[f], 0, sizeof(double) * (size_t)c.field_len(f), c.stream));
@@ -391,6 +397,7 @@ int gwam_init(gwam_ctx** out, const gwam_grid* grid, const gwam_params* params, 
         dalloc(c, c.budget, 1);
         dalloc(c, c.partials, (size_t)NTALLY * c.max_blocks);
         dalloc(c, c.flag_dev, 1);
+        dalloc(c, c.launch_cols, 8 * (size_t)G.ncol_all);
         GWAM_CUDA(cudaMallocHost((void**)&c.ctl_host, sizeof(Ctl)));
         GWAM_CUDA(cudaMallocHost((void**)&c.budget_host, sizeof(DevBudget)));
         GWAM_CUDA(cudaMallocHost((void**)&c.flag_host, sizeof(int)));

@@ -23,46 +23,35 @@ __device__ __forceinline__ long long warp_sum(long long v)
 // of by a memset before the projection: that kernel is bound by instruction issue (FP64 form) or by
 // its L1 gathers (precision form) and leaves HBM nearly idle, where the memsets were a pass over
 // all the fields on the step's critical path.  Nothing reads or writes these fields between the
-// advance and the projection.  The FP64 form clears with thread stores after its ray loop
-// (clear_fields); the precision form's gathers would compete with such stores for L1, so there one
+// advance and the projection.  The FP64 form clears with thread stores, a part in every
+// iteration of its ray loop (clear_fields; after the loop they were 32 us of the kernel with the
+// arithmetic idle); the precision form's gathers would compete with such stores for L1, so there one
 // thread per block issues bulk copies of a zeroed shared-memory buffer to the tensor-memory-access
 // unit, a few per iteration of its ray loop (clear_start / clear_issue / clear_finish).
 constexpr int kClearPiece = 16384;  // bytes per bulk copy (measured: 4 KB 0.698, 8 KB 0.607, 16 KB 0.572 ms)
 
+// (the fields lie one after another in one allocation, so a step's fields are one range)
 struct ClearSet {
-    double* p[NFIELD];
-    int64_t n[NFIELD];             // elements of each field
-    int64_t first[NFIELD + 1];     // first piece of each field; first[nf] = all pieces
-    int nf;
+    double2* p;
+    int64_t n;   // 16-byte elements
 };
 
-// the fields the step's projection accumulates into (the two temperature fields only when projected)
+// the fields the step's projection accumulates into (the two temperature fields, the last of the
+// range, only when projected)
 inline ClearSet clear_set(const Context& c)
 {
-    ClearSet z{};
-    z.nf = c.P.theta_flux ? NFIELD : F_TL;
-    z.first[0] = 0;
-    for (int f = 0; f < z.nf; ++f) {
-        z.p[f] = c.field[f];
-        z.n[f] = c.field_len(f);
-        // pieces over the field's whole 16-byte part (an odd last element is stored separately)
-        z.first[f + 1] = z.first[f] + ((z.n[f] >> 1) * 16 + kClearPiece - 1) / kClearPiece;
-    }
-    return z;
+    const int nf = c.P.theta_flux ? NFIELD : F_TL;
+    return ClearSet{reinterpret_cast<double2*>(c.field[0]), (c.field[nf - 1] - c.field[0] + c.field_len(nf - 1) + 1) / 2};
 }
 
-// All threads: grid-stride 16-byte streaming stores of zeros (fields start on 256-byte allocation
-// boundaries; an odd last element is stored by thread 0).
-__device__ __forceinline__ void clear_fields(const ClearSet& z)
+// All threads: 16-byte streaming stores of zeros to the elements of the range that belong to part m
+// of `parts` (grid-stride within the part).
+__device__ __forceinline__ void clear_fields(const ClearSet& z, int m, int parts)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t T = (int64_t)gridDim.x * blockDim.x;
-    for (int f = 0; f < z.nf; ++f) {
-        double2* q = reinterpret_cast<double2*>(z.p[f]);
-        const int64_t n2 = z.n[f] >> 1;
-        for (int64_t i = t; i < n2; i += T) __stcs(q + i, make_double2(0.0, 0.0));
-        if ((z.n[f] & 1) && t == 0) z.p[f][z.n[f] - 1] = 0.0;
-    }
+    const int64_t per = (z.n + parts - 1) / parts;
+    const int64_t end = (m + 1) * per < z.n ? (m + 1) * per : z.n;
+    for (int64_t i = m * per + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < end; i += (int64_t)gridDim.x * blockDim.x)
+        __stcs(z.p + i, make_double2(0.0, 0.0));
 }
 
 struct ClearState {
@@ -71,6 +60,8 @@ struct ClearState {
     uint32_t zbuf;     // shared-memory address of the zeroed buffer
 };
 
+__device__ __forceinline__ int64_t clear_pieces(const ClearSet& z) { return (z.n * 16 + kClearPiece - 1) / kClearPiece; }
+
 // All threads of the block: zero the buffer, make it visible to the bulk-copy unit, and spread the
 // block's pieces over the ray loop of thread 0 (n rays, grid-stride loop).
 __device__ __forceinline__ void clear_start(const ClearSet& z, float4* zbuf, int n, ClearState& st)
@@ -78,7 +69,7 @@ __device__ __forceinline__ void clear_start(const ClearSet& z, float4* zbuf, int
     for (int q = threadIdx.x; q < kClearPiece / 16; q += blockDim.x) zbuf[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    const int64_t total = z.first[z.nf];
+    const int64_t total = clear_pieces(z);
     st.g = blockIdx.x;
     st.zbuf = (uint32_t)__cvta_generic_to_shared(zbuf);
     const int64_t mine = st.g < total ? (total - 1 - st.g) / gridDim.x + 1 : 0;
@@ -90,31 +81,38 @@ __device__ __forceinline__ void clear_start(const ClearSet& z, float4* zbuf, int
 // Thread 0: issue up to `count` of the block's pieces as one bulk group.
 __device__ __forceinline__ void clear_issue(const ClearSet& z, ClearState& st, int count)
 {
-    const int64_t total = z.first[z.nf];
+    const int64_t total = clear_pieces(z);
     int issued = 0;
     for (; issued < count && st.g < total; ++issued, st.g += gridDim.x) {
-        int f = 0;
-        while (f + 1 < z.nf && st.g >= z.first[f + 1]) ++f;
-        const int64_t off = (st.g - z.first[f]) * kClearPiece;
-        const int64_t bytes16 = (z.n[f] >> 1) * 16;
-        const uint32_t bytes = (uint32_t)(bytes16 - off < kClearPiece ? bytes16 - off : kClearPiece);
-        char* dst = reinterpret_cast<char*>(z.p[f]) + off;
+        const int64_t off = st.g * kClearPiece;
+        const uint32_t bytes = (uint32_t)(z.n * 16 - off < kClearPiece ? z.n * 16 - off : kClearPiece);
         asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
-                     :: "l"(dst), "r"(st.zbuf), "r"(bytes) : "memory");
+                     :: "l"(reinterpret_cast<char*>(z.p) + off), "r"(st.zbuf), "r"(bytes) : "memory");
     }
     if (issued) asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
 // Thread 0 of every block: the rest of its pieces, then wait until all its copies are done (the
-// shared buffer must outlive them); thread 0 of block 0 also clears the odd last elements.
+// shared buffer must outlive them).
 __device__ __forceinline__ void clear_finish(const ClearSet& z, ClearState& st)
 {
     if (threadIdx.x != 0) return;
     clear_issue(z, st, 0x7fffffff);
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-    if (blockIdx.x == 0)
-        for (int f = 0; f < z.nf; ++f)
-            if (z.n[f] & 1) z.p[f][z.n[f] - 1] = 0.0;
+}
+
+// The FP64 ray step's loop: whole passes of the grid take consecutive rays block by block; the rays
+// that are left over go to the blocks in groups of 32, a warp of every block before the second of any
+// (the whole blocks of a partial last pass would leave most SMs idle, and a small population would run
+// on a few SMs: 2600 rays on 11 of 152, 41 -> 30 us).  The precision form, bound by its gathers,
+// is better off with neighbouring warps on neighbouring rays (210 K rays: 50 us, spread 54 us).  Ray of
+// this thread in pass m, n or more if none.
+__device__ __forceinline__ int loop_passes(int n) { return n / (int)(gridDim.x * blockDim.x) + 1; }
+__device__ __forceinline__ int loop_ray(int m, int passes)
+{
+    const int T = gridDim.x * blockDim.x;
+    if (m + 1 < passes) return m * T + blockIdx.x * blockDim.x + threadIdx.x;
+    return m * T + ((int)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
 }
 
 // Block sum in a fixed order (deterministic); the result is valid in thread 0.

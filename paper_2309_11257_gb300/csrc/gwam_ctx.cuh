@@ -66,6 +66,7 @@ struct Context {
     double* bg_scratch = nullptr;   // staging of caller fields ([nz][ny][nx], 4 fields)
     gwam_spec* spec_buf = nullptr;  // device copy of host spectral launches (grown, kept)
     int64_t spec_cap = 0;
+    double* launch_cols = nullptr;  // what the background source needs of each column (8 doubles a column)
 
     // ray volumes: A holds the canonical array between steps, B is the re-binned output
     bool f32 = false;               // precision form: FP32 records and background

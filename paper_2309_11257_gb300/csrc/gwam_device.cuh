@@ -163,11 +163,6 @@ __host__ __device__ __forceinline__ int64_t node_index(const Grid& G, int i, int
 
 // ---------------------------------------------------------------------------- background gather
 
-struct Bg {
-    double v[4];     // U V N2 G2
-    double d[4][3];  // coordinate derivatives of each
-};
-
 __device__ __forceinline__ int wrap_int(int i, int n)
 {
     int r = i % n;
@@ -203,20 +198,30 @@ __device__ __forceinline__ void bracket_clamped(double s, int n, int& q0, int& q
 // per-step gathers of the FP64 form run on the FP32 pipes (compensated sums), with about 48
 // significant bits.  Filled from the FP64 nodes whenever the background is set.
 struct __align__(128) NodeDF {
-    float4 q[8];   // q[e] = (hi, lo) of value 2e, then (hi, lo) of value 2e + 1
+    float4 q[8];   // q[e] = the high parts of values 2e and 2e + 1, then their low parts
 };
 
-// s + c += (wh + wl) (vh + vl): TwoProduct of the high parts, TwoSum into s, all lower-order terms
-// into the compensation c
-__device__ __forceinline__ void df_acc(float vh, float vl, float wh, float wl, float& s, float& c)
+// s + c += (wh + wl) (vh + vl) for two node values at a time: TwoProduct of the high parts, TwoSum
+// into s, all lower-order terms into the compensation c.  The product's error and the cross terms are
+// formed negated, from the negated weight that a corner's sixteen values share, and subtracted (a
+// packed instruction has no free negation): 12 packed operations for two values.
+struct CornerWeight {
+    float2 h, nh, nl;   // the weight's high part, and both parts negated, in both halves
+};
+
+__device__ __forceinline__ CornerWeight corner_weight(DF w) { return {dup2(w.hi), dup2(-w.hi), dup2(-w.lo)}; }
+
+__device__ __forceinline__ void df_acc2(float2 vh, float2 vl, const CornerWeight& w, float2& s, float2& c)
 {
-    const float p = __fmul_rn(wh, vh);
-    const float e = __fmaf_rn(wh, vh, -p);
-    const float t = __fadd_rn(s, p);
-    const float bb = __fsub_rn(t, s);
-    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(p, bb));
+    const float2 p = mul2(w.h, vh);
+    float2 g = fma2(w.nh, vh, p);
+    g = fma2(w.nl, vh, g);
+    g = fma2(w.nh, vl, g);
+    const float2 t = add2(s, p);
+    const float2 bb = sub2(t, s);
+    const float2 err = add2(sub2(s, sub2(t, bb)), sub2(p, bb));
     s = t;
-    c = __fadd_rn(c, __fadd_rn(err, __fmaf_rn(wh, vl, __fmaf_rn(wl, vh, e))));
+    c = add2(c, sub2(err, g));
 }
 
 // Trilinear interpolation of the FP64 node values (U, V, N^2, Gamma^2) to (X, Y, Z).
@@ -263,21 +268,32 @@ __device__ __forceinline__ int wrap_fast(int i, int n)
     return wrap_int(i, n);
 }
 
+// u - floor(u) of a renormalised u: hi - floor is exact for hi >= 0; for a negative hi (floor = -1 just
+// west of the first node) its rounding error comes from FastTwoSum, |floor| >= |hi|.  The difference
+// is zero or at least an ulp of hi, so the second FastTwoSum is exact too.
+__device__ __forceinline__ DF frac_df(DF u, float fl)
+{
+    const float d = __fsub_rn(u.hi, fl);
+    const float e = __fadd_rn(__fsub_rn(u.hi, __fadd_rn(d, fl)), u.lo);
+    const float t = __fadd_rn(d, e);
+    return {t, __fsub_rn(e, __fsub_rn(t, d))};
+}
+
 __device__ __forceinline__ void bracket_periodic_df(DF u, int n, int& q0, int& q1, DF& t)
 {
-    float fl = df_floor(u);
+    float fl = df_floor_sum(u);
     if (!(fabsf(fl) < 1e9f)) {
         fl = 0.0f;
         u = df_f(0.0f);
     }
-    t = df_sub(u, df_f(fl));
+    t = frac_df(u, fl);
     q0 = wrap_fast((int)fl, n);
     q1 = q0 + 1 == n ? 0 : q0 + 1;
 }
 
 __device__ __forceinline__ void bracket_clamped_df(DF u, int n, int& q0, int& q1, DF& t)
 {
-    float fl = df_floor(u);
+    float fl = df_floor_sum(u);
     if (!(fabsf(fl) < 1e9f)) {
         fl = 0.0f;
         u = df_f(0.0f);
@@ -288,19 +304,29 @@ __device__ __forceinline__ void bracket_clamped_df(DF u, int n, int& q0, int& q1
     } else if (q >= n - 1) {
         q0 = n - 2; q1 = n - 1; t = df_f(1.0f);
     } else {
-        q0 = q; q1 = q + 1; t = df_sub(u, df_f(fl));
+        q0 = q; q1 = q + 1; t = frac_df(u, fl);
     }
 }
 
-// Trilinear sums of the node quantities held in the float4 elements [E0, E1) of every NodeDF
-// (element e holds quantities 2e and 2e + 1), as unevaluated hi + compensation pairs, at the
-// double-float position (X, Y, Z).
-template <int E0, int E1>
-__device__ __forceinline__ void gather_df_sums(const Grid& G, const NodeDF* __restrict__ bg, DF X, DF Y, DF Z,
-                                               float (&s)[2 * (E1 - E0)], float (&c)[2 * (E1 - E0)])
+// The eight nodes around the double-float position (X, Y, Z): the lowest one's index and the steps to
+// the others, the four horizontal weights and the two vertical ones; jrow = the row whose centre is
+// nearest.  Corners in the order (i0 j0), (i1 j0), (i0 j1), (i1 j1), each at k0 then k1.
+struct CornersDF {
+    int base, ox, oy, oz;
+    DF w00, w10, w01, w11, Uz, Tz;
+    int jrow;
+    __device__ __forceinline__ int node(int q) const { return base + ((q & 2) ? ox : 0) + ((q & 4) ? oy : 0) + ((q & 1) ? oz : 0); }
+    __device__ __forceinline__ DF weight(int q) const
+    {
+        return df_mul2((q & 2) ? ((q & 4) ? w11 : w10) : ((q & 4) ? w01 : w00), (q & 1) ? Tz : Uz);
+    }
+};
+
+__device__ __forceinline__ CornersDF corners_df(const Grid& G, DF X, DF Y, DF Z)
 {
+    CornersDF r;
     int i0, i1, j0, j1, k0, k1;
-    DF Tx, Ty, Tz;
+    DF Tx, Ty;
     const DF half = df_f(0.5f);
     bracket_periodic_df(df_sub(df_mul2(X, DF{G.df_inv_dX.x, G.df_inv_dX.y}), half), G.nx, i0, i1, Tx);
     if (G.geometry == 1)
@@ -308,67 +334,115 @@ __device__ __forceinline__ void gather_df_sums(const Grid& G, const NodeDF* __re
                            G.ny, j0, j1, Ty);
     else
         bracket_periodic_df(df_sub(df_mul2(Y, DF{G.df_inv_dY.x, G.df_inv_dY.y}), half), G.ny, j0, j1, Ty);
-    bracket_clamped_df(df_sub(df_mul2(Z, DF{G.df_inv_dz.x, G.df_inv_dz.y}), half), G.nz, k0, k1, Tz);
+    bracket_clamped_df(df_sub(df_mul2(Z, DF{G.df_inv_dz.x, G.df_inv_dz.y}), half), G.nz, k0, k1, r.Tz);
     const DF one{1.0f, 0.0f};
-    const DF Ux = df_sub(one, Tx), Uy = df_sub(one, Ty), Uz = df_sub(one, Tz);
-    const DF w00 = df_mul2(Ux, Uy), w10 = df_mul2(Tx, Uy), w01 = df_mul2(Ux, Ty), w11 = df_mul2(Tx, Ty);
+    const DF Ux = df_add_fast(one, df_neg(Tx)), Uy = df_add_fast(one, df_neg(Ty));
+    r.Uz = df_add_fast(one, df_neg(r.Tz));
+    r.w00 = df_mul2(Ux, Uy);
+    r.w10 = df_mul2(Tx, Uy);
+    r.w01 = df_mul2(Ux, Ty);
+    r.w11 = df_mul2(Tx, Ty);
+    r.base = (j0 * G.nx + i0) * G.nz + k0;
+    r.ox = (i1 - i0) * G.nz;
+    r.oy = (j1 - j0) * G.nx * G.nz;
+    r.oz = k1 - k0;
+    r.jrow = Ty.hi < 0.5f ? j0 : j1;
+    return r;
+}
+
+// All 16 quantities at the positions of a warp's 32 rays, by eight lanes a node: lane l loads the
+// (l & 7)-th 16 bytes of the nodes of rays 4 j + (l >> 3), j = 0 .. 7, so every load covers whole
+// 128-byte nodes, and accumulates that element's two quantities for these eight rays.  With a ray a
+// lane, each of a node's eight 16-byte loads touched 32 lines where the rays of a warp sit at different
+// levels, and the kernel was bound by them (256 x 128 x 90 sphere, waves aloft: 64 loads a stage x 32
+// wavefronts = 0.5 ms of L1 per step).  The weights and node indices pass to the eight lanes through
+// the ray's row of shared memory, the sums come back in the same row (kGatherRow floats: 128 bytes and
+// a pad against bank conflicts).  All 32 lanes must call it; the row is free again after the call.
+constexpr int kGatherRow = 36;
+
+__device__ __forceinline__ void gather_warp_df(const Grid& G, const NodeDF* __restrict__ bg, int first, DF X, DF Y, DF Z,
+                                               float* rows, BgDF& b, int& jrow)
+{
+    const int lane = threadIdx.x & 31;
+    {
+        const CornersDF cn = corners_df(G, X, Y, Z);
+        jrow = cn.jrow;
+        float* row = rows + lane * kGatherRow;
 #pragma unroll
-    for (int q = 0; q < 2 * (E1 - E0); ++q) s[q] = c[q] = 0.0f;
-    const int dk = k1 - k0;
-    // corners in the order (i0 j0), (i1 j0), (i0 j1), (i1 j1), each at k0 then k1.  The loop is rolled,
-    // the corner's node and weight selected, not indexed: one copy of the eight loads and sixteen
-    // accumulations instead of eight keeps the ray-step kernels small (measured faster on GB300 than
-    // unrolling by 2 or 8: the kernels were stalling on instruction fetch)
+        for (int q = 0; q < 8; q += 2) {
+            const DF w0 = cn.weight(q), w1 = cn.weight(q + 1);
+            *reinterpret_cast<float4*>(row + 2 * q) = make_float4(w0.hi, w0.lo, w1.hi, w1.lo);
+        }
+        *reinterpret_cast<int4*>(row + 16) = make_int4(first + cn.base, cn.ox, cn.oy, cn.oz);
+    }
+    __syncwarp();
+    const float4* __restrict__ el = reinterpret_cast<const float4*>(bg) + (lane & 7);
+    float* row = rows + (lane >> 3) * kGatherRow;
+    float4 nxt[8];
+    auto fetch = [&](const float* r) {
+        const int4 o = *reinterpret_cast<const int4*>(r + 16);
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            nxt[q] = __ldg(el + 8 * (int64_t)(o.x + ((q & 2) ? o.y : 0) + ((q & 4) ? o.z : 0) + ((q & 1) ? o.w : 0)));
+    };
+    fetch(row);
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+        float4 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = nxt[q];
+        if (j < 7) fetch(row + 4 * kGatherRow);   // the next rays' nodes, while these are summed
+        float2 s = dup2(0.0f), c = dup2(0.0f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float2 w = *reinterpret_cast<const float2*>(row + 2 * q);
+            df_acc2(make_float2(v[q].x, v[q].y), make_float2(v[q].z, v[q].w), corner_weight(DF{w.x, w.y}), s, c);
+        }
+        const DF a0 = df_norm(s.x, c.x), a1 = df_norm(s.y, c.y);
+        __syncwarp();   // the four rays' weights have been read by their eight lanes
+        *reinterpret_cast<float4*>(row + 4 * (lane & 7)) = make_float4(a0.hi, a1.hi, a0.lo, a1.lo);
+        row += 4 * kGatherRow;
+    }
+    __syncwarp();
+    float4 e[8];
+    const float* own = rows + lane * kGatherRow;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) e[q] = *reinterpret_cast<const float4*>(own + 4 * q);
+    auto val = [&](int q) { return (q & 1) ? DF{e[q >> 1].y, e[q >> 1].w} : DF{e[q >> 1].x, e[q >> 1].z}; };
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        b.v[f] = val(f);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) b.d[f][q] = val(4 + 3 * f + q);
+    }
+    __syncwarp();
+}
+
+// N^2 and Gamma^2 (the second 16 bytes of each node) alone, as unevaluated hi + compensation pairs: what
+// the intrinsic quantities need.  The loop over the corners is rolled, the corner's node and weight
+// selected, not indexed (measured faster on GB300 than unrolling by 2 or 8: the kernels were stalling
+// on instruction fetch).
+__device__ __forceinline__ void gather_n2g2_sums(const Grid& G, const NodeDF* __restrict__ bg, DF X, DF Y, DF Z,
+                                                 float2& s, float2& c, int& jrow)
+{
+    const CornersDF cn = corners_df(G, X, Y, Z);
+    jrow = cn.jrow;
+    s = c = dup2(0.0f);
 #pragma unroll 1
     for (int q = 0; q < 8; ++q) {
-        const int cx = (q >> 1) & 1, cy = q >> 2;
-        const NodeDF* p = bg + node_index(G, cx ? i1 : i0, cy ? j1 : j0, k0) + ((q & 1) ? dk : 0);
-        const DF wxy = cx ? (cy ? w11 : w10) : (cy ? w01 : w00);
-        const DF w = df_mul2(wxy, (q & 1) ? Tz : Uz);
-#pragma unroll
-        for (int e = E0; e < E1; ++e) {
-            const float4 a = __ldg(p->q + e);
-            df_acc(a.x, a.y, w.hi, w.lo, s[2 * (e - E0)], c[2 * (e - E0)]);
-            df_acc(a.z, a.w, w.hi, w.lo, s[2 * (e - E0) + 1], c[2 * (e - E0) + 1]);
-        }
-    }
-}
-
-// gather with double-float results (no conversion back to FP64)
-__device__ __forceinline__ void gather_df(const Grid& G, const NodeDF* __restrict__ bg, DF X, DF Y, DF Z, BgDF& b)
-{
-    float s[16], c[16];
-    gather_df_sums<0, 8>(G, bg, X, Y, Z, s, c);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        b.v[f] = df_norm(s[f], c[f]);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) b.d[f][q] = df_norm(s[4 + 3 * f + q], c[4 + 3 * f + q]);
-    }
-}
-
-// gather with FP64 results from the double-float nodes (saturation and cap paths of the FP64 form)
-__device__ __forceinline__ void gather(const Grid& G, const NodeDF* __restrict__ bg, double X, double Y, double Z,
-                                       Bg& b)
-{
-    float s[16], c[16];
-    gather_df_sums<0, 8>(G, bg, df_split(X), df_split(Y), df_split(Z), s, c);
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-        b.v[f] = widen(s[f]) + widen(c[f]);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) b.d[f][q] = widen(s[4 + 3 * f + q]) + widen(c[4 + 3 * f + q]);
+        const float4 a = __ldg(bg[cn.node(q)].q + 1);
+        df_acc2(make_float2(a.x, a.y), make_float2(a.z, a.w), corner_weight(cn.weight(q)), s, c);
     }
 }
 
 // N^2 and Gamma^2 alone (the second float4 of each node): what the intrinsic quantities need
 __device__ __forceinline__ void gather_n2g2_df(const Grid& G, const NodeDF* __restrict__ bg, DF X, DF Y, DF Z,
-                                               DF& n2, DF& g2)
+                                               DF& n2, DF& g2, int& jrow)
 {
-    float s[2], c[2];
-    gather_df_sums<1, 2>(G, bg, X, Y, Z, s, c);
-    n2 = df_norm(s[0], c[0]);
-    g2 = df_norm(s[1], c[1]);
+    float2 s, c;
+    gather_n2g2_sums(G, bg, X, Y, Z, s, c, jrow);
+    n2 = df_norm(s.x, c.x);
+    g2 = df_norm(s.y, c.y);
 }
 
 // f^2 and d(f^2)/dphi (f = 2 Omega sin phi on the sphere, f0 on the f-plane)
@@ -440,14 +514,17 @@ struct DispDF {
     DF K2, iK2, D, w2, iw, c;
 };
 
+// w^2 as f^2 + D k_h^2 / K^2 (the same quantity as (f^2 (m^2 + G^2) + N^2 k_h^2) / K^2, one product fewer,
+// and D / K^2 serves c too)
 __device__ __forceinline__ void dispersion_df(DF kh2, DF mg2, DF n2, DF f2, DispDF& d)
 {
-    d.K2 = df_add(kh2, mg2);
+    d.K2 = df_add_same(kh2, mg2);
     d.D = df_sub(n2, f2);
     d.iK2 = df_rcp(d.K2);
-    d.w2 = df_mul2(df_add(df_mul2(f2, mg2), df_mul2(n2, kh2)), d.iK2);
+    const DF t = df_mul2(d.D, d.iK2);
+    d.w2 = df_add(f2, df_mul2(t, kh2));
     d.iw = df_rsqrt(d.w2);
-    d.c = df_mul2(df_mul2(d.D, df_mul2(d.iK2, d.iK2)), d.iw);
+    d.c = df_mul2(df_mul2(t, d.iK2), d.iw);
 }
 
 struct GeoDF {
@@ -458,11 +535,8 @@ struct GeoDF {
 // (|d| <= half a row): sin(p0 + d) = s0 cos d + c0 sin d, cos(p0 + d) = c0 cos d - s0 sin d, with
 // sin d and cos d from their Taylor series -- the terms up to d^3 and d^4 in DF, the smaller ones
 // (below 3e-8 for rows of up to 9 degrees) in FP32, truncated after d^7 and d^8
-__device__ __forceinline__ void lat_sincos_df(const Grid& G, DF Y, DF& sphi, DF& cphi)
+__device__ __forceinline__ void lat_sincos_row_df(const Grid& G, int j, DF Y, DF& sphi, DF& cphi)
 {
-    // the row only selects the expansion point: a neighbouring row near a boundary is as good
-    const float fj = df_floor(df_mul2(df_sub(Y, DF{G.df_y0.x, G.df_y0.y}), DF{G.df_inv_dY.x, G.df_inv_dY.y}));
-    const int j = fj < 0.0f ? 0 : (fj >= (float)(G.ny - 1) ? G.ny - 1 : (int)fj);
     const float2 rl = G.row_lat_df[j];
     const DF d = df_sub(Y, DF{rl.x, rl.y});
     const DF dd = df_mul2(d, d);
@@ -480,10 +554,19 @@ __device__ __forceinline__ void lat_sincos_df(const Grid& G, DF Y, DF& sphi, DF&
     cphi = df_sub(df_mul2(c0, cosd), df_mul2(s0, sind));
 }
 
-__device__ __forceinline__ void geometry_df(const Grid& G, DF Y, DF Z, GeoDF& g)
+// the same with the row found from Y: it only selects the expansion point, so a neighbouring row near
+// a boundary is as good
+__device__ __forceinline__ void lat_sincos_df(const Grid& G, DF Y, DF& sphi, DF& cphi)
+{
+    const float fj = df_floor(df_mul2(df_sub(Y, DF{G.df_y0.x, G.df_y0.y}), DF{G.df_inv_dY.x, G.df_inv_dY.y}));
+    const int j = fj < 0.0f ? 0 : (fj >= (float)(G.ny - 1) ? G.ny - 1 : (int)fj);
+    lat_sincos_row_df(G, j, Y, sphi, cphi);
+}
+
+__device__ __forceinline__ void geometry_df(const Grid& G, int j, DF Y, DF Z, GeoDF& g)
 {
     if (G.geometry == 1) {
-        lat_sincos_df(G, Y, g.sphi, g.cphi);
+        lat_sincos_row_df(G, j, Y, g.sphi, g.cphi);
         const DF r = df_add(DF{G.df_radius.x, G.df_radius.y}, Z);
         g.ir = df_rcp(r);
         const DF ic = df_rcp(g.cphi);
@@ -498,15 +581,62 @@ __device__ __forceinline__ void geometry_df(const Grid& G, DF Y, DF Z, GeoDF& g)
     }
 }
 
-// ext_sh: when given, the three extents are read from there (float2 pairs kThreads apart) instead of
-// y[6..8], which the caller then need not hold in registers
-__device__ __forceinline__ void ray_rhs_df(const Grid& G, const NodeDF* __restrict__ bg, const DF y[9], DF R[9],
-                                           const float2* ext_sh = nullptr)
+// Where rk3 and ray_rhs_df keep a thread's nine components between the passes: shared memory, two
+// components (their high parts, then their low parts) in a float4, a warp's pairs 32 lanes apart.  The
+// state y, the low-storage register q, the increment sums acc and the rates r wait there instead of in
+// the registers that the ray equations need; r shares its place with the gather's rows, which are
+// free once the background is in registers.
+constexpr int kRkPairs = 5;                                       // nine components and a spare half
+constexpr int kRkWarp = 3 * kRkPairs * 32 + 32 * kGatherRow / 4;  // float4s a warp: y, q, acc, rows (or r)
+constexpr size_t kRkSmem = kRkWarp * (kThreads / 32) * sizeof(float4);
+static_assert(kRkPairs * 32 <= 32 * kGatherRow / 4, "the rates fit the gather's rows");
+
+struct RkSlots {
+    float4 *y, *q, *acc, *r;   // this thread's
+    float* rows;               // its warp's
+    __device__ __forceinline__ explicit RkSlots(void* smem)
+    {
+        float4* w = static_cast<float4*>(smem) + (threadIdx.x >> 5) * kRkWarp;
+        y = w + (threadIdx.x & 31);
+        q = y + kRkPairs * 32;
+        acc = q + kRkPairs * 32;
+        r = acc + kRkPairs * 32;
+        rows = reinterpret_cast<float*>(w + 3 * kRkPairs * 32);
+    }
+};
+
+__device__ __forceinline__ DF rk_get(const float4* p, int c)
 {
+    const float* f = reinterpret_cast<const float*>(p + (c >> 1) * 32) + (c & 1);
+    return {f[0], f[2]};
+}
+__device__ __forceinline__ void rk_put(float4* p, int c, DF v)
+{
+    float* f = reinterpret_cast<float*>(p + (c >> 1) * 32) + (c & 1);
+    f[0] = v.hi;
+    f[2] = v.lo;
+}
+__device__ __forceinline__ DFP rk_get2(const float4* p, int pair)
+{
+    const float4 v = p[pair * 32];
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ void rk_put2(float4* p, int pair, DFP v)
+{
+    p[pair * 32] = make_float4(v.hi.x, v.hi.y, v.lo.x, v.lo.y);
+}
+
+// the nine rates (into sl.r) at the state sl.y; first = the first node of the ray's ensemble member.  All
+// 32 lanes of a warp must call it.
+__device__ __forceinline__ void ray_rhs_df(const Grid& G, const NodeDF* __restrict__ bg, int first, const RkSlots& sl)
+{
+    const DFP y01 = rk_get2(sl.y, 0);
+    const DF X = dfp_x(y01), Y = dfp_y(y01), Z = rk_get(sl.y, 2);
     BgDF b;
-    gather_df(G, bg, y[0], y[1], y[2], b);
+    int jrow;
+    gather_warp_df(G, bg, first, X, Y, Z, sl.rows, b, jrow);
     GeoDF g;
-    geometry_df(G, y[1], y[2], g);
+    geometry_df(G, jrow, Y, Z, g);
     DF f2, df2;
     if (G.geometry == 1) {
         const DF f = df_mul2(DF{G.df_2omega.x, G.df_2omega.y}, g.sphi);
@@ -516,10 +646,11 @@ __device__ __forceinline__ void ray_rhs_df(const Grid& G, const NodeDF* __restri
         f2 = DF{G.df_f0sq.x, G.df_f0sq.y};
         df2 = df_f(0.0f);
     }
-    const DF k = y[3], l = y[4], m = y[5];
+    const DFP y45 = rk_get2(sl.y, 2);
+    const DF k = rk_get(sl.y, 3), l = dfp_x(y45), m = dfp_y(y45);
     const DF U = b.v[0], V = b.v[1], N2 = b.v[2], G2 = b.v[3];
-    const DF kh2 = df_add(df_mul2(k, k), df_mul2(l, l)), m2 = df_mul2(m, m);
-    const DF mg2 = df_add(m2, G2);
+    const DF kh2 = df_add_same(df_mul2(k, k), df_mul2(l, l));
+    const DF mg2 = df_add_same(df_mul2(m, m), G2);
     DispDF d;
     dispersion_df(kh2, mg2, N2, f2, d);
     const DF mg2c = df_mul2(mg2, d.c);
@@ -538,79 +669,67 @@ __device__ __forceinline__ void ray_rhs_df(const Grid& G, const NodeDF* __restri
     Gq[1] = df_add(Gq[1], df_mul2(aF, df2));
     if (G.columnar) {
         // single-column mode: k and l fixed, m by the vertical gradient of Omega alone
-        R[3] = df_f(0.0f);
-        R[4] = df_f(0.0f);
-        R[5] = df_neg(Gq[2]);
+        rk_put(sl.r, 3, df_f(0.0f));
+        rk_put(sl.r, 4, df_f(0.0f));
+        rk_put(sl.r, 5, df_neg(Gq[2]));
     } else if (G.geometry == 1) {
         const DF ir = g.ir;
-        R[3] = df_add(df_neg(df_mul2(Gq[0], g.ihX)), df_mul2(df_mul2(k, ir), df_sub(df_mul2(g.tphi, cgy), cgz)));
-        R[4] = df_sub(df_neg(df_mul2(Gq[1], ir)), df_mul2(ir, df_add(df_mul2(l, cgz), df_mul2(df_mul2(k, g.tphi), cgx))));
-        R[5] = df_add(df_neg(Gq[2]), df_mul2(ir, df_add(df_mul2(k, cgx), df_mul2(l, cgy))));
+        rk_put(sl.r, 3, df_add(df_neg(df_mul2(Gq[0], g.ihX)), df_mul2(df_mul2(k, ir), df_sub(df_mul2(g.tphi, cgy), cgz))));
+        rk_put(sl.r, 4, df_sub(df_neg(df_mul2(Gq[1], ir)),
+                               df_mul2(ir, df_add(df_mul2(l, cgz), df_mul2(df_mul2(k, g.tphi), cgx)))));
+        rk_put(sl.r, 5, df_add(df_neg(Gq[2]), df_mul2(ir, df_add(df_mul2(k, cgx), df_mul2(l, cgy)))));
     } else {
-        R[3] = df_neg(Gq[0]);
-        R[4] = df_neg(Gq[1]);
-        R[5] = df_neg(Gq[2]);
+        rk_put(sl.r, 3, df_neg(Gq[0]));
+        rk_put(sl.r, 4, df_neg(Gq[1]));
+        rk_put(sl.r, 5, df_neg(Gq[2]));
     }
-    // faces: first-order Taylor values along the face's own axis.  The six face evaluations run as
-    // one rolled loop (axis q, side sd) with the per-axis operands selected, not indexed: one copy of
-    // the dispersion relation in the code instead of six keeps the kernel body small.
+    // faces: first-order Taylor values along the face's own axis, the two faces of an axis in the halves
+    // of packed pairs.  Relative to the centre a face changes m^2 + G^2 and K^2 by +-tg and D by
+    // +-(tn - tf), so its dispersion terms start from the centre's sums; with b = (m^2 + G^2) c the mean and
+    // the difference of the two face velocities are (A (b+ + b-) / 2 + W) S and (A (b+ - b-) + 2 tw) S
+    // (horizontal), -m k_h^2 times those of c (vertical).  108 operations a face instead of 197 for a
+    // face evaluated from its own values.  The axes run as a rolled loop, the per-axis operands selected,
+    // not indexed: unrolled, the kernel outgrew the instruction cache (a third of its stall cycles
+    // were instruction fetch).
     int q0 = 0;
     if (G.columnar) {
         // no horizontal propagation or advection
-        R[0] = R[1] = R[6] = R[7] = df_f(0.0f);
+        rk_put(sl.r, 0, df_f(0.0f));
+        rk_put(sl.r, 1, df_f(0.0f));
+        rk_put(sl.r, 6, df_f(0.0f));
+        rk_put(sl.r, 7, df_f(0.0f));
         q0 = 2;
     }
-    const DF zero = df_f(0.0f);
-    const DF mkh2 = df_mul2(m, kh2);
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        if (q < q0) continue;
-        DF ext;
-        if (ext_sh) {
-            const float2 e2 = ext_sh[q * kThreads];
-            ext = DF{e2.x, e2.y};
-        } else {
-            ext = q == 0 ? y[6] : (q == 1 ? y[7] : y[8]);
-        }
+    const DF mkh2 = df_neg(df_mul2(m, kh2));
+#pragma unroll 1
+    for (int q = q0; q < 3; ++q) {
+        const DF ext = rk_get(sl.y, 6 + q);
         const DF dn = q == 0 ? b.d[2][0] : (q == 1 ? b.d[2][1] : b.d[2][2]);
         const DF dg = q == 0 ? b.d[3][0] : (q == 1 ? b.d[3][1] : b.d[3][2]);
-        const DF dfq = q == 1 ? df2 : zero;     // f^2 varies along the meridional axis only
-        const DF A = q == 0 ? k : l;
-        const DF W = q == 0 ? U : V;
-        const DF dW = q == 0 ? b.d[0][0] : b.d[1][1];
-        const DF S = q == 0 ? g.ihX : g.ir;
-        // the Taylor increments at the +h face, h = ext / 2; the -h face takes their negations (a
-        // product by -h is the negated product by h, bit for bit)
         const DF h = df_pow2(ext, 0.5f);
-        const DF tn = df_mul2(dn, h), tg = df_mul2(dg, h), tw = df_mul2(dW, h);
-        const DF tf = q == 1 ? df_mul2(dfq, h) : zero;
-        DF vel0 = zero, vel1 = zero;
-#pragma unroll 1
-        for (int sd = 0; sd < 2; ++sd) {
-            const DF N2f = df_add(N2, sd == 0 ? tn : df_neg(tn));
-            const DF G2f = df_add(G2, sd == 0 ? tg : df_neg(tg));
-            const DF f2f = q == 1 ? df_add(f2, sd == 0 ? tf : df_neg(tf)) : f2;
-            const DF mg2f = df_add(m2, G2f);
-            DispDF e;
-            dispersion_df(kh2, mg2f, N2f, f2f, e);
-            const DF v = q < 2 ? df_mul2(df_add(df_add(df_mul2(df_mul2(A, mg2f), e.c), W), sd == 0 ? tw : df_neg(tw)), S)
-                               : df_neg(df_mul2(mkh2, e.c));
-            if (sd == 0)
-                vel0 = v;
-            else
-                vel1 = v;
+        const DF tg = df_mul2(dg, h);
+        DF td = df_mul2(dn, h);
+        DFP f2f = dfp_dup(f2);
+        if (q == 1) {   // f^2 varies along the meridional axis only
+            const DF tf = df_mul2(df2, h);
+            td = df_sub(td, tf);
+            f2f = dfp_add(f2f, dfp_pm(tf));
         }
-        const DF rc = df_pow2(df_add(vel0, vel1), 0.5f), re = df_sub(vel0, vel1);
-        if (q == 0) {
-            R[0] = rc;
-            R[6] = re;
-        } else if (q == 1) {
-            R[1] = rc;
-            R[7] = re;
-        } else {
-            R[2] = rc;
-            R[8] = re;
+        const DFP iK2 = dfp_rcp(dfp_add(dfp_dup(d.K2), dfp_pm(tg)));
+        const DFP t = dfp_mul(dfp_add(dfp_dup(d.D), dfp_pm(td)), iK2);
+        const DFP iw = dfp_rsqrt(dfp_add(f2f, dfp_mul(t, dfp_dup(kh2))));
+        DFP c = dfp_mul(dfp_mul(t, iK2), iw);
+        if (q < 2) c = dfp_mul(dfp_add(dfp_dup(mg2), dfp_pm(tg)), c);
+        const DF A = q == 0 ? k : (q == 1 ? l : mkh2);
+        DF mean = df_mul2(A, df_pow2(df_add(dfp_x(c), dfp_y(c)), 0.5f));
+        DF diff = df_mul2(A, df_sub(dfp_x(c), dfp_y(c)));
+        if (q < 2) {
+            const DF W = q == 0 ? U : V, S = q == 0 ? g.ihX : g.ir, dW = q == 0 ? b.d[0][0] : b.d[1][1];
+            mean = df_mul2(df_add(mean, W), S);
+            diff = df_mul2(df_add(diff, df_mul2(dW, ext)), S);   // dW ext = 2 tw
         }
+        rk_put(sl.r, q, mean);
+        rk_put(sl.r, 6 + q, diff);
     }
 }
 
@@ -626,11 +745,12 @@ __device__ __forceinline__ void intrinsic_df(const Grid& G, const NodeDF* __rest
                                              IntrDF& in)
 {
     DF g2;
+    int jrow;
     const DF Y = df_split(s[SY]);
-    gather_n2g2_df(G, bg, df_split(s[SX]), Y, df_split(s[SZ]), in.n2, g2);
+    gather_n2g2_df(G, bg, df_split(s[SX]), Y, df_split(s[SZ]), in.n2, g2, jrow);
     if (G.geometry == 1) {
         DF sphi, cphi;
-        lat_sincos_df(G, Y, sphi, cphi);
+        lat_sincos_row_df(G, jrow, Y, sphi, cphi);
         in.f = df_mul2(DF{G.df_2omega.x, G.df_2omega.y}, sphi);
         in.f2 = df_mul2(in.f, in.f);
     } else {
@@ -640,24 +760,28 @@ __device__ __forceinline__ void intrinsic_df(const Grid& G, const NodeDF* __rest
     in.k = df_split(s[SK]);
     in.l = df_split(s[SL]);
     in.m = df_split(s[SM]);
-    in.kh2 = df_add(df_mul2(in.k, in.k), df_mul2(in.l, in.l));
+    in.kh2 = df_add_same(df_mul2(in.k, in.k), df_mul2(in.l, in.l));
     in.m2 = df_mul2(in.m, in.m);
-    in.mg2 = df_add(in.m2, g2);
+    in.mg2 = df_add_same(in.m2, g2);
     dispersion_df(in.kh2, in.mg2, in.n2, in.f2, in.d);
 }
 
 // Williamson (1980) low-storage RK3 on the 9 propagated components; background frozen.  The rates
 // and the low-storage register q are double-float; the step's increments B q of the three stages
-// are summed in double-float and added to the FP64 state once, at the end (one FP64 rounding per
-// component instead of three: the sum is far smaller than the state, so its 48 bits are ample), and
-// a double-float copy of the state, updated by the same B q, feeds the next evaluation.  The FP64
-// state and the increment sums wait in shared memory during the stages (sh: this thread's first
-// slot, slots kThreads apart: 9 doubles, then 9 float2 sums at sh + 9 kThreads), which keeps them
-// out of the registers the ray equations need; with kQShared the low-storage register q waits there
-// too (9 float2 at sh + 18 kThreads; 27 kThreads doubles in all).
-template <bool kQShared = false, bool kExtShared = false>
-__device__ __forceinline__ void rk3(const Grid& G, const NodeDF* __restrict__ bg, double s[NSTATE], double dt,
-                                    double* sh)
+// are summed in double-float (sl.acc) and added to the FP64 state once, by the caller (rk_increment: one
+// FP64 rounding per component instead of three: the sum is far smaller than the state, so its 48 bits
+// are ample), and a double-float copy of the state, updated by the same B q, feeds the next
+// evaluation.  The update takes two components at a time in packed pairs, as a rolled loop (a small
+// kernel body: see ray_rhs_df).
+__device__ __forceinline__ void rk3_start(const RkSlots& sl, const double (&s)[9])
+{
+#pragma unroll
+    for (int c = 0; c < 9; ++c) rk_put(sl.y, c, df_split(s[c]));
+    rk_put(sl.y, 9, df_f(0.0f));
+}
+
+// first: the first node of the ray's ensemble member; all 32 lanes of a warp must call it
+__device__ __forceinline__ void rk3(const Grid& G, const NodeDF* __restrict__ bg, int first, double dt, const RkSlots& sl)
 {
     constexpr DF A1{-5.0f / 9.0f, (float)(-5.0 / 9.0 - (double)(-5.0f / 9.0f))};
     constexpr DF A2{-153.0f / 128.0f, 0.0f};
@@ -665,54 +789,30 @@ __device__ __forceinline__ void rk3(const Grid& G, const NodeDF* __restrict__ bg
     constexpr DF B1{15.0f / 16.0f, 0.0f};
     constexpr DF B2{8.0f / 15.0f, (float)(8.0 / 15.0 - (double)(8.0f / 15.0f))};
     const DF dtd = df_split(dt);
-    DF y[9], q[kQShared ? 1 : 9];
-    float2* acc = reinterpret_cast<float2*>(sh + 9 * kThreads);
-    float2* qs = acc + 9 * kThreads;
-    float2* es = qs + 9 * kThreads;   // the extents' double-float copy (kExtShared)
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-        y[c] = df_split(s[c]);
-        if (!kQShared) q[c] = df_f(0.0f);
-        sh[c * kThreads] = s[c];
-        acc[c * kThreads] = make_float2(0.0f, 0.0f);
-        if (kExtShared && c >= 6) es[(c - 6) * kThreads] = make_float2(y[c].hi, y[c].lo);
-    }
 #pragma unroll 1
     for (int st = 0; st < 3; ++st) {
-        DF F[9];
-        ray_rhs_df(G, bg, y, F, kExtShared ? es : nullptr);
-        const DF a = st == 1 ? A1 : A2;
-        const DF b = st == 0 ? B0 : (st == 1 ? B1 : B2);
-#pragma unroll
-        for (int c = 0; c < 9; ++c) {
-            DF qc;
-            if (kQShared) {
-                const float2 qo = qs[c * kThreads];
-                qc = st == 0 ? df_mul2(dtd, F[c]) : df_add(df_mul2(a, DF{qo.x, qo.y}), df_mul2(dtd, F[c]));
-                qs[c * kThreads] = make_float2(qc.hi, qc.lo);
-            } else {
-                qc = st == 0 ? df_mul2(dtd, F[c]) : df_add(df_mul2(a, q[c]), df_mul2(dtd, F[c]));
-                q[c] = qc;
+        ray_rhs_df(G, bg, first, sl);
+        rk_put(sl.r, 9, df_f(0.0f));
+        const DFP a = dfp_dup(st == 1 ? A1 : A2);
+        const DFP b = dfp_dup(st == 0 ? B0 : (st == 1 ? B1 : B2));
+        const DFP h = dfp_dup(dtd);
+#pragma unroll 1
+        for (int p = 0; p < kRkPairs; ++p) {
+            DFP q = dfp_mul(h, rk_get2(sl.r, p));
+            if (st > 0) q = dfp_add(dfp_mul(a, rk_get2(sl.q, p)), q);
+            const DFP bq = dfp_mul(b, q);
+            if (st < 2) {   // the last stage's state is not evaluated
+                rk_put2(sl.q, p, q);
+                rk_put2(sl.y, p, dfp_add(rk_get2(sl.y, p), bq));
             }
-            const DF bq = df_mul2(b, qc);
-            const float2 o = acc[c * kThreads];
-            const DF na = df_add(DF{o.x, o.y}, bq);
-            acc[c * kThreads] = make_float2(na.hi, na.lo);
-            if (kExtShared && c >= 6) {
-                const float2 ye = es[(c - 6) * kThreads];
-                const DF yn = df_add(DF{ye.x, ye.y}, bq);
-                es[(c - 6) * kThreads] = make_float2(yn.hi, yn.lo);
-            } else {
-                y[c] = df_add(y[c], bq);
-            }
+            rk_put2(sl.acc, p, st > 0 ? dfp_add(rk_get2(sl.acc, p), bq) : bq);
         }
-    }
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-        const float2 o = acc[c * kThreads];
-        s[c] = sh[c * kThreads] + df_to_double(DF{o.x, o.y});
+        __syncwarp();   // the rates have been read: their place is the next stage's gather rows
     }
 }
+
+// the step's increment of component c
+__device__ __forceinline__ double rk_increment(const RkSlots& sl, int c) { return df_to_double(rk_get(sl.acc, c)); }
 
 // ---------------------------------------------------------------------------- bookkeeping
 
@@ -833,17 +933,19 @@ struct Intr {
 __device__ __forceinline__ void intrinsic_at(const Grid& G, const NodeDF* __restrict__ bg, const double s[NSTATE],
                                              Geo& g, Intr& in)
 {
-    Bg b;
-    gather(G, bg, s[SX], s[SY], s[SZ], b);
+    float2 sum, cmp;
+    int jrow;
+    gather_n2g2_sums(G, bg, df_split(s[SX]), df_split(s[SY]), df_split(s[SZ]), sum, cmp, jrow);
+    const double n2 = widen(sum.x) + widen(cmp.x), g2 = widen(sum.y) + widen(cmp.y);
     geometry_at(G, s[SY], s[SZ], g);
     double df2;
     coriolis(G, g.sphi, g.cphi, in.f2, df2);
     in.kh2 = s[SK] * s[SK] + s[SL] * s[SL];
     in.m2 = s[SM] * s[SM];
-    in.n2 = b.v[2];
-    in.mg2 = in.m2 + b.v[3];
+    in.n2 = n2;
+    in.mg2 = in.m2 + g2;
     Disp d;
-    dispersion(in.kh2, in.mg2, b.v[2], in.f2, d);
+    dispersion(in.kh2, in.mg2, n2, in.f2, d);
     in.K2 = d.K2;
     in.iK2 = d.iK2;
     in.D = d.D;

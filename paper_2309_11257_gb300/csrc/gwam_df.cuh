@@ -177,30 +177,159 @@ __device__ __forceinline__ DF df_norm(float s, float c)
     return {h, __fadd_rn(__fsub_rn(s, __fsub_rn(h, bb)), __fsub_rn(c, bb))};
 }
 
-// 1 / x: the FP32 hardware approximation (about 23 correct bits) refined by one Newton step
-// y <- y + y (1 - x y) in DF, which squares the relative error to about 2^-45
+// a + b for |a| >= |b| (or a = 0): FastTwoSum in place of df_add's TwoSum, 8 operations instead of 11
+__device__ __forceinline__ DF df_add_fast(DF a, DF b)
+{
+    const float s = __fadd_rn(a.hi, b.hi);
+    const float e = __fadd_rn(__fsub_rn(b.hi, __fsub_rn(s, a.hi)), __fadd_rn(a.lo, b.lo));
+    const float h = __fadd_rn(s, e);
+    return {h, __fsub_rn(e, __fsub_rn(h, s))};
+}
+
+// a + b of two values of the same sign: no cancellation, so the pair needs no renormalisation (as a
+// product's, |lo| at most a few ulp(hi)); 8 operations instead of 11
+__device__ __forceinline__ DF df_add_same(DF a, DF b)
+{
+    const float s = __fadd_rn(a.hi, b.hi);
+    const float bb = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
+    return {s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
+}
+
+// 1 / x: the FP32 hardware approximation r0 (about 23 correct bits) and its remainder.  e = 1 - x r0
+// comes from two FMAs: x.hi r0 lies within 2^-21 of 1 and has at most 48 bits, so 1 - x.hi r0 needs
+// about 25 of them and the FMA's single rounding leaves it to 2^-47.  1 / x = r0 (1 + e + e^2 + ...) =
+// r0 + r0 (e + e^2), renormalised by FastTwoSum (e reaches 2^-22: as an unevaluated pair its low part
+// is four ulps, and products of two such pairs, which drop lo x lo, lose 2^-44).  Relative error about
+// 2^-46 in 7 FP32 operations; a Newton step in double-float (1 - x r0 as a df_mul and a df_sub, the
+// update as a df_mul and a df_add) had taken 36 for 2^-45.
 __device__ __forceinline__ DF df_rcp(DF x)
 {
     float r0;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x.hi));
-    const DF e = df_sub(df_f(1.0f), df_mul(x, r0));
-    return df_add(df_f(r0), df_mul(e, r0));
+    float e = __fmaf_rn(-x.hi, r0, 1.0f);
+    e = __fmaf_rn(-x.lo, r0, e);
+    const float d = __fmul_rn(r0, __fmaf_rn(e, e, e)), h = __fadd_rn(r0, d);
+    return {h, __fsub_rn(d, __fsub_rn(h, r0))};
 }
 
-// 1 / sqrt(x): the FP32 hardware approximation refined by one Newton step
-// y <- y + y (1 - x y^2) / 2 in DF (relative error about 2^-45, as df_rcp)
+// 1 / sqrt(x): likewise from the FP32 approximation r0: e = 1 - x r0^2 (r0^2 as an exact product
+// pair), 1 / sqrt(x) = r0 (1 - e)^(-1/2) = r0 (1 + e/2 + 3 e^2 / 8 + ...).  Relative error about 2^-46 in 11
+// FP32 operations (37 as a Newton step in double-float, 2^-45).
 __device__ __forceinline__ DF df_rsqrt(DF x)
 {
     float r0;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x.hi));
-    const DF e = df_sub(df_f(1.0f), df_mul2(x, df_prod(r0, r0)));
-    return df_add(df_f(r0), df_pow2(df_mul(e, r0), 0.5f));
+    const float p = __fmul_rn(r0, r0), pe = __fmaf_rn(r0, r0, -p);
+    float e = __fmaf_rn(-x.hi, p, 1.0f);
+    e = __fmaf_rn(-x.hi, pe, e);
+    e = __fmaf_rn(-x.lo, p, e);
+    const float d = __fmul_rn(__fmul_rn(r0, e), __fmaf_rn(0.375f, e, 0.5f)), h = __fadd_rn(r0, d);
+    return {h, __fsub_rn(d, __fsub_rn(h, r0))};
+}
+
+// Two double-float values in the two halves of packed FP32 pairs.  GB300's packed FP32 instructions
+// (add, mul, fma on two floats) run at the same 128 lanes a clock and SM as the scalar ones but take
+// half the issue slots and bring two independent chains into each warp; every lane rounds as the
+// scalar instruction does.  (A negated operand is free in a scalar instruction but costs a packed one
+// an extra operation, so negations are placed on operands that are reused.)
+struct DFP {
+    float2 hi, lo;
+};
+
+// (PTX with an explicit rounding, which the compiler never contracts; its __fmul2_rn / __fadd2_rn
+// builtins were contracted to FMAs, which breaks the error-free transformations)
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{.reg .b64 a, b, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; add.rn.f32x2 d, a, b; mov.b64 {%0, %1}, d;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{.reg .b64 a, b, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; sub.rn.f32x2 d, a, b; mov.b64 {%0, %1}, d;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{.reg .b64 a, b, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; mul.rn.f32x2 d, a, b; mov.b64 {%0, %1}, d;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{.reg .b64 a, b, c, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; mov.b64 c, {%6, %7}; "
+        "fma.rn.f32x2 d, a, b, c; mov.b64 {%0, %1}, d;}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ DFP dfp_dup(DF a) { return {dup2(a.hi), dup2(a.lo)}; }
+// (a, -a)
+__device__ __forceinline__ DFP dfp_pm(DF a) { return {make_float2(a.hi, -a.hi), make_float2(a.lo, -a.lo)}; }
+__device__ __forceinline__ DF dfp_x(DFP a) { return {a.hi.x, a.lo.x}; }
+__device__ __forceinline__ DF dfp_y(DFP a) { return {a.hi.y, a.lo.y}; }
+
+__device__ __forceinline__ DFP dfp_add(DFP a, DFP b)
+{
+    const float2 s = add2(a.hi, b.hi);
+    const float2 bb = sub2(s, a.hi);
+    const float2 e = add2(add2(sub2(a.hi, sub2(s, bb)), sub2(b.hi, bb)), add2(a.lo, b.lo));
+    const float2 h = add2(s, e);
+    return {h, sub2(e, sub2(h, s))};
+}
+
+__device__ __forceinline__ DFP dfp_mul(DFP a, DFP b)
+{
+    const float2 p = mul2(a.hi, b.hi);
+    float2 e = fma2(a.hi, b.hi, neg2(p));
+    e = fma2(a.hi, b.lo, e);
+    return {p, fma2(a.lo, b.hi, e)};
+}
+
+// 1 / x and 1 / sqrt(x) of the two halves (df_rcp, df_rsqrt)
+__device__ __forceinline__ DFP dfp_rcp(DFP x)
+{
+    float2 r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(x.hi.x));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(x.hi.y));
+    const float2 nr = neg2(r);
+    float2 e = fma2(x.hi, nr, dup2(1.0f));
+    e = fma2(x.lo, nr, e);
+    const float2 d = mul2(r, fma2(e, e, e)), h = add2(r, d);
+    return {h, sub2(d, sub2(h, r))};
+}
+
+__device__ __forceinline__ DFP dfp_rsqrt(DFP x)
+{
+    float2 r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(x.hi.x));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(x.hi.y));
+    const float2 nr = neg2(r);
+    const float2 p = mul2(r, r), npe = fma2(r, nr, p), np = neg2(p);   // r^2 = p - npe
+    float2 e = fma2(x.hi, np, dup2(1.0f));
+    e = fma2(x.hi, npe, e);
+    e = fma2(x.lo, np, e);
+    const float2 d = mul2(mul2(r, e), fma2(dup2(0.375f), e, dup2(0.5f))), h = add2(r, d);
+    return {h, sub2(d, sub2(h, r))};
 }
 
 // floor and ceil of hi + lo (renormalised first, so that lo only matters when hi is an integer)
 __device__ __forceinline__ float df_floor(DF x)
 {
     x = df_norm(x.hi, x.lo);
+    const float f = floorf(x.hi);
+    return (f == x.hi && x.lo < 0.0f) ? f - 1.0f : f;
+}
+// floor of a renormalised pair (a df_add's result)
+__device__ __forceinline__ float df_floor_sum(DF x)
+{
     const float f = floorf(x.hi);
     return (f == x.hi && x.lo < 0.0f) ? f - 1.0f : f;
 }

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256, 3) k_node_gradients(Grid G, Node* __restr
         if (bgdf) {
             NodeDF o;
 #pragma unroll
-            for (int el = 0; el < 8; ++el) o.q[el] = make_float4(q[2 * el].hi, q[2 * el].lo, q[2 * el + 1].hi, q[2 * el + 1].lo);
+            for (int el = 0; el < 8; ++el) o.q[el] = make_float4(q[2 * el].hi, q[2 * el + 1].hi, q[2 * el].lo, q[2 * el + 1].lo);
             bgdf[c] = o;
         }
         if (bg32) {
@@ -160,11 +160,6 @@ __global__ void __launch_bounds__(256, 3) k_node_gradients(Grid G, Node* __restr
             bg32[c] = o;
         }
     }
-}
-
-void configure_launch_kernels()
-{
-    cudaFuncSetAttribute(k_set_background, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
 }
 
 void launch_set_background(Context& c, int member, const double* u, const double* v, const double* n2,
@@ -380,31 +375,35 @@ __device__ __forceinline__ double f_am(double p, double tau, double fs, double f
     return 0.5 * (sol_p * (1.0 + ct) + sol_m * (1.0 - ct));
 }
 
-struct Bin {
-    int i, j, member;
-    double z_launch, dz_launch, theta, c, lambda_h, flux, frac;
+// What a launch needs of its column at the launch level; flux = the flux of one bin, hY = 0 where the
+// source does not launch.  64 bytes.
+struct LaunchColumn {
+    double U, V, N2, G2, f2, hX, hY, flux;
 };
 
-// 0 = filtered, 1 = launched (state in s)
-__device__ __forceinline__ int make_launch(const Grid& G, const Node* __restrict__ bg_all, const Bin& b,
-                                           double s[NSTATE])
+__device__ __forceinline__ void launch_column(const Grid& G, const Node* __restrict__ bg, int i, int j, double Z,
+                                              LaunchColumn& col)
 {
-    const Node* bg = bg_all + (int64_t)b.member * G.ncell;
-    const double X = __dmul_rn(b.i + 0.5, G.dX);
-    const double Y = row_lat(G, b.j);
-    const double Z = b.z_launch + 0.5 * b.dz_launch;
-    Bg bk;
-    gather_values_fp64(G, bg, X, Y, Z, bk.v);
+    const double X = __dmul_rn(i + 0.5, G.dX), Y = row_lat(G, j);
+    double v[4];
+    gather_values_fp64(G, bg, X, Y, Z, v);
     Geo g;
     geometry_at(G, Y, Z, g);
-    double f2, df2;
-    coriolis(G, g.sphi, g.cphi, f2, df2);
-    const double U = bk.v[0], V = bk.v[1], N2 = bk.v[2], G2 = bk.v[3];
-    const double kh = 2.0 * kPi / b.lambda_h;
-    double st, ct;
-    sincos(b.theta, &st, &ct);
+    double df2;
+    coriolis(G, g.sphi, g.cphi, col.f2, df2);
+    col.U = v[0]; col.V = v[1]; col.N2 = v[2]; col.G2 = v[3];
+    col.hX = g.hX; col.hY = g.hY;
+}
+
+// The launch state of a bin (horizontal wavenumber kh in direction (ct, st), phase speed c) in column
+// (i, j): 0 = filtered, 1 = launched (state in s)
+__device__ __forceinline__ int launch_state(const Grid& G, const LaunchColumn& col, int i, int j, double z_launch,
+                                            double dz_launch, double kh, double st, double ct, double c,
+                                            double flux, double frac, double s[NSTATE])
+{
+    const double U = col.U, V = col.V, N2 = col.N2, G2 = col.G2, f2 = col.f2;
     const double k = kh * ct, l = kh * st;
-    const double w = kh * b.c - (k * U + l * V);
+    const double w = kh * c - (k * U + l * V);
     if (!(w > 0.0 && w * w > f2 && w * w < N2)) return 0;
     const double m2 = kh * kh * (N2 - w * w) / (w * w - f2) - G2;
     if (!(m2 > 0.0)) return 0;
@@ -412,53 +411,49 @@ __device__ __forceinline__ int make_launch(const Grid& G, const Node* __restrict
     Disp d;
     dispersion(kh * kh, m2 + G2, N2, f2, d);
     const double chr = -m * kh * kh * d.c;
-    const double A = b.flux / (kh * chr);   // once per launched ray: IEEE division is fine here
-    const double dk = b.frac * kh, dl = b.frac * kh, dm = b.frac * fabs(m);
-    s[SX] = X; s[SY] = Y; s[SZ] = Z;
+    const double A = flux / (kh * chr);   // once per launched ray: IEEE division is fine here
+    const double dk = frac * kh, dl = frac * kh, dm = frac * fabs(m);
+    s[SX] = __dmul_rn(i + 0.5, G.dX); s[SY] = row_lat(G, j); s[SZ] = z_launch + 0.5 * dz_launch;
     s[SK] = k; s[SL] = l; s[SM] = m;
-    s[SEX] = G.dX; s[SEY] = G.dY; s[SEZ] = b.dz_launch;
-    s[SPX] = g.hX * G.dX * dk;
-    s[SPY] = g.hY * G.dY * dl;
-    s[SPZ] = b.dz_launch * dm;
+    s[SEX] = G.dX; s[SEY] = G.dY; s[SEZ] = dz_launch;
+    s[SPX] = col.hX * G.dX * dk;
+    s[SPY] = col.hY * G.dY * dl;
+    s[SPZ] = dz_launch * dm;
     s[SN] = A / (dk * dl * dm);
     return ray_status(G, s) == 0 ? 1 : 0;
 }
 
-__device__ __forceinline__ bool source_bin(const Grid& G, const gwam_bg_source& src, int t, Bin& b)
+// The background source's columns, a thread each: the trilinear values, the metric and the seasonal
+// flux are FP64 work that all bins of a column share (they took most of a launch while every bin
+// repeated them).
+__global__ void k_launch_columns(Grid G, const Node* __restrict__ bg, gwam_bg_source src, LaunchColumn* __restrict__ cols)
 {
-    const int nbins = src.n_az * src.n_c;
-    const int gcol = t / nbins, bin = t % nbins;
-    b.member = gcol / G.ncol;
-    const int col = gcol - b.member * G.ncol;
-    b.j = col / G.nx;
-    b.i = col % G.nx;
-    const double pdeg = row_lat(G, b.j) * (180.0 / kPi);
-    if (fabs(pdeg) > src.phi_max_deg) return false;
-    const double fbin = f_am(pdeg, src.tau, src.f_s, src.f_w) / nbins;
-    if (fbin == 0.0 && !src.launch_zero_flux) return false;
-    const int a = bin / src.n_c, q = bin % src.n_c;
-    b.theta = 2.0 * kPi * a / src.n_az;
-    b.c = src.n_c == 1 ? src.c_min : src.c_min * pow(src.c_max / src.c_min, (double)q / (src.n_c - 1));
-    b.z_launch = src.z_launch;
-    b.dz_launch = src.dz_launch;
-    b.lambda_h = src.lambda_h;
-    b.flux = fbin;
-    b.frac = src.spectral_frac;
-    return true;
+    const double Z = src.z_launch + 0.5 * src.dz_launch;
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G.ncol_all; g += gridDim.x * blockDim.x) {
+        const int mem = g / G.ncol, col = g - mem * G.ncol;
+        const int j = col / G.nx, i = col - j * G.nx;
+        const double pdeg = row_lat(G, j) * (180.0 / kPi);
+        LaunchColumn o{};
+        bool on = !(fabs(pdeg) > src.phi_max_deg);
+        if (on) {
+            const double fbin = f_am(pdeg, src.tau, src.f_s, src.f_w) / (src.n_az * src.n_c);
+            on = !(fbin == 0.0 && !src.launch_zero_flux);
+            if (on) {
+                launch_column(G, bg + (int64_t)mem * G.ncell, i, j, Z, o);
+                o.flux = fbin;
+            }
+        }
+        cols[g] = o;
+    }
 }
 
-__device__ __forceinline__ bool spec_bin(const Grid& G, Ctl* ctl, const gwam_spec& sp, Bin& b)
+// device-resident specs are not seen by the host: a column or member outside the grid is an
+// input error (status GWAM_EINVAL, read at the next synchronising call), never an index
+__device__ __forceinline__ bool spec_in_grid(const Grid& G, Ctl* ctl, const gwam_spec& sp)
 {
-    // device-resident specs are not seen by the host: a column or member outside the grid is an
-    // input error (status GWAM_EINVAL, read at the next synchronising call), never an index
-    if (sp.i < 0 || sp.i >= G.nx || sp.j < 0 || sp.j >= G.ny || sp.member < 0 || sp.member >= G.members) {
-        set_status(ctl, GWAM_EINVAL);
-        return false;
-    }
-    b.i = sp.i; b.j = sp.j; b.member = sp.member;
-    b.z_launch = sp.z_launch; b.dz_launch = sp.dz_launch; b.theta = sp.theta; b.c = sp.c;
-    b.lambda_h = sp.lambda_h; b.flux = sp.flux; b.frac = sp.spectral_frac;
-    return true;
+    if (sp.i >= 0 && sp.i < G.nx && sp.j >= 0 && sp.j < G.ny && sp.member >= 0 && sp.member < G.members) return true;
+    set_status(ctl, GWAM_EINVAL);
+    return false;
 }
 
 // Ghost-layer emission (Sec. 3c): the launch state s fills the layer [z_launch, z_launch + dz_launch]
@@ -466,16 +461,22 @@ __device__ __forceinline__ bool spec_bin(const Grid& G, Ctl* ctl, const gwam_spe
 // on the grid this kernel is given).  Returns 1 with s = the part above the layer top (vertical
 // extent from the layer top, or the ghost's own bottom if it left whole, to its top; P_z in
 // proportion; the ghost's m), 0 when the ghost was reflected in the layer (m no longer negative) or
-// the part lies outside the domain, 2 when nothing has left the layer.
-__device__ __forceinline__ int ghost_emit(const Grid& G, const NodeDF* __restrict__ bgdf, const Bin& b, double dt,
-                                          double s[NSTATE], double* sh)
+// the part lies outside the domain, 2 when nothing has left the layer.  All 32 lanes of a warp must
+// call it (their stages gather together); lanes without a launch state (on = false) return 0.
+__device__ __forceinline__ int ghost_emit(const Grid& G, const NodeDF* __restrict__ bgdf, bool on, int member,
+                                          double z_launch, double dz_launch, double dt, double s[NSTATE],
+                                          const RkSlots& sl)
 {
-    double y[NSTATE];
+    double y[9];
 #pragma unroll
-    for (int c = 0; c < NSTATE; ++c) y[c] = s[c];
-    rk3(G, bgdf + (int64_t)b.member * G.ncell, y, dt, sh);
+    for (int c = 0; c < 9; ++c) y[c] = on ? s[c] : 0.0;
+    rk3_start(sl, y);
+    rk3(G, bgdf, on ? member * G.ncell : 0, dt, sl);
+    if (!on) return 0;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) y[c] += rk_increment(sl, c);
     if (!(y[SM] < 0.0)) return 0;
-    const double layer_top = b.z_launch + b.dz_launch;
+    const double layer_top = z_launch + dz_launch;
     const double top = y[SZ] + 0.5 * y[SEZ], bot = y[SZ] - 0.5 * y[SEZ];
     if (!(top > layer_top)) return 2;
     const double lo = bot > layer_top ? bot : layer_top;
@@ -486,59 +487,125 @@ __device__ __forceinline__ int ghost_emit(const Grid& G, const NodeDF* __restric
     return ray_status(G, s) == 0 ? 1 : 0;
 }
 
-// pass 0: flag[t] = launches?, count filtered bins; pass 1: write launched rays in order.
-// kGhost: emit what left the ghost layer over ghost_dt instead of the launch state itself.
+// Launch states of all bins: flag[t] = launched, the state (record of the context's form, id = the
+// member alone) staged at position t of S / S32, filtered bins counted; k_launch_place then moves the
+// launched ones behind the live rays.  (While both passes computed the states, a ghost-layer launch
+// into 8192 columns took 2 x 390 us.)  kGhost: what left the ghost layer over ghost_dt instead of
+// the launch state itself.  Dynamic shared memory: the ghost's kRkSmem, then the source's sines and cosines
+// of the azimuths and its phase speeds (2 n_az + n_c doubles).
 template <bool kSpec, bool kGhost>
-__global__ void k_launch(Grid G, const Node* __restrict__ bg, const NodeDF* __restrict__ bgdf, RaySoA A,
-                         Ray32SoA A32, bool f32, Ctl* ctl, int64_t max_rays,
-                         gwam_bg_source src, const gwam_spec* __restrict__ specs, int total, double ghost_dt,
-                         int pass, int* __restrict__ flag, double* __restrict__ partials, int pstride)
+__global__ void __launch_bounds__(kThreads, 2) k_launch(Grid G, const Node* __restrict__ bg,
+                                                        const NodeDF* __restrict__ bgdf, RaySoA S, Ray32SoA S32s, bool f32,
+                                                        Ctl* ctl, gwam_bg_source src,
+                                                        const LaunchColumn* __restrict__ cols,
+                                                        const gwam_spec* __restrict__ specs, int total, double ghost_dt,
+                                                        int* __restrict__ flag)
 {
-    __shared__ double sh_state[kGhost ? 18 * kThreads : 1];
+    extern __shared__ float4 sh_launch[];
+    double* const az = reinterpret_cast<double*>(sh_launch + (kGhost ? kRkSmem / sizeof(float4) : 0));
+    double* const speed = az + 2 * src.n_az;
+    const int nbins = kSpec ? 1 : src.n_az * src.n_c;
+    if (!kSpec) {
+        for (int a = threadIdx.x; a < src.n_az; a += blockDim.x) sincos(2.0 * kPi * a / src.n_az, &az[2 * a], &az[2 * a + 1]);
+        for (int q = threadIdx.x; q < src.n_c; q += blockDim.x)
+            speed[q] = src.n_c == 1 ? src.c_min : src.c_min * pow(src.c_max / src.c_min, (double)q / (src.n_c - 1));
+        __syncthreads();
+    }
+    const double kh_src = kSpec ? 0.0 : 2.0 * kPi / src.lambda_h;
+    long long filtered = 0;
+    for (int t0 = blockIdx.x * blockDim.x; t0 < total; t0 += gridDim.x * blockDim.x) {
+        const int t = t0 + threadIdx.x;
+        double s[NSTATE];
+        bool eligible = t < total;
+        int ok = 0, mem = 0;
+        double z_launch = src.z_launch, dz_launch = src.dz_launch;
+        if (eligible && kSpec) {
+            const gwam_spec sp = specs[t];
+            eligible = spec_in_grid(G, ctl, sp);
+            if (eligible) {
+                mem = sp.member;
+                z_launch = sp.z_launch;
+                dz_launch = sp.dz_launch;
+                LaunchColumn col;
+                launch_column(G, bg + (int64_t)mem * G.ncell, sp.i, sp.j, z_launch + 0.5 * dz_launch, col);
+                double st, ct;
+                sincos(sp.theta, &st, &ct);
+                ok = launch_state(G, col, sp.i, sp.j, z_launch, dz_launch, 2.0 * kPi / sp.lambda_h, st, ct, sp.c, sp.flux,
+                                  sp.spectral_frac, s);
+            }
+        } else if (eligible) {
+            const int g = t / nbins, bin = t - g * nbins;
+            const LaunchColumn col = cols[g];
+            eligible = col.hY != 0.0;
+            if (eligible) {
+                mem = g / G.ncol;
+                const int c = g - mem * G.ncol, j = c / G.nx, a = bin / src.n_c;
+                ok = launch_state(G, col, c - j * G.nx, j, z_launch, dz_launch, kh_src, az[2 * a], az[2 * a + 1],
+                                  speed[bin - a * src.n_c], col.flux, src.spectral_frac, s);
+            }
+        }
+        if (kGhost && __any_sync(0xffffffffu, ok)) {
+            const int e = ghost_emit(G, bgdf, ok != 0, mem, z_launch, dz_launch, ghost_dt, s, RkSlots(sh_launch));
+            if (e == 2) eligible = false;      // nothing left the layer: neither launched nor filtered
+            ok = e == 1;
+        }
+        if (t >= total) continue;
+        if (eligible && !ok) ++filtered;
+        flag[t] = ok;
+        if (!ok) continue;
+        if (f32) {
+            S32 r;
+            from_double(G, s, with_member(mem, 0), r);
+            store32(G, S32s, t, r);
+        } else {
+            store_ray(S, t, s, with_member(mem, 0));
+        }
+    }
+    const long long fb = block_sum(filtered);
+    if (threadIdx.x == 0 && fb) atomicAdd((unsigned long long*)&ctl->n_filtered, (unsigned long long)fb);
+}
+
+// The staged launches t with off[t + 1] > off[t] to position n + off[t], id next_id + off[t]
+__global__ void k_launch_place(Grid G, RaySoA S, Ray32SoA S32s, RaySoA A, Ray32SoA A32, bool f32, Ctl* ctl,
+                               int64_t max_rays, int total, const int* __restrict__ off, double* __restrict__ partials,
+                               int pstride)
+{
     const int n0 = ctl->n;
     const long long next = ctl->next_id;
     double w = 0.0;
-    long long filtered = 0;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        Bin b;
-        bool eligible = kSpec ? spec_bin(G, ctl, specs[t], b) : source_bin(G, src, t, b);
-        double s[NSTATE];
-        int ok = 0;
-        if (eligible) {
-            ok = make_launch(G, bg, b, s);
-            if (kGhost && ok) {
-                const int e = ghost_emit(G, bgdf, b, ghost_dt, s, sh_state + threadIdx.x);
-                ok = e == 1;
-                if (e == 2) eligible = false;      // nothing left the layer: neither launched nor filtered
-            }
-            if (eligible && !ok) ++filtered;
+        const int o = off[t];
+        if (off[t + 1] == o) continue;
+        const int64_t pos = (int64_t)n0 + o;
+        if (pos >= max_rays) {
+            set_status(ctl, GWAM_ECAPACITY);
+            continue;
         }
-        if (pass == 0) {
-            flag[t] = ok;
-        } else if (ok) {
-            const int64_t pos = (int64_t)n0 + flag[t];
-            if (pos >= max_rays) {
-                set_status(ctl, GWAM_ECAPACITY);
-                continue;
-            }
-            const long long id = with_member(b.member, next + flag[t]);
-            if (f32) {
-                S32 r;
-                from_double(G, s, id, r);
-                store32(G, A32, pos, r);
-                w += (double)action32(r);
-            } else {
-                store_ray(A, pos, s, id);
-                w += ray_action(s);
-            }
+        if (f32) {
+            S32 r;
+            load32(G, S32s, t, r);
+            r.id += next + o;
+            store32(G, A32, pos, r);
+            w += (double)action32(r);
+        } else {
+            double s[NSTATE];
+            long long id;
+            load_ray(S, t, s, id);
+            store_ray(A, pos, s, id + next + o);
+            w += ray_action(s);
         }
     }
     const double wb = block_sum(w);
-    const long long fb = block_sum(filtered);
-    if (threadIdx.x == 0) {
-        if (pass == 1) partials[T_LAUNCH * pstride + blockIdx.x] = wb;
-        if (pass == 0 && fb) atomicAdd((unsigned long long*)&ctl->n_filtered, (unsigned long long)fb);
-    }
+    if (threadIdx.x == 0) partials[T_LAUNCH * pstride + blockIdx.x] = wb;
+}
+
+void configure_launch_kernels()
+{
+    cudaFuncSetAttribute(k_set_background, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    // a source has at most 1024 bins, so n_az + n_c <= 1025
+    cudaFuncSetAttribute(k_launch<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(kRkSmem + 2050 * sizeof(double)));
+    cudaFuncSetAttribute(k_launch<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRkSmem);
 }
 
 __global__ void k_launch_close(Ctl* ctl, int64_t max_rays, const int* off, int total)
@@ -551,60 +618,52 @@ __global__ void k_launch_close(Ctl* ctl, int64_t max_rays, const int* off, int t
     ctl->n_launched += added;
 }
 
-static int* launch_scratch(Context& c, int64_t need)
-{
-    if (need + 1 > c.max_rays + 1) {
-        // the per-ray scratch `newid` holds max_rays + 1 ints; larger launches need their own
-        int* p = nullptr;
-        if (cudaMallocAsync((void**)&p, sizeof(int) * (size_t)(need + 1), c.stream) != cudaSuccess) {
-            c.err = "launch: scratch allocation failed";
-            throw (int)GWAM_ENOMEM;
-        }
-        return p;
-    }
-    return c.newid;
-}
-
-static void launch_pass(Context& c, const Grid& G, const gwam_bg_source& s0, const gwam_spec* specs, int total,
-                        double ghost_dt, int pass, int* flag)
-{
-    const int nb = c.grid_blocks;
-    const bool ghost = ghost_dt > 0.0;
-    if (specs && ghost)
-        k_launch<true, true><<<nb, kThreads, 0, c.stream>>>(G, c.bg, c.bgdf, c.A, c.A32, c.f32, c.ctl, c.max_rays, s0,
-                                                            specs, total, ghost_dt, pass, flag, c.partials,
-                                                            c.max_blocks);
-    else if (specs)
-        k_launch<true, false><<<nb, kThreads, 0, c.stream>>>(G, c.bg, c.bgdf, c.A, c.A32, c.f32, c.ctl, c.max_rays, s0,
-                                                             specs, total, ghost_dt, pass, flag, c.partials,
-                                                             c.max_blocks);
-    else if (ghost)
-        k_launch<false, true><<<nb, kThreads, 0, c.stream>>>(G, c.bg, c.bgdf, c.A, c.A32, c.f32, c.ctl, c.max_rays, s0,
-                                                             specs, total, ghost_dt, pass, flag, c.partials,
-                                                             c.max_blocks);
-    else
-        k_launch<false, false><<<nb, kThreads, 0, c.stream>>>(G, c.bg, c.bgdf, c.A, c.A32, c.f32, c.ctl, c.max_rays, s0,
-                                                              specs, total, ghost_dt, pass, flag, c.partials,
-                                                              c.max_blocks);
-}
-
 static void launch_common(Context& c, const gwam_bg_source* src, const gwam_spec* specs, int64_t total,
                           double ghost_dt = 0.0)
 {
     if (total <= 0) return;
-    int* flag = launch_scratch(c, total);
+    const int nb = c.grid_blocks;
+    const bool ghost = ghost_dt > 0.0;
+    // The re-binned ray buffer is free between steps: launch states of up to max_rays bins are staged
+    // there, their flags in the per-ray scratch.  Larger launches (most bins filtered, or an overflow
+    // to be reported) bring their own.
+    RaySoA S = c.B;
+    Ray32SoA S32s = c.B32;
+    int* flag = c.newid;
+    char* own = nullptr;
+    if (total > c.max_rays) {
+        const size_t rec = c.f32 ? 4 * sizeof(float4) : 7 * sizeof(double2);
+        if (cudaMallocAsync((void**)&own, rec * (size_t)total + sizeof(int) * (size_t)(total + 1), c.stream) != cudaSuccess) {
+            cudaGetLastError();
+            c.err = "launch: scratch allocation failed";
+            throw (int)GWAM_ENOMEM;
+        }
+        for (int q = 0; q < 7; ++q) S.a[q] = reinterpret_cast<double2*>(own) + q * total;
+        for (int q = 0; q < 4; ++q) S32s.q[q] = reinterpret_cast<float4*>(own) + q * total;
+        flag = reinterpret_cast<int*>(own + rec * (size_t)total);
+    }
     gwam_bg_source s0{};
     if (src) s0 = *src;
     // the ghost layer propagates vertically only: the single-column equations on this grid copy
     Grid G = c.G;
-    if (ghost_dt > 0.0) G.columnar = 1;
-    launch_pass(c, G, s0, specs, (int)total, ghost_dt, 0, flag);
+    if (ghost) G.columnar = 1;
+    const size_t shm = (ghost ? kRkSmem : 0) + (specs ? 0 : (2 * s0.n_az + s0.n_c) * sizeof(double));
+    if (!specs) {
+        const int cb = std::min((c.G.ncol_all + 63) / 64, 32 * c.num_sms);
+        k_launch_columns<<<cb, 64, 0, c.stream>>>(c.G, c.bg, s0, reinterpret_cast<LaunchColumn*>(c.launch_cols));
+    }
+    auto* kernel = specs ? (ghost ? k_launch<true, true> : k_launch<true, false>)
+                         : (ghost ? k_launch<false, true> : k_launch<false, false>);
+    kernel<<<std::min<int>(nb, (int)((total + kThreads - 1) / kThreads)), kThreads, shm, c.stream>>>(
+        G, c.bg, c.bgdf, S, S32s, c.f32, c.ctl, s0, reinterpret_cast<const LaunchColumn*>(c.launch_cols), specs,
+        (int)total, ghost_dt, flag);
     exclusive_scan(c, flag, flag, total, nullptr);
     cudaMemsetAsync(c.partials, 0, sizeof(double) * NTALLY * (size_t)c.max_blocks, c.stream);
-    launch_pass(c, G, s0, specs, (int)total, ghost_dt, 1, flag);
+    k_launch_place<<<nb, kThreads, 0, c.stream>>>(c.G, S, S32s, c.A, c.A32, c.f32, c.ctl, c.max_rays, (int)total, flag,
+                                                  c.partials, c.max_blocks);
     finalize_tallies(c, 1 << T_LAUNCH, 0);
     k_launch_close<<<1, 1, 0, c.stream>>>(c.ctl, c.max_rays, flag, (int)total);
-    if (flag != c.newid) cudaFreeAsync(flag, c.stream);
+    if (own) cudaFreeAsync(own, c.stream);
 }
 
 void launch_background_source(Context& c, const gwam_bg_source& src)

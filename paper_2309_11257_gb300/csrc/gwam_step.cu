@@ -297,12 +297,9 @@ void exclusive_scan2(Context& c, const int* in0, int* out0, int64_t n0, const in
 
 // ============================================================================ advance
 
-// Shared memory of k_advance, per thread (slots kThreads apart): the RK3 state, increment sums,
-// low-storage register and the extents' double-float copy (36 doubles, rk3<true, true>), then the
-// exit / invalid action sums and four counters (6) -- out of the 128 registers the ray equations
-// need at two blocks per SM (no spills)
-constexpr int kAdvanceRkSlots = 36;
-constexpr size_t kAdvanceSmem = sizeof(double) * (kAdvanceRkSlots + 6) * kThreads;
+// Shared memory of k_advance: rk3's slots, then per thread (kThreads apart) the exit / invalid action
+// sums and four counters -- out of the 128 registers the ray equations need at two blocks per SM
+constexpr size_t kAdvanceSmem = kRkSmem + 6 * kThreads * sizeof(double);
 
 __global__ void __launch_bounds__(kThreads, 2) k_advance(Grid G, Params P, RaySoA A, const NodeDF* __restrict__ bg,
                                                         Ctl* ctl, double dt, int* __restrict__ info,
@@ -310,40 +307,52 @@ __global__ void __launch_bounds__(kThreads, 2) k_advance(Grid G, Params P, RaySo
                                                         int* __restrict__ newid, int* __restrict__ cnt,
                                                         double* __restrict__ partials, int pstride, ClearSet zs)
 {
-    extern __shared__ double sh_state[];   // kAdvanceSmem bytes
+    extern __shared__ float4 sh_advance[];   // kAdvanceSmem bytes
+    const RkSlots sl(sh_advance);
     const int n = ctl->n;
     // this thread's exit / invalid action sums and its exit, invalid, vertical- and horizontal-split
     // counters, updated in shared memory where they occur: not held in registers across the stages
-    double* const tw = sh_state + kAdvanceRkSlots * kThreads + threadIdx.x;
+    double* const tw = reinterpret_cast<double*>(sh_advance + kRkSmem / sizeof(float4)) + threadIdx.x;
     long long* const tn = reinterpret_cast<long long*>(tw + 2 * kThreads);
     tw[0] = 0.0;
     tw[kThreads] = 0.0;
 #pragma unroll
     for (int c = 0; c < 4; ++c) tn[c * kThreads] = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int passes = loop_passes(n);
+    for (int m = 0; m < passes; ++m) {
+        // the projected fields, with stores (bulk copies were measured slower here: 0.680 -> 0.741 ms)
+        clear_fields(zs, m, passes);
+        const int ray = loop_ray(m, passes);
+        if (ray - (int)(threadIdx.x & 31) >= n) continue;   // a whole warp without rays
+        // lanes past the last ray follow it through the stages (their warp gathers together), then stop
+        const int i = min(ray, n - 1);
         double s[NSTATE];
-        long long id;
-        // the nine propagated components and the id (its member selects the background) now;
-        // P_x, P_y, P_z and N, which the stages do not touch, after them: out of the registers the
-        // ray equations need
+        const long long id = __ldg(reinterpret_cast<const long long*>(&A.a[6][i]) + 1);
+        {
+            // the nine propagated components; the whole record is read again after the stages, out of
+            // the registers the ray equations need
+            double y[9];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const double2 v = __ldg(&A.a[q][i]);
+            for (int q = 0; q < 4; ++q) {
+                const double2 v = __ldg(&A.a[q][i]);
+                y[2 * q] = v.x;
+                y[2 * q + 1] = v.y;
+            }
+            y[8] = __ldg(reinterpret_cast<const double*>(&A.a[4][i]));
+            rk3_start(sl, y);
+        }
+        const int mem = member_of(id);
+        rk3(G, bg, mem * G.ncell, dt, sl);
+        if (ray >= n) continue;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            const double2 v = A.a[q][i];
             s[2 * q] = v.x;
             s[2 * q + 1] = v.y;
         }
-        s[SEZ] = __ldg(reinterpret_cast<const double*>(&A.a[4][i]));
-        id = __ldg(reinterpret_cast<const long long*>(&A.a[6][i]) + 1);
-        const int mem = member_of(id);
-        const NodeDF* bgm = bg + (int64_t)mem * G.ncell;
-        rk3<true, true>(G, bgm, s, dt, sh_state + threadIdx.x);
-        s[SPX] = __ldg(reinterpret_cast<const double*>(&A.a[4][i]) + 1);
-        {
-            const double2 v = __ldg(&A.a[5][i]);
-            s[SPY] = v.x;
-            s[SPZ] = v.y;
-        }
-        s[SN] = __ldg(reinterpret_cast<const double*>(&A.a[6][i]));
+        s[SN] = A.a[6][i].x;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) s[c] += rk_increment(sl, c);
         wrap_position(G, s);
         const int st = ray_status(G, s);
         int code = 0, nch = 0;
@@ -380,8 +389,6 @@ __global__ void __launch_bounds__(kThreads, 2) k_advance(Grid G, Params P, RaySo
         cslot[i] = make_int4(sl[0], sl[1], sl[2], sl[3]);
         newid[i] = nch > 0 ? nch - 1 : 0;
     }
-    // the projected fields, with stores (bulk copies were measured slower here: 0.680 -> 0.741 ms)
-    clear_fields(zs);
     const double we = block_sum(tw[0]);
     const double wi = block_sum(tw[kThreads]);
     const long long ne = block_sum(tn[0]), ni = block_sum(tn[kThreads]), nv = block_sum(tn[2 * kThreads]),
@@ -660,7 +667,7 @@ __global__ void k_sat_kappa(const Ctl* ctl, const int* __restrict__ off2, const 
 // Centre fields: cell averages over the ray volumes whose carrier is in the cell, weight V_j/V_c.
 // Interface fields (z = kk dz, 1 <= kk < nz): staggered-cell overlap, weight w_h * overlap / dz.
 template <bool THETA>
-__global__ void __launch_bounds__(kThreads) k_project(Grid G, Params P, RaySoA B, const NodeDF* __restrict__ bg,
+__global__ void __launch_bounds__(kThreads, THETA ? 3 : 4) k_project(Grid G, Params P, RaySoA B, const NodeDF* __restrict__ bg,
                                                         const Ctl* ctl, const int* __restrict__ off2,
                                                         const double* __restrict__ kappa,
                                                         const double* __restrict__ k2, double dt,
