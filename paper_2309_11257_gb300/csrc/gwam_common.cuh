@@ -145,6 +145,135 @@ __device__ __forceinline__ bool warp_run_interior(int key)
     return start > 0 && end < 31;
 }
 
+// ---------------------------------------------------------------------------- per-column cap (App. B.5)
+
+// Doubles as unsigned integers of the same order (-0 = +0, NaN above everything): comparisons on the
+// integer pipe (an FP64 compare runs at GB300's FP64 rate).
+__device__ __forceinline__ unsigned long long order_key(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x), top = 1ull << 63;
+    if ((b & ~top) > 0x7FF0000000000000ull) return ~0ull;
+    if (b & top) return b == top ? top : ~b;
+    return b | top;
+}
+// the key of a number's multiple by f
+__device__ __forceinline__ unsigned long long key_scaled(unsigned long long key, double f)
+{
+    const unsigned long long top = 1ull << 63;
+    return order_key(__longlong_as_double((long long)((key & top) ? key ^ top : ~key)) * f);
+}
+
+constexpr int kCapThreads = 128;
+constexpr int kCapKeys = 1024;   // keys held in shared memory; longer columns keep theirs in global scratch
+constexpr double kCapDelta = 1.0 / (1ll << 36);
+
+// The entries [a, a + count) that the cap removes from an over-full column: the `drop` with the lowest
+// energies, ties by the larger id first, as one block (kCapThreads).  energy(e) may be off by kCapDelta / 2
+// relative: the drop-th lowest is found by a radix select over the keys (8 bits a pass, until one
+// key is left; counting every entry's rank took count^2 FP64 comparisons), entries clearly below it go,
+// entries clearly above it stay, and the few within kCapDelta of it are ranked by exact(e).
+// A NaN energy always goes and counts towards nobody's rank.  remove(e) is called for each.
+template <class Energy, class Exact, class Remove>
+__device__ __forceinline__ void cap_column(int a, int count, int drop, const long long* __restrict__ ent_id,
+                                           double* __restrict__ scratch, Energy energy, Exact exact, Remove remove)
+{
+    __shared__ unsigned long long sh_keys[kCapKeys];
+    __shared__ int hist[256];
+    __shared__ int sh_digit, sh_left, sh_bin, sh_low, sh_amb;
+    __shared__ unsigned long long sh_cut;
+    unsigned long long* keys = count <= kCapKeys ? sh_keys : reinterpret_cast<unsigned long long*>(scratch) + a;
+    for (int e = threadIdx.x; e < count; e += kCapThreads) keys[e] = order_key(energy(a + e));
+    if (threadIdx.x == 0) sh_low = sh_amb = 0;
+    unsigned long long prefix = 0, mask = 0;
+    int left = drop;   // the drop-th lowest key (1 .. count) among those with this prefix
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        for (int q = threadIdx.x; q < 256; q += kCapThreads) hist[q] = 0;
+        __syncthreads();
+        for (int e = threadIdx.x; e < count; e += kCapThreads)
+            if ((keys[e] & mask) == prefix) atomicAdd(&hist[(int)(keys[e] >> shift) & 255], 1);
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            int h[8], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                h[q] = hist[8 * threadIdx.x + q];
+                sum += h[q];
+            }
+            int before = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int o = __shfl_up_sync(0xffffffffu, before, d);
+                if ((int)threadIdx.x >= d) before += o;
+            }
+            before -= sum;
+            if (before < left && left <= before + sum) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (before < left && left <= before + h[q]) {
+                        sh_digit = 8 * threadIdx.x + q;
+                        sh_left = left - before;
+                        sh_bin = h[q];
+                    }
+                    before += h[q];
+                }
+            }
+        }
+        __syncthreads();
+        prefix |= (unsigned long long)sh_digit << shift;
+        mask |= 255ull << shift;
+        left = sh_left;
+        if (sh_bin == 1) break;
+    }
+    // the one key with the prefix, or the common value of those that share all its digits
+    for (int e = threadIdx.x; e < count; e += kCapThreads)
+        if ((keys[e] & mask) == prefix) sh_cut = keys[e];
+    __syncthreads();
+    const unsigned long long cut = sh_cut;
+    if (cut == ~0ull) {   // more to drop than there are numbers
+        for (int e = threadIdx.x; e < count; e += kCapThreads) remove(a + e);
+        __syncthreads();
+        return;
+    }
+    const unsigned long long k0 = key_scaled(cut, 1.0 - kCapDelta), k1 = key_scaled(cut, 1.0 + kCapDelta);
+    const unsigned long long lo = k0 < k1 ? k0 : k1, hi = k0 < k1 ? k1 : k0;
+    int low = 0, amb = 0;
+    for (int e = threadIdx.x; e < count; e += kCapThreads) {
+        const unsigned long long k = keys[e];
+        low += k < lo;
+        amb += k >= lo && k <= hi;
+    }
+    if (low) atomicAdd(&sh_low, low);
+    if (amb) atomicAdd(&sh_amb, amb);
+    __syncthreads();
+    const int need = drop - sh_low;   // of the sh_amb around the cut
+    if (need == sh_amb) {
+        for (int e = threadIdx.x; e < count; e += kCapThreads)
+            if (keys[e] <= hi || keys[e] == ~0ull) remove(a + e);
+    } else {
+        // entries around the cut get their exact keys, those below 0 (no double's key) and those above
+        // ~0 - 1 (likewise); the exact ones are ranked among themselves
+        for (int e = threadIdx.x; e < count; e += kCapThreads) {
+            const unsigned long long k = keys[e];
+            if (k != ~0ull) keys[e] = k < lo ? 0ull : (k > hi ? ~0ull - 1 : order_key(exact(a + e)));
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < count; e += kCapThreads) {
+            const unsigned long long k = keys[e];
+            if (k == ~0ull - 1) continue;
+            int rank = 0;
+            if (k != 0ull && k != ~0ull) {
+                const long long id = ent_id[a + e];
+                for (int q = 0; q < count; ++q) {
+                    const unsigned long long o = keys[q];
+                    rank += o != 0ull && (o < k || (o == k && ent_id[a + q] > id));
+                }
+            }
+            if (k == 0ull || k == ~0ull || rank < need) remove(a + e);
+        }
+    }
+    __syncthreads();
+}
+
 __device__ __forceinline__ void set_status(Ctl* ctl, int code)
 {
     atomicCAS(&ctl->status, 0, code);

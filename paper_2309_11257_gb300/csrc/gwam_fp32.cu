@@ -463,51 +463,43 @@ __global__ void k_scatter32(Grid G, Ray32SoA A, Ctl* ctl, int64_t max_rays, cons
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_cap_apply32(Grid G, Params P, Ray32SoA A,
-                                                            const Node32* __restrict__ bg, Ctl* ctl,
-                                                            const int* __restrict__ info, const int* __restrict__ off,
-                                                            const int* __restrict__ overlist,
-                                                            const long long* __restrict__ ent_id, int* ent_src,
-                                                            double* ecap, int* cnt, double* __restrict__ partials,
-                                                            int pstride)
+// the cap's choice as in k_cap_apply; here w_hat is an FP32 value either way
+__global__ void __launch_bounds__(kCapThreads) k_cap_apply32(Grid G, Params P, Ray32SoA A,
+                                                               const Node32* __restrict__ bg, Ctl* ctl,
+                                                               const int* __restrict__ info,
+                                                               const int* __restrict__ off,
+                                                               const int* __restrict__ overlist,
+                                                               const long long* __restrict__ ent_id, int* ent_src,
+                                                               const int* __restrict__ ent_cell, double* ecap,
+                                                               int* cnt, double* __restrict__ partials, int pstride)
 {
     double w_cap = 0.0;
     long long n_cap = 0;
     const int nover = ctl->status ? 0 : ctl->n_over;
+    auto child = [&](int e, S32& ch) {
+        const int src = ent_src[e];
+        S32 s;
+        load32(G, A, src >> 2, s);
+        make_child32(G, s, info[src >> 2] & 7, src & 3, ch);
+    };
+    auto energy = [&](int e) {
+        S32 ch;
+        child(e, ch);
+        Intr32 in;
+        intrinsic32(G, bg + (int64_t)member_of(ch.id) * G.ncell, ch, in);
+        return (double)in.w * action32(ch);
+    };
     for (int w = blockIdx.x; w < nover; w += gridDim.x) {
         const int col = overlist[w];
-        const int a = off[col * G.nz], b = off[(col + 1) * G.nz];
-        const int count = b - a;
-        for (int e = a + threadIdx.x; e < b; e += blockDim.x) {
-            const int src = ent_src[e];
-            S32 s, ch;
-            load32(G, A, src >> 2, s);
-            make_child32(G, s, info[src >> 2] & 7, src & 3, ch);
-            Intr32 in;
-            intrinsic32(G, bg + (int64_t)member_of(s.id) * G.ncell, ch, in);
-            ecap[e] = (double)in.w * action32(ch);
-        }
-        __syncthreads();
-        for (int e = a + threadIdx.x; e < b; e += blockDim.x) {
-            const double E = ecap[e];
-            const long long id = ent_id[e];
-            int rank = 0;
-            for (int q = a; q < b; ++q) {
-                const double Eq = ecap[q];
-                rank += (Eq < E) || (Eq == E && ent_id[q] > id);
-            }
-            if (rank < count - P.cap) {
-                const int src = ent_src[e];
-                S32 s, ch;
-                load32(G, A, src >> 2, s);
-                make_child32(G, s, info[src >> 2] & 7, src & 3, ch);
-                w_cap += action32(ch);
-                ++n_cap;
-                atomicSub(&cnt[member_of(s.id) * G.ncell + cell32(G, ch)], 1);
-                ent_src[e] = -1 - src;
-            }
-        }
-        __syncthreads();
+        const int a = off[col * G.nz], count = off[(col + 1) * G.nz] - a;
+        cap_column(a, count, count - P.cap, ent_id, ecap, energy, energy, [&](int e) {
+            S32 ch;
+            child(e, ch);
+            w_cap += action32(ch);
+            ++n_cap;
+            atomicSub(&cnt[ent_cell[e]], 1);
+            ent_src[e] = -1 - ent_src[e];
+        });
     }
     const double wc = block_sum(w_cap);
     const long long nc = block_sum(n_cap);
@@ -758,8 +750,8 @@ void run_step32(Context& c, double dt, double* du, double* dv)
     const int* off2 = c.off;
     if (P.cap > 0) {
         k_cap_find<<<col_blocks, kThreads, 0, s>>>(G, P, c.ctl, c.off, c.overlist);
-        k_cap_apply32<<<nb, kThreads, 0, s>>>(G, P, c.A32, c.bg32, c.ctl, c.info, c.off, c.overlist, c.ent_id,
-                                              c.ent_src, c.ecap, c.cnt, c.partials, c.max_blocks);
+        k_cap_apply32<<<c.max_blocks, kCapThreads, 0, s>>>(G, P, c.A32, c.bg32, c.ctl, c.info, c.off, c.overlist, c.ent_id,
+                                                           c.ent_src, c.ent_cell, c.ecap, c.cnt, c.partials, c.max_blocks);
         exclusive_scan(c, c.cnt, c.off2, G.ncell_all, nullptr);
         off2 = c.off2;
         mask |= 1 << T_CAP;
