@@ -366,17 +366,22 @@ __global__ void __launch_bounds__(kThreads) k_advance32(Grid G, Params P, Ray32S
                                                           double* __restrict__ partials, int pstride, ClearSet zs)
 {
     __shared__ __align__(128) float4 zbuf[kClearPiece / 16];
+    __shared__ float4 sh_rows[kThreads * kRow32 / 4];
+    float* const rows = reinterpret_cast<float*>(sh_rows) + (threadIdx.x >> 5) * 32 * kRow32;
     const int n = ctl->n;
     ClearState cs;
     clear_start(zs, zbuf, n, cs);
     double w_exit = 0.0, w_inv = 0.0;
     long long n_exit = 0, n_inv = 0, n_sv = 0, n_sh = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); i0 < n; i0 += gridDim.x * blockDim.x) {
         if (threadIdx.x == 0) clear_issue(zs, cs, cs.per);
+        // lanes past the last ray follow it through the stages (their warp gathers together), then stop
+        const int ray = i0 + (threadIdx.x & 31), i = min(ray, n - 1);
         S32 s;
         load32(G, A, i, s);
         const int mem = member_of(s.id);
-        rk3_32(G, bg + (int64_t)mem * G.ncell, s, dt);
+        rk3_32(G, bg, mem * G.ncell, s, dt, rows);
+        if (ray >= n) continue;
         const int st = renormalize32(G, s);
         int code = 0, nch = 0;
         int cc[4] = {-1, -1, -1, -1}, sl[4] = {0, 0, 0, 0};

@@ -83,70 +83,129 @@ __device__ __forceinline__ void bracket32(int b, float o, int n, bool periodic, 
     }
 }
 
-// acc += w * node.  kWide: the node's 64 bytes as two 32-byte loads per lane (ld.global.nc.v8.f32;
-// nodes are 64-byte aligned) instead of four 16-byte ones -- half the L1 requests of the gather,
-// whose lanes touch up to 32 distinct lines per request (the ray step: 0.63 -> 0.55 ms per step on
-// the 512 x 256 sphere; the projection and saturation kernels were measured slightly slower with
-// it and keep the 16-byte loads)
-template <bool kWide>
-__device__ __forceinline__ void accumulate32(const Node32* __restrict__ p, float w, float* acc)
-{
-    if (kWide) {
-        const float* q = reinterpret_cast<const float*>(p);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            float a[8];
-            asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(a[4]), "=f"(a[5]), "=f"(a[6]), "=f"(a[7])
-                : "l"(q + 8 * h));
-#pragma unroll
-            for (int e = 0; e < 8; ++e) acc[8 * h + e] = fmaf(w, a[e], acc[8 * h + e]);
-        }
-    } else {
-        const float4* q = reinterpret_cast<const float4*>(p);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const float4 a = __ldg(q + e);
-            acc[4 * e] = fmaf(w, a.x, acc[4 * e]);
-            acc[4 * e + 1] = fmaf(w, a.y, acc[4 * e + 1]);
-            acc[4 * e + 2] = fmaf(w, a.z, acc[4 * e + 2]);
-            acc[4 * e + 3] = fmaf(w, a.w, acc[4 * e + 3]);
-        }
-    }
-}
+// the eight nodes around a position (index of the lowest and steps to the others) and their weights, in
+// the order (i0 j0), (i1 j0), (i0 j1), (i1 j1), each at k0 then k1
+struct Corners32 {
+    int base, ox, oy, oz;
+    float w[8];
+    __device__ __forceinline__ int node(int q) const { return base + ((q & 2) ? ox : 0) + ((q & 4) ? oy : 0) + ((q & 1) ? oz : 0); }
+};
 
-template <bool kWide = false>
-__device__ __forceinline__ void gather32(const Grid& G, const Node32* __restrict__ bg, const S32& s, const float o[3],
-                                         Bg32& b)
+__device__ __forceinline__ Corners32 corners32(const Grid& G, const S32& s, const float o[3])
 {
     int i0, i1, j0, j1, k0, k1;
     float tx, ty, tz;
     bracket32(s.i, o[0], G.nx, true, i0, i1, tx);
     bracket32(s.j, o[1], G.ny, G.geometry == 0, j0, j1, ty);
     bracket32(s.k, o[2], G.nz, false, k0, k1, tz);
+    const float ux = 1.0f - tx, uy = 1.0f - ty, uz = 1.0f - tz;
+    Corners32 c;
+    c.base = (j0 * G.nx + i0) * G.nz + k0;
+    c.ox = (i1 - i0) * G.nz;
+    c.oy = (j1 - j0) * G.nx * G.nz;
+    c.oz = k1 - k0;
+    c.w[0] = ux * uy * uz;
+    c.w[1] = ux * uy * tz;
+    c.w[2] = tx * uy * uz;
+    c.w[3] = tx * uy * tz;
+    c.w[4] = ux * ty * uz;
+    c.w[5] = ux * ty * tz;
+    c.w[6] = tx * ty * uz;
+    c.w[7] = tx * ty * tz;
+    return c;
+}
+
+__device__ __forceinline__ void gather32(const Grid& G, const Node32* __restrict__ bg, const S32& s, const float o[3],
+                                         Bg32& b)
+{
+    const Corners32 c = corners32(G, s, o);
     float acc[16];
 #pragma unroll
     for (int q = 0; q < 16; ++q) acc[q] = 0.0f;
-    const float ux = 1.0f - tx, uy = 1.0f - ty, uz = 1.0f - tz;
-    const int dk = k1 - k0;
-    const Node32* c00 = bg + node_index(G, i0, j0, k0);
-    const Node32* c10 = bg + node_index(G, i1, j0, k0);
-    const Node32* c01 = bg + node_index(G, i0, j1, k0);
-    const Node32* c11 = bg + node_index(G, i1, j1, k0);
-    accumulate32<kWide>(c00, ux * uy * uz, acc);
-    accumulate32<kWide>(c00 + dk, ux * uy * tz, acc);
-    accumulate32<kWide>(c10, tx * uy * uz, acc);
-    accumulate32<kWide>(c10 + dk, tx * uy * tz, acc);
-    accumulate32<kWide>(c01, ux * ty * uz, acc);
-    accumulate32<kWide>(c01 + dk, ux * ty * tz, acc);
-    accumulate32<kWide>(c11, tx * ty * uz, acc);
-    accumulate32<kWide>(c11 + dk, tx * ty * tz, acc);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const float4* p = reinterpret_cast<const float4*>(bg + c.node(q));
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float4 a = __ldg(p + e);
+            acc[4 * e] = fmaf(c.w[q], a.x, acc[4 * e]);
+            acc[4 * e + 1] = fmaf(c.w[q], a.y, acc[4 * e + 1]);
+            acc[4 * e + 2] = fmaf(c.w[q], a.z, acc[4 * e + 2]);
+            acc[4 * e + 3] = fmaf(c.w[q], a.w, acc[4 * e + 3]);
+        }
+    }
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
         b.v[f] = acc[f];
 #pragma unroll
         for (int q = 0; q < 3; ++q) b.d[f][q] = acc[4 + 3 * f + q];
     }
+}
+
+// The same sums for a warp's 32 rays by four lanes a node: lane l loads the (l & 3)-th 16 bytes of the
+// nodes of rays 8 j + (l >> 2), j = 0 .. 3, so every load covers whole 64-byte nodes, and sums that
+// element for these four rays (the same additions in the same order).  With a ray a lane every load
+// touched a line per lane where the rays of a warp sit at different levels, and the ray step was bound
+// by them.  Weights and node indices pass to the four lanes through the ray's row of shared memory, the
+// sums come back in it (kRow32 floats: 64 bytes and a pad against bank conflicts).  All 32 lanes must
+// call it; `first` is the first node of the ray's ensemble member.
+constexpr int kRow32 = 20;
+
+__device__ __forceinline__ void gather32_warp(const Grid& G, const Node32* __restrict__ bg, int first, const S32& s,
+                                              const float o[3], float* rows, Bg32& b)
+{
+    const int lane = threadIdx.x & 31;
+    {
+        const Corners32 c = corners32(G, s, o);
+        float* row = rows + lane * kRow32;
+        *reinterpret_cast<float4*>(row) = make_float4(c.w[0], c.w[1], c.w[2], c.w[3]);
+        *reinterpret_cast<float4*>(row + 4) = make_float4(c.w[4], c.w[5], c.w[6], c.w[7]);
+        *reinterpret_cast<int4*>(row + 8) = make_int4(first + c.base, c.ox, c.oy, c.oz);
+    }
+    __syncwarp();
+    const float4* __restrict__ el = reinterpret_cast<const float4*>(bg) + (lane & 3);
+    float4 sum[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float* row = rows + (8 * j + (lane >> 2)) * kRow32;
+        const int4 n = *reinterpret_cast<const int4*>(row + 8);
+        const float4 wa = *reinterpret_cast<const float4*>(row), wb = *reinterpret_cast<const float4*>(row + 4);
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+        float4 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            v[q] = __ldg(el + 4 * (int64_t)(n.x + ((q & 2) ? n.y : 0) + ((q & 4) ? n.z : 0) + ((q & 1) ? n.w : 0)));
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            a.x = fmaf(w[q], v[q].x, a.x);
+            a.y = fmaf(w[q], v[q].y, a.y);
+            a.z = fmaf(w[q], v[q].z, a.z);
+            a.w = fmaf(w[q], v[q].w, a.w);
+        }
+        sum[j] = a;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        *reinterpret_cast<float4*>(rows + (8 * j + (lane >> 2)) * kRow32 + 4 * (lane & 3)) = sum[j];
+    __syncwarp();
+    float acc[16];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float4 a = *reinterpret_cast<const float4*>(rows + lane * kRow32 + 4 * e);
+        acc[4 * e] = a.x;
+        acc[4 * e + 1] = a.y;
+        acc[4 * e + 2] = a.z;
+        acc[4 * e + 3] = a.w;
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        b.v[f] = acc[f];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) b.d[f][q] = acc[4 + 3 * f + q];
+    }
+    __syncwarp();
 }
 
 // ------------------------------------------------------------------------------ geometry, dispersion
@@ -202,13 +261,14 @@ __device__ __forceinline__ void dispersion32(float kh2, float mg2, float n2, flo
 
 // ------------------------------------------------------------------------------ ray equations
 
-// y = (ox, oy, oz in cell units relative to the base cell, k, l, m, eX, eY, eZ); F the rates
-__device__ __forceinline__ void rhs32(const Grid& G, const Node32* __restrict__ bg, const S32& s, const float y[9],
-                                      float F[9])
+// y = (ox, oy, oz in cell units relative to the base cell, k, l, m, eX, eY, eZ); F the rates.  All 32
+// lanes of a warp must call it (gather32_warp: first, rows).
+__device__ __forceinline__ void rhs32(const Grid& G, const Node32* __restrict__ bg, int first, const S32& s,
+                                      const float y[9], float* rows, float F[9])
 {
     const float k = y[3], l = y[4], m = y[5];
     Bg32 b;
-    gather32<true>(G, bg, s, y, b);
+    gather32_warp(G, bg, first, s, y, rows, b);
     Geo32 g;
     geo32(G, s, y, g);
     float f2, df2;
@@ -274,7 +334,8 @@ __device__ __forceinline__ void rhs32(const Grid& G, const Node32* __restrict__ 
     }
 }
 
-__device__ __forceinline__ void rk3_32(const Grid& G, const Node32* __restrict__ bg, S32& s, float dt)
+__device__ __forceinline__ void rk3_32(const Grid& G, const Node32* __restrict__ bg, int first, S32& s, float dt,
+                                       float* rows)
 {
     float y[9] = {s.o[0], s.o[1], s.o[2], s.w[0], s.w[1], s.w[2], s.e[0], s.e[1], s.e[2]};
     float q[9];
@@ -283,7 +344,7 @@ __device__ __forceinline__ void rk3_32(const Grid& G, const Node32* __restrict__
 #pragma unroll 1
     for (int st = 0; st < 3; ++st) {
         float F[9];
-        rhs32(G, bg, s, y, F);
+        rhs32(G, bg, first, s, y, rows, F);
         // the stage's coefficients selected, not indexed (an array indexed by the rolled stage
         // counter would live in local memory, whose loads share L1 with the gathers)
         const float a = st == 0 ? 0.0f : (st == 1 ? -5.0f / 9.0f : -153.0f / 128.0f);
