@@ -118,7 +118,7 @@ __device__ __forceinline__ float gelu_grad(float z)
 // pre-activations of EPI_BWD.
 template <int MODE>
 __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, float (&v)[32], const float* sbias,
-                                      float ps, float pm, const float (&zz)[32], int rowmask, double& sq,
+                                      float ps, float pm, const float (&zz)[32], int rowmask, gwam::DF& sq,
                                       uint32_t stg, int cc0)
 {
     const bool live = row < e.M;
@@ -175,15 +175,38 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
             }
         } else {  // EPI_LOSS
             if (e.cf) {
+                float* p = e.cf + (size_t)row * e.ldcf + nb;
+                if (full && (e.ldcf & 3) == 0) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (nb + j < e.N) e.cf[(size_t)row * e.ldcf + nb + j] = v[j];
+                    for (int q = 0; q < 8; ++q)
+                        reinterpret_cast<float4*>(p)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (nb + j < e.N) p[j] = v[j];
+                }
             }
-            const float* tp = e.tgt + (size_t)row * e.ldt + nb;
+            const float* tg = e.tgt + (size_t)row * e.ldt + nb;
+            float tp[32];
+            if (full && (e.ldt & 3) == 0) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const float4 t4 = reinterpret_cast<const float4*>(tg)[q];
+                    tp[4 * q] = t4.x;
+                    tp[4 * q + 1] = t4.y;
+                    tp[4 * q + 2] = t4.z;
+                    tp[4 * q + 3] = t4.w;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) tp[j] = nb + j < e.n_true ? tg[j] : 0.0f;
+            }
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
+                // the squares (exact products) summed in double-float: FP64 additions and conversions
+                // had made this kernel 55 us
                 const float d = nb + j < e.n_true ? v[j] - tp[j] : 0.0f;
-                sq += (double)d * (double)d;
+                sq = gwam::df_add(sq, gwam::df_prod(d, d));
                 v[j] = e.gscale * d;
             }
         }
@@ -240,6 +263,32 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
         for (int j = 0; j < 32; ++j)
             if (nb + j < e.N) e.ct[(size_t)(nb + j) * e.ldct + row] = __float2bfloat16_rn(v[j]);
     }
+}
+
+// 32 accumulator columns of this warp's 32 TMEM lanes, one row a lane
+__device__ __forceinline__ void tmem_ld32(uint32_t addr, uint32_t (&rr)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(rr[0]), "=r"(rr[1]), "=r"(rr[2]), "=r"(rr[3]), "=r"(rr[4]), "=r"(rr[5]), "=r"(rr[6]), "=r"(rr[7]),
+          "=r"(rr[8]), "=r"(rr[9]), "=r"(rr[10]), "=r"(rr[11]), "=r"(rr[12]), "=r"(rr[13]), "=r"(rr[14]), "=r"(rr[15]),
+          "=r"(rr[16]), "=r"(rr[17]), "=r"(rr[18]), "=r"(rr[19]), "=r"(rr[20]), "=r"(rr[21]), "=r"(rr[22]),
+          "=r"(rr[23]), "=r"(rr[24]), "=r"(rr[25]), "=r"(rr[26]), "=r"(rr[27]), "=r"(rr[28]), "=r"(rr[29]),
+          "=r"(rr[30]), "=r"(rr[31])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// 16 columns likewise
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&rr)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(rr[0]), "=r"(rr[1]), "=r"(rr[2]), "=r"(rr[3]), "=r"(rr[4]), "=r"(rr[5]), "=r"(rr[6]), "=r"(rr[7]),
+          "=r"(rr[8]), "=r"(rr[9]), "=r"(rr[10]), "=r"(rr[11]), "=r"(rr[12]), "=r"(rr[13]), "=r"(rr[14]), "=r"(rr[15])
+        : "r"(addr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // Persistent, warp-specialised GEMM.  Warp 0 (one lane) streams the K blocks of every tile the
@@ -311,7 +360,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     const uint32_t tmem = tmem_slot;
     const unsigned long long wlim = e.wait_ns ? e.wait_ns : kWaitNs;
     bool ok = true;
-    double sq = 0.0;
+    DF sq{0.0f, 0.0f};
 
     if (warp == 0) {
         if (lane == 0) {
@@ -467,16 +516,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
                     for (int j = 0; j < 32; ++j) zz[j] = 0.0f;
                 }
                 uint32_t rr[32];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                    "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                    : "=r"(rr[0]), "=r"(rr[1]), "=r"(rr[2]), "=r"(rr[3]), "=r"(rr[4]), "=r"(rr[5]), "=r"(rr[6]),
-                      "=r"(rr[7]), "=r"(rr[8]), "=r"(rr[9]), "=r"(rr[10]), "=r"(rr[11]), "=r"(rr[12]), "=r"(rr[13]),
-                      "=r"(rr[14]), "=r"(rr[15]), "=r"(rr[16]), "=r"(rr[17]), "=r"(rr[18]), "=r"(rr[19]), "=r"(rr[20]),
-                      "=r"(rr[21]), "=r"(rr[22]), "=r"(rr[23]), "=r"(rr[24]), "=r"(rr[25]), "=r"(rr[26]), "=r"(rr[27]),
-                      "=r"(rr[28]), "=r"(rr[29]), "=r"(rr[30]), "=r"(rr[31])
-                    : "r"(tacc + (uint32_t)(32 * k)));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tmem_ld32(tacc + (uint32_t)(32 * k), rr);
                 float v[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rr[j]);
@@ -518,9 +558,10 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
         __syncwarp();
         if (!ok) abort_flag = 1;
         if (MODE == EPI_LOSS) {
+            double sum = df_to_double(sq);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            if (lane == 0 && sq != 0.0) atomicAdd(e.loss, sq);
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0 && sum != 0.0) atomicAdd(e.loss, sum);
         }
     }
     // every MMA has finished before the TMEM is released (bounded wait; immediate normally)
@@ -530,12 +571,262 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
-int sm_count()
+// Weight gradients and weight updates of all layers (GradSet), the roles of the warps as in k_gemm_bf16:
+// warp 0 streams K blocks, warp 1 issues the MMAs of slice after slice into kGradAcc accumulators by turns,
+// the epilogue warps (a row a lane, kGradCols columns each) add each slice to FP32 registers in order
+// and, after the last, run Adam on the tile.  Sixteen of them: Adam's divisions and square root are IEEE
+// ones, about 100 instructions an element, which four warps took 23 us for.  The slices define the order of the sum (deterministic); adding them
+// here instead of writing each to memory and summing them in another kernel (up to 64 slices, 33 MB
+// per 512 x 512 layer) leaves one pass over the weights.
+constexpr int kGradStages = 7;
+constexpr uint32_t kGradStage = kABytes + kGradBN * kBK * 2;
+constexpr int kGradPitch = kGradBN + 4;   // floats a row of the update's tile
+constexpr int kGradEpi = 16;              // epilogue warps
+constexpr int kGradAcc = 4;               // accumulators (slices in flight to the epilogue)
+constexpr int kGradCols = kGradBN / (kGradEpi / 4);
+static_assert(kGradCols == 16, "an epilogue warp reads 16 columns at a time");
+__global__ void __launch_bounds__(64 + 32 * kGradEpi, 1) k_grad_update(const __grid_constant__ GradSet G, int K, int* err)
 {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    return n > 0 ? n : 1;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kGradStages], empty_bar[kGradStages], accf_bar[kGradAcc], acce_bar[kGradAcc], done_bar;
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+    constexpr uint32_t kCols = kGradAcc * kGradBN;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t base = (saddr(smem_raw) + 1023u) & ~1023u;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr(&tmem_slot)),
+                     "r"(kCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < kGradStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&full_bar[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&empty_bar[s])));
+        }
+        for (int a = 0; a < kGradAcc; ++a) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&accf_bar[a])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(&acce_bar[a])), "r"(kGradEpi));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&done_bar)));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        abort_flag = 0;
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    tc_before();
+    __syncthreads();
+    tc_after();
+    const uint32_t tmem = tmem_slot;
+    const int total = G.end[G.n - 1], kb = K / kBK;
+    float* const tile = reinterpret_cast<float*>(smem_raw + (base - saddr(smem_raw)) + kGradStages * kGradStage);
+    auto epi_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(32 * kGradEpi) : "memory"); };   // the epilogue warps
+    bool ok = true;
+    // job, corner and K blocks a slice of tile t
+    auto decode = [&](int t, int& j, int& m0, int& n0) {
+        j = 0;
+        while (t >= G.end[j]) ++j;
+        t -= j ? G.end[j - 1] : 0;
+        const int nx = G.N[j] / kGradBN;
+        m0 = (t / nx) * kBM;
+        n0 = (t % nx) * kGradBN;
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+                int j, m0, n0;
+                decode(t, j, m0, n0);
+                for (int i = 0; i < kb; ++i, ++it) {
+                    const int s = it % kGradStages;
+                    if ((it >= kGradStages &&
+                         !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((it / kGradStages - 1) & 1), kWaitNs)) ||
+                        abort_flag) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t fb = saddr(&full_bar[s]);
+                    const uint32_t dA = base + (uint32_t)s * kGradStage, dB = dA + kABytes;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(kGradStage)
+                                 : "memory");
+                    asm volatile(
+                        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
+                        "{%2, %3}], [%4];" ::"r"(dA),
+                        "l"(reinterpret_cast<uint64_t>(&G.ta[j])), "r"(i * kBK), "r"(m0), "r"(fb)
+                        : "memory");
+                    asm volatile(
+                        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, "
+                        "{%2, %3}], [%4];" ::"r"(dB),
+                        "l"(reinterpret_cast<uint64_t>(&G.tb[j])), "r"(i * kBK), "r"(n0), "r"(fb)
+                        : "memory");
+                }
+            }
+            if (!ok) abort_flag = 1;
+            // every issued copy has landed before the CTA may exit (immediate in the normal case)
+            for (int i = it > kGradStages ? it - kGradStages : 0; i < it; ++i)
+                if (!mbar_wait(saddr(&full_bar[i % kGradStages]), (uint32_t)((i / kGradStages) & 1), kWaitNs)) ok = false;
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = idesc_bf16(kBM, kGradBN);
+            int it = 0, sl = 0;   // K blocks and slices so far
+            for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+                int j, m0, n0;
+                decode(t, j, m0, n0);
+                const int nk = kb / G.S[j];
+                for (int z = 0; z < G.S[j] && ok; ++z, ++sl) {
+                    const int acc = sl % kGradAcc;
+                    if (sl >= kGradAcc &&
+                        !mbar_wait(saddr(&acce_bar[acc]), (uint32_t)((sl / kGradAcc - 1) & 1), kWaitNs)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_after();
+                    for (int i = 0; i < nk; ++i, ++it) {
+                        const int s = it % kGradStages;
+                        if (abort_flag || !mbar_wait(saddr(&full_bar[s]), (uint32_t)((it / kGradStages) & 1), kWaitNs)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_after();
+                        const uint32_t a0 = base + (uint32_t)s * kGradStage, b0 = a0 + kABytes;
+#pragma unroll
+                        for (int kk = 0; kk < kBK / 16; ++kk) {
+                            const uint64_t ad = desc_sw128(a0 + 32u * kk), bd = desc_sw128(b0 + 32u * kk);
+                            const uint32_t accum = (i > 0 || kk > 0) ? 1u : 0u;
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(
+                                    tmem + (uint32_t)(acc * kGradBN)),
+                                "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
+                                : "memory");
+                        }
+                        asm volatile(
+                            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                saddr(&empty_bar[s]))
+                            : "memory");
+                    }
+                    if (!ok) break;
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     saddr(&accf_bar[acc]))
+                                 : "memory");
+                }
+            }
+            if (!ok) abort_flag = 1;
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             saddr(&done_bar))
+                         : "memory");
+        }
+        __syncwarp();
+    } else {
+        const int q = warp & 3, part = (warp - 2) >> 2;
+        const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(part * kGradCols);
+        int sl = 0;
+        for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+            int j, m0, n0;
+            decode(t, j, m0, n0);
+            __syncwarp();
+            float g[kGradCols];
+#pragma unroll
+            for (int c = 0; c < kGradCols; ++c) g[c] = 0.0f;
+#pragma unroll 1
+            for (int z = 0; z < G.S[j]; ++z, ++sl) {
+                const int acc = sl % kGradAcc;
+                const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((sl / kGradAcc) & 1), kWaitNs);
+                if (!__all_sync(0xffffffffu, got) || abort_flag) {
+                    ok = false;
+                    break;
+                }
+                tc_after();
+                uint32_t rr[16];
+                tmem_ld16(tacc + (uint32_t)(acc * kGradBN), rr);
+#pragma unroll
+                for (int c = 0; c < kGradCols; ++c) g[c] += __uint_as_float(rr[c]);
+                tc_before();
+                __syncwarp();
+                // one arrival a warp (512 of them a slice took as long as its MMAs)
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&acce_bar[acc])) : "memory");
+            }
+            // the epilogue warps go on together or give up together (the barriers below would wait for
+            // a warp that had left)
+            uint32_t all;
+            asm volatile(
+                "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n barrier.cta.red.and.pred p, 1, %2, q;\n"
+                " selp.u32 %0, 1, 0, p;\n}"
+                : "=r"(all)
+                : "r"((uint32_t)ok), "n"(32 * kGradEpi)
+                : "memory");
+            ok = all != 0;
+            if (!ok) break;
+            // the tile's gradients through shared memory, so that the update reads and writes whole rows
+            // (a row a lane, every access touched 32 lines and waited for the one before: 40 us)
+            const int Mj = G.M[j], Di = G.N[j], no = G.n_o[j], ni = G.n_i[j];
+            float* const mine = tile + (q * 32 + lane) * kGradPitch + part * kGradCols;
+#pragma unroll
+            for (int c = 0; c < kGradCols; c += 4)
+                *reinterpret_cast<float4*>(mine + c) = make_float4(g[c], g[c + 1], g[c + 2], g[c + 3]);
+            epi_sync();
+            const bool upd = G.adam.lr > 0.0f;
+            const int et = tid - 64, c0 = (et & 15) * 4;   // 16 threads a row
+#pragma unroll 4
+            for (int r = et >> 4; r < kBM; r += 2 * kGradEpi) {
+                const int o = m0 + r;
+                if (o >= Mj) break;
+                float4* const gp = reinterpret_cast<float4*>(tile + r * kGradPitch + c0);
+                const float4 g4 = *gp;
+                const size_t at = (size_t)o * Di + n0 + c0;
+                float gg[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (o >= no || n0 + c0 + u >= ni) gg[u] = 0.0f;
+                *reinterpret_cast<float4*>(G.g[j] + at) = make_float4(gg[0], gg[1], gg[2], gg[3]);
+                if (!upd || o >= no) {
+                    *gp = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    continue;
+                }
+                const float4 w4 = *reinterpret_cast<const float4*>(G.W[j] + at);
+                const float4 m4 = *reinterpret_cast<const float4*>(G.m[j] + at);
+                const float4 v4 = *reinterpret_cast<const float4*>(G.v[j] + at);
+                float w[4] = {w4.x, w4.y, w4.z, w4.w}, mm[4] = {m4.x, m4.y, m4.z, m4.w}, vv[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (n0 + c0 + u < ni) w[u] = G.adam(w[u], gg[u], mm[u], vv[u]);
+                const float4 wn = make_float4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<float4*>(G.W[j] + at) = wn;
+                *reinterpret_cast<float4*>(G.m[j] + at) = make_float4(mm[0], mm[1], mm[2], mm[3]);
+                *reinterpret_cast<float4*>(G.v[j] + at) = make_float4(vv[0], vv[1], vv[2], vv[3]);
+                const __nv_bfloat162 h0 = __floats2bfloat162_rn(w[0], w[1]), h1 = __floats2bfloat162_rn(w[2], w[3]);
+                *reinterpret_cast<uint2*>(G.Wb[j] + at) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+                *gp = wn;
+            }
+            epi_sync();
+            if (upd) {
+                // the transposed copy: four rows a lane, a column a warp and pass
+                const int r = 4 * lane;
+                if (m0 + r < Mj) {
+#pragma unroll 4
+                    for (int c = warp - 2; c < kGradBN; c += kGradEpi) {
+                        const float* col = tile + r * kGradPitch + c;
+                        const __nv_bfloat162 h0 = __floats2bfloat162_rn(col[0], col[kGradPitch]);
+                        const __nv_bfloat162 h1 = __floats2bfloat162_rn(col[2 * kGradPitch], col[3 * kGradPitch]);
+                        *reinterpret_cast<uint2*>(G.WbT[j] + (size_t)(n0 + c) * Mj + m0 + r) =
+                            make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+                    }
+                }
+            }
+            epi_sync();   // the tile is free for the next one
+        }
+        if (!ok) abort_flag = 1;
+    }
+    // every MMA has finished before the TMEM is released (bounded wait; immediate normally)
+    const bool fin = mbar_wait(saddr(&done_bar), 0u, kWaitNs);
+    if (!__syncthreads_and(ok && fin) && tid == 0 && err) atomicOr(err, 1);
+    tc_after();
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
 template <int BN, int ST, int EPW, int MODE>
@@ -553,16 +844,13 @@ bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap
     // dynamic shared memory limit raised per device to the largest size launched so far (the
     // opt-in limit counts the kernel's static shared memory too)
     static size_t configured[64] = {};
-    static int sms[64] = {};
     if (shm > configured[dev]) {
-        if (cudaFuncSetAttribute(k_gemm_bf16<BN, ST, EPW, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) !=
-            cudaSuccess)
+        if (cudaFuncSetAttribute(k_gemm_bf16<BN, ST, EPW, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess)
             return false;
         configured[dev] = shm;
-        sms[dev] = sm_count();
     }
     const long long tiles = (long long)((e.N + BN - 1) / BN) * ((e.M + kBM - 1) / kBM) * ksplit;
-    const int grid = (int)std::min<long long>(tiles, sms[dev]);
+    const int grid = (int)std::min<long long>(tiles, gemm_sm_count());
     // launched with programmatic stream serialisation: the set-up of this GEMM (barriers, tensor
     // memory) overlaps the tail of the kernel before it, which it waits for before its first read
     cudaLaunchConfig_t cfg = {};
@@ -624,13 +912,66 @@ bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t 
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int gemm_sm_count()
+{
+    static int sms[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 1;
+    if (!sms[dev]) {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        sms[dev] = n > 0 ? n : 1;
+    }
+    return sms[dev];
+}
+
 int gemm_pick_bn(int M, int N)
 {
-    (void)M;
-    if (N <= 64) return 64;
-    if (N <= 128) return 128;
-    if (N <= 192) return 192;
-    return 256;
+    const int sms = gemm_sm_count();
+    int best = 256;
+    long long cost = -1;
+    for (int bn : {256, 192, 128, 64}) {
+        const long long tiles = (long long)((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
+        const long long c = (tiles + sms - 1) / sms * (bn + 48);
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = bn;
+        }
+    }
+    return best;
+}
+
+bool gemm_bf16_grad_launch(GradSet& g, int K, int* err, cudaStream_t s)
+{
+    if (g.n < 1 || g.n > kGradMax || K < kBK || K % kBK) return false;
+    int tiles = 0;
+    for (int j = 0; j < g.n; ++j) {
+        if (g.M[j] < 64 || g.M[j] % 64 || g.N[j] < 64 || g.N[j] % 64 || g.S[j] < 1 || (K / kBK) % g.S[j]) return false;
+        tiles += ((g.M[j] + kBM - 1) / kBM) * (g.N[j] / kGradBN);
+        g.end[j] = tiles;
+    }
+    constexpr size_t shm = kGradStages * kGradStage + 1024 + kBM * kGradPitch * sizeof(float);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 64) return false;
+    static bool configured[64] = {};
+    if (!configured[dev]) {
+        if (cudaFuncSetAttribute(k_grad_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess)
+            return false;
+        configured[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min(tiles, gemm_sm_count()));
+    cfg.blockDim = dim3(64 + 32 * kGradEpi);
+    cfg.dynamicSmemBytes = shm;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_grad_update, g, K, err) == cudaSuccess;
 }
 
 bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ksplit,

@@ -66,6 +66,36 @@ struct GemmEpi {
 bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
                     uint32_t box_rows);
 
+// One Adam update (Kingma & Ba 2015) of a parameter w with gradient g; returns the new value
+struct Adam {
+    float lr, b1, b2, eps, c1, c2;   // lr = 0: gradients only
+    __device__ __forceinline__ float operator()(float w, float g, float& m, float& v) const
+    {
+        const float mm = __fmaf_rn(1.0f - b1, g, __fmul_rn(b1, m));
+        const float vv = __fmaf_rn(__fmul_rn(1.0f - b2, g), g, __fmul_rn(b2, v));
+        m = mm;
+        v = vv;
+        return w - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
+    }
+};
+
+// The weight gradients and weight updates of all layers as one launch: job j forms dW_j[M_j, N_j] =
+// A_j . B_j^T over the batch (K), in S_j slices along K whose sums are added in order (K / 64 divisible by
+// S_j), stores it to g and updates W, m, v and the BF16 copies (row-major and transposed).  M_j, N_j
+// multiples of 64; entries outside [n_o][n_i] stay zero.
+constexpr int kGradMax = 8;
+constexpr int kGradBN = 64;
+struct GradSet {
+    CUtensorMap ta[kGradMax], tb[kGradMax];   // box rows 128 and kGradBN
+    float *g[kGradMax], *W[kGradMax], *m[kGradMax], *v[kGradMax];
+    __nv_bfloat16 *Wb[kGradMax], *WbT[kGradMax];
+    int M[kGradMax], N[kGradMax], n_o[kGradMax], n_i[kGradMax], S[kGradMax];
+    int end[kGradMax];                        // tiles of jobs 0 .. j (filled in by the launch)
+    int n;
+    Adam adam;
+};
+bool gemm_bf16_grad_launch(GradSet& set, int K, int* err, cudaStream_t s);
+
 // Launch: A described by ta (box rows 128), B by tb (box rows bn); K a multiple of 64, split into
 // ksplit slices along K (K / 64 must be divisible by ksplit).  tc (or null): tensor map of the BF16
 // output cb (box 64 columns x 32 rows) -- the epilogue then stages each warp's rows in shared memory
@@ -74,7 +104,12 @@ bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t 
 bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ksplit,
                       const GemmEpi& e, cudaStream_t s);
 
-// The tile width gemm_bf16_launch uses for N when bn = 0 (the caller builds tb with this box).
+// The tile width gemm_bf16_launch uses when bn = 0 (the caller builds tb with this box): the one with
+// the least waves x (width + 48) over the GPU's SMs -- a tile's time grows with its width, 48 columns
+// stand for its fixed part.  Wide tiles for large M (32 768 x 512: 256), narrow ones where wide ones
+// would leave SMs idle (4096 x 512: 128 instead of 64 tiles of 256; 1000 x 512: 64).
 int gemm_pick_bn(int M, int N);
+// compute units of the current device
+int gemm_sm_count();
 
 }  // namespace gwam

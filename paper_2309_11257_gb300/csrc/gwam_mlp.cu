@@ -9,8 +9,8 @@
 //   activations  act_l [B][D_l] BF16 (l = 0 the normalised input), actT_l [D_l][B] BF16 (operand of
 //                the weight-gradient GEMM), Z_l [B][D_l] FP32 pre-activations, dz_l / dzT_l the
 //                BF16 gradients of Z_l in both layouts.
-//   gradients    dW_l by split-K GEMM into FP32 partial slices, summed in a fixed order by the Adam
-//                kernel (deterministic), db_l by row sums of dzT_l.
+//   gradients    dW_l as sums of K slices added in a fixed order (deterministic), each layer's update in
+//                the same kernel (k_grad_update); db_l by row sums of dzT_l.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
@@ -41,106 +41,115 @@ __device__ __forceinline__ int64_t batch_row(const int32_t* rows, uint64_t seed,
     return (int64_t)(splitmix64(seed + (uint64_t)(r + 1) * 0x9E3779B97F4A7C15ull) % (uint64_t)n);
 }
 
-// normalised, zero-padded input batch in both layouts: Xb [B][D0], XT [D0][ldT]
-__global__ void k_batch_inputs(const float* __restrict__ X, int64_t n, int n_in, int D0, const int32_t* rows,
-                               uint64_t seed, const float* __restrict__ mu, const float* __restrict__ isig,
-                               __nv_bfloat16* Xb, __nv_bfloat16* XT, int ldT, int* err)
+// programmatic dependent launch: let the next kernel set up, wait for the previous one to complete
+__device__ __forceinline__ void pdl_enter()
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// The batch, 32 rows x 32 columns a block: normalised, zero-padded inputs in both layouts, Xb [B][D0] and
+// XT [D0][ldT] (blocks x < D0 / 32), and normalised, zero-padded targets T [B][Dn] (the others).  The
+// drawn rows are found once per block (a 64-bit remainder each).
+__global__ void k_batch(const float* __restrict__ X, const float* __restrict__ Y, int64_t n, int n_in, int D0,
+                        int n_out, int Dn, const int32_t* rows, uint64_t seed, const float* __restrict__ mu,
+                        const float* __restrict__ isig, const float* __restrict__ ymu, const float* __restrict__ yisig,
+                        __nv_bfloat16* Xb, __nv_bfloat16* XT, int ldT, float* T, int* err)
+{
+    pdl_enter();
     __shared__ __nv_bfloat16 tile[32][33];
-    const int f0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    __shared__ int64_t src[32];
+    const int r0 = blockIdx.y * 32;
     const int tx = threadIdx.x, ty = threadIdx.y;
-    for (int rr = ty; rr < 32; rr += 8) {
-        const int r = r0 + rr, f = f0 + tx;
-        const int64_t src = batch_row(rows, seed, n, r);
-        float xn = 0.0f;
-        if (src < 0 || src >= n) {
-            if (tx == 0) atomicOr(err, 2);
-        } else if (f < n_in) {
-            xn = (X[src * n_in + f] - mu[f]) * isig[f];
+    if (ty == 0) {
+        const int64_t q = batch_row(rows, seed, n, r0 + tx);
+        src[tx] = q;
+        if (q < 0 || q >= n) atomicOr(err, 2);
+    }
+    __syncthreads();
+    const int xb = D0 / 32;
+    if ((int)blockIdx.x >= xb) {
+        const int o = (blockIdx.x - xb) * 32 + tx;
+        for (int rr = ty; rr < 32; rr += 8) {
+            const int64_t q = src[rr];
+            T[(size_t)(r0 + rr) * Dn + o] = (o < n_out && q >= 0 && q < n) ? (Y[q * n_out + o] - ymu[o]) * yisig[o] : 0.0f;
         }
+        return;
+    }
+    const int f0 = blockIdx.x * 32, f = f0 + tx;
+    for (int rr = ty; rr < 32; rr += 8) {
+        const int64_t q = src[rr];
+        const float xn = (f < n_in && q >= 0 && q < n) ? (X[q * n_in + f] - mu[f]) * isig[f] : 0.0f;
         const __nv_bfloat16 h = __float2bfloat16_rn(xn);
-        if (f < D0) Xb[(size_t)r * D0 + f] = h;
+        Xb[(size_t)(r0 + rr) * D0 + f] = h;
         tile[rr][tx] = h;
     }
     __syncthreads();
-    for (int ff = ty; ff < 32; ff += 8) {
-        const int f = f0 + ff;
-        if (f < D0) XT[(size_t)f * ldT + r0 + tx] = tile[tx][ff];
-    }
+    for (int ff = ty; ff < 32; ff += 8) XT[(size_t)(f0 + ff) * ldT + r0 + tx] = tile[tx][ff];
 }
 
-// normalised, zero-padded targets T [B][Dn]
-__global__ void k_batch_targets(const float* __restrict__ Y, int64_t n, int n_out, int Dn, int B, const int32_t* rows,
-                                uint64_t seed, const float* __restrict__ mu, const float* __restrict__ isig,
-                                float* T)
-{
-    const int r = blockIdx.x;
-    if (r >= B) return;
-    const int64_t src = batch_row(rows, seed, n, r);
-    const bool okrow = src >= 0 && src < n;
-    for (int o = threadIdx.x; o < Dn; o += blockDim.x)
-        T[(size_t)r * Dn + o] = (o < n_out && okrow) ? (Y[src * n_out + o] - mu[o]) * isig[o] : 0.0f;
-}
+// The bias gradients of all layers and their updates, a warp per output: db = the sum of dzT's row over
+// the batch.  The FP32 sum keeps the order of a 256-thread block (thread t adds rows t, t + 256, ...,
+// then a tree over the threads): lane l stands for threads 8 l .. 8 l + 7, whose rows are one 16-byte
+// load.
+struct BiasSet {
+    const __nv_bfloat16* dzT[kMaxL];   // [D][ld]
+    float *gb[kMaxL], *b[kMaxL], *mb[kMaxL], *vb[kMaxL];
+    int n_o[kMaxL], end[kMaxL];        // end: outputs of layers 0 .. q
+    int nl, ld, B;
+    gwam::Adam adam;
+};
 
-// db[o] = sum over the batch of dzT[o][r] (FP32 sum of BF16 values in a fixed order)
-__global__ void k_rowsum(const __nv_bfloat16* __restrict__ dzT, int ld, int B, int D, float* db)
+__global__ void __launch_bounds__(256) k_bias_update(const __grid_constant__ BiasSet u)
 {
-    const int o = blockIdx.x;
-    if (o >= D) return;
-    float s = 0.0f;
-    for (int r = threadIdx.x; r < B; r += blockDim.x) s += __bfloat162float(dzT[(size_t)o * ld + r]);
-    __shared__ float red[256];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) db[o] = red[0];
-}
-
-// sum of the split-K partial slices (fixed order) -> g; Adam update of the master weights when
-// lr > 0, refreshing the BF16 copies in both layouts.  Entries outside [n_o][n_i] stay zero.
-__global__ void k_adam_weights(const float* __restrict__ part, int S, long long slice, int Do, int Di, int n_o,
-                               int n_i, float* g, float* W, float* m, float* v, __nv_bfloat16* Wb,
-                               __nv_bfloat16* WbT, float lr, float b1, float b2, float eps, float c1, float c2)
-{
-    const long long total = (long long)Do * Di;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int o = (int)(idx / Di), i = (int)(idx - (long long)o * Di);
-        float s = 0.0f;
-        for (int k = 0; k < S; ++k) s += part[k * slice + idx];
-        if (o >= n_o || i >= n_i) s = 0.0f;
-        g[idx] = s;
-        if (lr > 0.0f && o < n_o && i < n_i) {
-            const float mm = b1 * m[idx] + (1.0f - b1) * s;
-            const float vv = b2 * v[idx] + (1.0f - b2) * s * s;
-            m[idx] = mm;
-            v[idx] = vv;
-            const float w = W[idx] - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
-            W[idx] = w;
-            const __nv_bfloat16 h = __float2bfloat16_rn(w);
-            Wb[idx] = h;
-            WbT[(size_t)i * Do + o] = h;
+    pdl_enter();
+    const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (w >= u.end[u.nl - 1]) return;
+    int q = 0;
+    while (w >= u.end[q]) ++q;
+    const int o = w - (q ? u.end[q - 1] : 0);
+    const __nv_bfloat16* row = u.dzT[q] + (size_t)o * u.ld + 8 * lane;
+    float s[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) s[h] = 0.0f;
+#pragma unroll 4
+    for (int r = 0; r < u.B - 8 * lane; r += 256) {
+        const uint4 v = *reinterpret_cast<const uint4*>(row + r);
+        const uint32_t p[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            s[2 * h] += __uint_as_float(p[h] << 16);
+            s[2 * h + 1] += __uint_as_float(p[h] & 0xFFFF0000u);
         }
     }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+        for (int h = 0; h < 8; ++h) s[h] += __shfl_down_sync(0xffffffffu, s[h], d);
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1)
+#pragma unroll
+        for (int h = 0; h < d; ++h) s[h] += s[h + d];
+    if (lane != 0) return;
+    const float g = o < u.n_o[q] ? s[0] : 0.0f;
+    u.gb[q][o] = g;
+    if (u.adam.lr > 0.0f && o < u.n_o[q]) u.b[q][o] = u.adam(u.b[q][o], g, u.mb[q][o], u.vb[q][o]);
 }
 
-__global__ void k_adam_bias(const float* __restrict__ gsrc, int D, int n_o, float* g, float* b, float* m, float* v,
-                            float lr, float b1, float b2, float eps, float c1, float c2)
+// launch with programmatic stream serialisation (the kernel begins with pdl_enter)
+template <class... P, class... A>
+bool launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args)
 {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= D) return;
-    const float s = o < n_o ? gsrc[o] : 0.0f;
-    g[o] = s;
-    if (lr > 0.0f && o < n_o) {
-        const float mm = b1 * m[o] + (1.0f - b1) * s;
-        const float vv = b2 * v[o] + (1.0f - b2) * s * s;
-        m[o] = mm;
-        v[o] = vv;
-        b[o] = b[o] - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
-    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...) == cudaSuccess;
 }
 
 // inference input: one warp per column -- normalise, envelope test, BF16 row; mask = 1 (ray
@@ -150,6 +159,7 @@ __global__ void k_pack_infer(const float* __restrict__ X, int64_t ncol, int64_t 
                              const float* __restrict__ lo, const float* __restrict__ hi, __nv_bfloat16* Xb,
                              int32_t* mask, int32_t* nfb)
 {
+    pdl_enter();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= rows) return;
     const int64_t c = c0 + warp;
@@ -293,12 +303,11 @@ struct gwam_mlp {
     float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     long long t = 0;
     float *W[kMaxL + 1] = {}, *b[kMaxL + 1] = {}, *mW[kMaxL + 1] = {}, *vW[kMaxL + 1] = {}, *mb[kMaxL + 1] = {},
-          *vb[kMaxL + 1] = {}, *gW[kMaxL + 1] = {}, *gb[kMaxL + 1] = {}, *db_raw[kMaxL + 1] = {};
+          *vb[kMaxL + 1] = {}, *gW[kMaxL + 1] = {}, *gb[kMaxL + 1] = {};
     __nv_bfloat16 *Wb[kMaxL + 1] = {}, *WbT[kMaxL + 1] = {};
     __nv_bfloat16 *act[kMaxL + 1] = {}, *actT[kMaxL + 1] = {}, *dz[kMaxL + 1] = {}, *dzT[kMaxL + 1] = {};
     float* Z[kMaxL + 1] = {};
-    float *Y = nullptr, *T = nullptr, *partial = nullptr;
-    size_t partial_elems = 0;
+    float *Y = nullptr, *T = nullptr;
     float *xmu = nullptr, *xisig = nullptr, *ymu = nullptr, *yisig = nullptr, *ysig = nullptr, *lo = nullptr,
           *hi = nullptr;
     int* err = nullptr;
@@ -306,9 +315,9 @@ struct gwam_mlp {
     int32_t* nfb = nullptr;
     bool has_norm = false;
     int last_batch = 0;
-    CUtensorMap tf_a[kMaxL + 1], tf_b[kMaxL + 1], tx_a[kMaxL + 1], tx_b[kMaxL + 1], tw_a[kMaxL + 1], tw_b[kMaxL + 1];
-    CUtensorMap to_act[kMaxL + 1], to_dz[kMaxL + 1];   // BF16 outputs written by TMA stores
-    int bn_f[kMaxL + 1] = {}, bn_x[kMaxL + 1] = {}, bn_w[kMaxL + 1] = {};
+    CUtensorMap tf_a[kMaxL + 1], tx_a[kMaxL + 1], tw_a[kMaxL + 1], tw_b[kMaxL + 1];
+    CUtensorMap tf_b[kMaxL + 1][4], tx_b[kMaxL + 1][4];   // by tile width (64, 128, 192, 256)
+    CUtensorMap to_act[kMaxL + 1], to_dz[kMaxL + 1];      // BF16 outputs written by TMA stores
     std::vector<void*> allocs;
     std::string last_error;
     // inference timing: events before the pack kernel, before the first GEMM, after the last GEMM
@@ -365,11 +374,11 @@ bool dalloc(gwam_mlp* m, T** p, size_t elems)
     return true;
 }
 
-// split-K factor of the weight-gradient GEMM of layer l for a batch of B rows
+// K slices of the weight gradient of layer l for a batch of B rows: they fix the order of its sum
 int wgrad_split(const gwam_mlp* m, int l, int B)
 {
-    const int kb = B / 64;
-    const int tiles = ((m->D[l] + 127) / 128) * ((m->D[l - 1] + m->bn_w[l] - 1) / m->bn_w[l]);
+    const int kb = B / 64, Di = m->D[l - 1], bn = Di <= 64 ? 64 : (Di <= 128 ? 128 : (Di <= 192 ? 192 : 256));
+    const int tiles = ((m->D[l] + 127) / 128) * ((Di + bn - 1) / bn);
     int S = 1;
     while (S * 2 <= 64 && kb % (S * 2) == 0 && tiles * S * 2 <= 2 * 152) S *= 2;
     return S;
@@ -434,14 +443,16 @@ bool forward(gwam_mlp* m, int B, bool train, const gwam::GemmEpi& last)
             e.ct = m->actT[l];
             e.ldct = m->max_batch;
         }
-        if (!gemm(m, m->tf_a[l], m->tf_b[l], &m->to_act[l], m->D[l - 1], m->bn_f[l], 1, e)) return false;
+        const int bn = gwam::gemm_pick_bn(B, m->D[l]);
+        if (!gemm(m, m->tf_a[l], m->tf_b[l][bn / 64 - 1], &m->to_act[l], m->D[l - 1], bn, 1, e)) return false;
     }
     gwam::GemmEpi e = last;
     e.M = B;
     e.N = m->D[m->nl];
     e.bias = m->b[m->nl];
-    return gemm(m, m->tf_a[m->nl], m->tf_b[m->nl], e.cb ? &m->to_dz[m->nl] : nullptr, m->D[m->nl - 1],
-                m->bn_f[m->nl], 1, e);
+    const int bn = gwam::gemm_pick_bn(B, e.N);
+    return gemm(m, m->tf_a[m->nl], m->tf_b[m->nl][bn / 64 - 1], e.cb ? &m->to_dz[m->nl] : nullptr, m->D[m->nl - 1],
+                bn, 1, e);
 }
 
 }  // namespace
@@ -474,17 +485,12 @@ int gwam_mlp_create(gwam_mlp** out, const gwam_mlp_config* cfg, void* stream)
     const int Bm = m->max_batch;
     bool ok = true;
     for (int l = 1; l <= m->nl && ok; ++l) {
-        m->bn_f[l] = gwam::gemm_pick_bn(Bm, m->D[l]);
-        m->bn_x[l] = gwam::gemm_pick_bn(Bm, m->D[l - 1]);
-        m->bn_w[l] = gwam::gemm_pick_bn(m->D[l], m->D[l - 1]);
         const size_t nw = (size_t)m->D[l] * m->D[l - 1];
         ok = ok && dalloc(m, &m->W[l], nw) && dalloc(m, &m->mW[l], nw) && dalloc(m, &m->vW[l], nw) &&
              dalloc(m, &m->gW[l], nw) && dalloc(m, &m->Wb[l], nw) && dalloc(m, &m->WbT[l], nw) &&
              dalloc(m, &m->b[l], m->D[l]) && dalloc(m, &m->mb[l], m->D[l]) && dalloc(m, &m->vb[l], m->D[l]) &&
-             dalloc(m, &m->gb[l], m->D[l]) && dalloc(m, &m->db_raw[l], m->D[l]) &&
+             dalloc(m, &m->gb[l], m->D[l]) &&
              dalloc(m, &m->dz[l], (size_t)Bm * m->D[l]) && dalloc(m, &m->dzT[l], (size_t)Bm * m->D[l]);
-        const int Smax = 64;
-        m->partial_elems = std::max(m->partial_elems, (size_t)Smax * nw);
     }
     for (int l = 0; l < m->nl && ok; ++l) {
         ok = ok && dalloc(m, &m->act[l], (size_t)Bm * m->D[l]) && dalloc(m, &m->actT[l], (size_t)Bm * m->D[l]);
@@ -492,10 +498,11 @@ int gwam_mlp_create(gwam_mlp** out, const gwam_mlp_config* cfg, void* stream)
     }
     const int Dn = m->D[m->nl];
     ok = ok && dalloc(m, &m->Y, (size_t)Bm * Dn) && dalloc(m, &m->T, (size_t)Bm * Dn) &&
-         dalloc(m, &m->partial, m->partial_elems) && dalloc(m, &m->xmu, m->D[0]) && dalloc(m, &m->xisig, m->D[0]) &&
+         dalloc(m, &m->xmu, m->D[0]) && dalloc(m, &m->xisig, m->D[0]) &&
          dalloc(m, &m->lo, m->D[0]) && dalloc(m, &m->hi, m->D[0]) && dalloc(m, &m->ymu, Dn) &&
-         dalloc(m, &m->yisig, Dn) && dalloc(m, &m->ysig, Dn) && dalloc(m, &m->err, 1) && dalloc(m, &m->loss, 1) &&
+         dalloc(m, &m->yisig, Dn) && dalloc(m, &m->ysig, Dn) && dalloc(m, &m->loss, 2) &&
          dalloc(m, &m->nfb, 1);
+    m->err = reinterpret_cast<int*>(m->loss + 1);   // cleared together
     if (!ok) {
         gwam_mlp_destroy(m);
         return GWAM_ENOMEM;
@@ -504,13 +511,14 @@ int gwam_mlp_create(gwam_mlp** out, const gwam_mlp_config* cfg, void* stream)
     for (int l = 1; l <= m->nl && ok; ++l) {
         const int Di = m->D[l - 1], Do = m->D[l];
         ok = ok && gwam::make_tmap_bf16(&m->tf_a[l], m->act[l - 1], Bm, Di, Di, 128) &&
-             gwam::make_tmap_bf16(&m->tf_b[l], m->Wb[l], Do, Di, Di, m->bn_f[l]) &&
              gwam::make_tmap_bf16(&m->tx_a[l], m->dz[l], Bm, Do, Do, 128) &&
-             gwam::make_tmap_bf16(&m->tx_b[l], m->WbT[l], Di, Do, Do, m->bn_x[l]) &&
              gwam::make_tmap_bf16(&m->tw_a[l], m->dzT[l], Do, Bm, Bm, 128) &&
-             gwam::make_tmap_bf16(&m->tw_b[l], m->actT[l - 1], Di, Bm, Bm, m->bn_w[l]) &&
+             gwam::make_tmap_bf16(&m->tw_b[l], m->actT[l - 1], Di, Bm, Bm, gwam::kGradBN) &&
              gwam::make_tmap_bf16(&m->to_dz[l], m->dz[l], Bm, Do, Do, 32) &&
              (l == m->nl || gwam::make_tmap_bf16(&m->to_act[l], m->act[l], Bm, Do, Do, 32));
+        for (int w = 0; w < 4 && ok; ++w)
+            ok = gwam::make_tmap_bf16(&m->tf_b[l][w], m->Wb[l], Do, Di, Di, 64 * (w + 1)) &&
+                 gwam::make_tmap_bf16(&m->tx_b[l][w], m->WbT[l], Di, Do, Do, 64 * (w + 1));
     }
     if (!ok) {
         gwam_mlp_destroy(m);
@@ -642,17 +650,11 @@ int gwam_mlp_get_params_host(gwam_mlp* m, int layer, int which, float* W, float*
 {
     // which: 0 master weights, 1 gradients of the last train step
     if (!m || layer < 1 || layer > m->nl || (which != 0 && which != 1)) return fail(m, GWAM_EINVAL, "bad arguments");
-    const int Do = m->D[layer], Di = m->D[layer - 1], no = m->N[layer], ni = m->N[layer - 1];
-    std::vector<float> Wp((size_t)Do * Di), bp(Do);
-    cudaMemcpyAsync(Wp.data(), which ? m->gW[layer] : m->W[layer], Wp.size() * 4, cudaMemcpyDeviceToHost, m->s);
-    cudaMemcpyAsync(bp.data(), which ? m->gb[layer] : m->b[layer], bp.size() * 4, cudaMemcpyDeviceToHost, m->s);
-    if (cudaStreamSynchronize(m->s) != cudaSuccess) return fail(m, GWAM_ECUDA, "copy failed");
-    for (int o = 0; o < no; ++o) {
-        if (W)
-            for (int i = 0; i < ni; ++i) W[(size_t)o * ni + i] = Wp[(size_t)o * Di + i];
-        if (b) b[o] = bp[o];
-    }
-    return GWAM_OK;
+    const size_t Di = m->D[layer - 1], no = m->N[layer], ni = m->N[layer - 1];
+    if (W)
+        cudaMemcpy2DAsync(W, ni * 4, which ? m->gW[layer] : m->W[layer], Di * 4, ni * 4, no, cudaMemcpyDeviceToHost, m->s);
+    if (b) cudaMemcpyAsync(b, which ? m->gb[layer] : m->b[layer], no * 4, cudaMemcpyDeviceToHost, m->s);
+    return cudaStreamSynchronize(m->s) == cudaSuccess ? GWAM_OK : fail(m, GWAM_ECUDA, "copy failed");
 }
 
 int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, const int32_t* rows, int batch,
@@ -662,11 +664,10 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
         return fail(m, GWAM_EINVAL, "bad arguments (batch must be a multiple of 64 up to max_batch)");
     if (!m->has_norm) return fail(m, GWAM_ESTATE, "normalisation not set");
     const int B = batch, L = m->nl, Dn = m->D[L];
-    cudaMemsetAsync(m->loss, 0, sizeof(double), m->s);
-    cudaMemsetAsync(m->err, 0, sizeof(int), m->s);
-    k_batch_inputs<<<dim3((m->D[0] + 31) / 32, B / 32), dim3(32, 8), 0, m->s>>>(
-        X, n, m->N[0], m->D[0], rows, seed, m->xmu, m->xisig, m->act[0], m->actT[0], m->max_batch, m->err);
-    k_batch_targets<<<B, 128, 0, m->s>>>(Y, n, m->N[L], Dn, B, rows, seed, m->ymu, m->yisig, m->T);
+    cudaMemsetAsync(m->loss, 0, 2 * sizeof(double), m->s);   // and err
+    bool ok = launch_pdl(k_batch, dim3((m->D[0] + Dn) / 32, B / 32), dim3(32, 8), m->s, X, Y, n, m->N[0], m->D[0],
+                         m->N[L], Dn, rows, seed, (const float*)m->xmu, (const float*)m->xisig, (const float*)m->ymu,
+                         (const float*)m->yisig, m->act[0], m->actT[0], m->max_batch, m->T, m->err);
     gwam::GemmEpi last{};
     last.mode = gwam::EPI_LOSS;
     last.cf = m->Y;
@@ -680,46 +681,59 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
     last.ldcb = Dn;
     last.ct = m->dzT[L];
     last.ldct = m->max_batch;
-    bool ok = forward(m, B, true, last);
-    for (int l = L; l >= 1 && ok; --l) {
-        // weight gradient: dW_l = dz_l^T act_{l-1} (split-K partial slices)
-        const int S = wgrad_split(m, l, B);
-        gwam::GemmEpi e{};
-        e.mode = gwam::EPI_STORE;
-        e.M = m->D[l];
-        e.N = m->D[l - 1];
-        e.cf = m->partial;
-        e.ldcf = m->D[l - 1];
-        e.cf_slice = (long long)m->D[l] * m->D[l - 1];
-        ok = gemm(m, m->tw_a[l], m->tw_b[l], nullptr, B, m->bn_w[l], S, e);
-        k_rowsum<<<m->D[l], 256, 0, m->s>>>(m->dzT[l], m->max_batch, B, m->D[l], m->db_raw[l]);
-        // input gradient of the layer below, times GELU'(Z_{l-1})
-        if (l > 1 && ok) {
-            gwam::GemmEpi x{};
-            x.mode = gwam::EPI_BWD;
-            x.M = B;
-            x.N = m->D[l - 1];
-            x.z = m->Z[l - 1];
-            x.ldz = m->D[l - 1];
-            x.cb = m->dz[l - 1];
-            x.ldcb = m->D[l - 1];
-            x.ct = m->dzT[l - 1];
-            x.ldct = m->max_batch;
-            ok = gemm(m, m->tx_a[l], m->tx_b[l], &m->to_dz[l - 1], m->D[l], m->bn_x[l], 1, x);
+    ok = ok && forward(m, B, true, last);
+    // input gradients down the layers, times GELU'(Z_{l-1})
+    for (int l = L; l > 1 && ok; --l) {
+        gwam::GemmEpi x{};
+        x.mode = gwam::EPI_BWD;
+        x.M = B;
+        x.N = m->D[l - 1];
+        x.z = m->Z[l - 1];
+        x.ldz = m->D[l - 1];
+        x.cb = m->dz[l - 1];
+        x.ldcb = m->D[l - 1];
+        x.ct = m->dzT[l - 1];
+        x.ldct = m->max_batch;
+        const int bn = gwam::gemm_pick_bn(B, x.N);
+        ok = gemm(m, m->tx_a[l], m->tx_b[l][bn / 64 - 1], &m->to_dz[l - 1], m->D[l], bn, 1, x);
+    }
+    // then the weight gradients of all layers, dW_l = dz_l^T act_{l-1}, with the weight updates in one
+    // launch and the biases in one: with a GEMM, a row sum and two updates per layer a step was 33 launches
+    if (ok) {
+        const long long t = lr > 0 ? m->t + 1 : std::max(1ll, m->t);
+        const gwam::Adam adam{lr, m->b1, m->b2, m->eps, (float)(1.0 - std::pow((double)m->b1, (double)t)),
+                              (float)(1.0 - std::pow((double)m->b2, (double)t))};
+        gwam::GradSet g{};
+        BiasSet u{};
+        int outputs = 0;
+        for (int l = 1; l <= L; ++l) {
+            const int j = l - 1;
+            g.ta[j] = m->tw_a[l];
+            g.tb[j] = m->tw_b[l];
+            g.g[j] = m->gW[l];
+            g.W[j] = m->W[l];
+            g.m[j] = m->mW[l];
+            g.v[j] = m->vW[l];
+            g.Wb[j] = m->Wb[l];
+            g.WbT[j] = m->WbT[l];
+            g.M[j] = m->D[l];
+            g.N[j] = m->D[l - 1];
+            g.n_o[j] = u.n_o[j] = m->N[l];
+            g.n_i[j] = m->N[l - 1];
+            g.S[j] = wgrad_split(m, l, B);
+            u.dzT[j] = m->dzT[l];
+            u.gb[j] = m->gb[l];
+            u.b[j] = m->b[l];
+            u.mb[j] = m->mb[l];
+            u.vb[j] = m->vb[l];
+            u.end[j] = outputs += m->D[l];
         }
-        // Adam (or gradients only when lr = 0)
-        if (ok) {
-            const long long t = lr > 0 ? m->t + 1 : std::max(1ll, m->t);
-            const float c1 = (float)(1.0 - std::pow((double)m->b1, (double)t));
-            const float c2 = (float)(1.0 - std::pow((double)m->b2, (double)t));
-            const long long nw = (long long)m->D[l] * m->D[l - 1];
-            const int blocks = (int)std::min<long long>((nw + 255) / 256, 4 * 152);
-            k_adam_weights<<<blocks, 256, 0, m->s>>>(m->partial, S, nw, m->D[l], m->D[l - 1], m->N[l], m->N[l - 1],
-                                                     m->gW[l], m->W[l], m->mW[l], m->vW[l], m->Wb[l], m->WbT[l], lr,
-                                                     m->b1, m->b2, m->eps, c1, c2);
-            k_adam_bias<<<(m->D[l] + 127) / 128, 128, 0, m->s>>>(m->db_raw[l], m->D[l], m->N[l], m->gb[l], m->b[l],
-                                                                 m->mb[l], m->vb[l], lr, m->b1, m->b2, m->eps, c1, c2);
-        }
+        g.n = u.nl = L;
+        u.ld = m->max_batch;
+        u.B = B;
+        g.adam = u.adam = adam;
+        ok = gwam::gemm_bf16_grad_launch(g, B, m->err, m->s) &&
+             launch_pdl(k_bias_update, dim3((outputs + 7) / 8), dim3(256), m->s, u);
     }
     if (!ok || cudaPeekAtLastError() != cudaSuccess) return fail(m, GWAM_ECUDA, "kernel launch failed");
     if (lr > 0) ++m->t;
@@ -763,8 +777,10 @@ int gwam_mlp_infer(gwam_mlp* m, const float* X, int64_t ncol, double* dudt, doub
         const int rows = (int)std::min<int64_t>(m->max_batch, ncol - c0);
         if (m->prof && m->prof_used + 3 > 3 * 64) prof_harvest(m);
         if (m->prof) prof_mark(m);
-        k_pack_infer<<<(rows + 7) / 8, 256, 0, m->s>>>(X, ncol, c0, rows, m->N[0], m->D[0], m->xmu, m->xisig, m->lo,
-                                                      m->hi, m->act[0], fallback_mask, n_fallback);
+        if (!launch_pdl(k_pack_infer, dim3((rows + 7) / 8), dim3(256), m->s, X, ncol, c0, rows, m->N[0], m->D[0],
+                        (const float*)m->xmu, (const float*)m->xisig, (const float*)m->lo, (const float*)m->hi,
+                        m->act[0], fallback_mask, n_fallback))
+            return fail(m, GWAM_ECUDA, "kernel launch failed");
         gwam::GemmEpi last{};
         last.mode = gwam::EPI_DRAG;
         last.n_true = m->N[m->nl];
