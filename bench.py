@@ -755,13 +755,13 @@ def surrogate_arm(args):
 
 
 def launches_per_step(params, fp32=False) -> int:
-    """Kernels of the library per eager gwam_step (memsets excluded): begin, advance, the two kernels
+    """Kernels of the library per eager gwam_step: advance, the two kernels
     that scan the new-id and per-cell counts together, scatter, segment sort, materialise, project,
     divergence, budget fold; the cap's find, apply and scan; the saturation's run list and kappa; in
     the FP64 form the smoothing, or without smoothing the split of the fields into double-float
     pairs; in the precision form the smoothing (which narrows the FP64 fields as it reads them), or
     without smoothing the narrowing pass."""
-    n = 1 + 1 + 2 + 1 + 1 + 1 + 1 + 1 + 1
+    n = 1 + 2 + 1 + 1 + 1 + 1 + 1 + 1
     if params.get("cap_per_column", 0) > 0:
         n += 2 + 2
     if params.get("saturation", 0):

@@ -35,7 +35,7 @@ static void free_all(Context& c)
 {
     void* ptrs[] = {c.bg, c.bg32, c.bgdf, c.ray32_mem[0], c.ray32_mem[1], c.rho, c.rho_inv, c.tables, c.tables32, c.tables_df,
                     c.bg_scratch, c.theta,
-                    c.ray_mem[0], c.ray_mem[1], c.info, c.ccell, c.cslot, c.newid,
+                    c.ray_mem[0], c.ray_mem[1], c.info, c.child0, c.ccell, c.cslot, c.newid,
                     c.ent_id, c.ent_src, c.ent_cell, c.sorted_src, c.pj, c.k2, c.kappa, c.raycell, c.ecap, c.cnt, c.off, c.off2,
                     c.overlist, c.biglist, c.scan_tmp, c.dudt_buf, c.dvdt_buf, c.ctl,
                     c.budget, c.partials, c.flag_dev, c.spec_buf, c.launch_cols};
@@ -351,6 +351,7 @@ int gwam_init(gwam_ctx** out, const gwam_grid* grid, const gwam_params* params, 
         if (c.f32) dalloc(c, c.bg32, ncell);
         else dalloc(c, c.bgdf, ncell);
         dalloc(c, c.info, nr);
+        dalloc(c, c.child0, nr);
         dalloc(c, c.ccell, nr);
         dalloc(c, c.cslot, nr);
         dalloc(c, c.newid, nr + 1);
@@ -403,7 +404,7 @@ int gwam_init(gwam_ctx** out, const gwam_grid* grid, const gwam_params* params, 
         GWAM_CUDA(cudaMallocHost((void**)&c.flag_host, sizeof(int)));
         GWAM_CUDA(cudaMemsetAsync(c.ctl, 0, sizeof(Ctl), c.stream));
         GWAM_CUDA(cudaMemsetAsync(c.budget, 0, sizeof(DevBudget), c.stream));
-        GWAM_CUDA(cudaMemsetAsync(c.partials, 0, sizeof(double) * NTALLY * c.max_blocks, c.stream));
+        GWAM_CUDA(cudaMemsetAsync(c.cnt, 0, sizeof(int) * (ncell + 1), c.stream));   // then cleared by every step
         configure_kernels();
         GWAM_CUDA(cudaStreamSynchronize(c.stream));
         GWAM_CUDA(cudaGetLastError());
@@ -1270,6 +1271,9 @@ int gwam_load(gwam_ctx* ctx, const char* path)
         GWAM_CUDA(cudaMemcpyAsync(dst, rays.data() + q * bytes, bytes, cudaMemcpyHostToDevice, c.stream));
     }
     *c.ctl_host = h.ctl;
+    // the step's own counts start every step at zero (a file may hold those of its last step)
+    c.ctl_host->n_over = c.ctl_host->n_big = c.ctl_host->n_children = 0;
+    c.ctl_host->new_ids = 0;
     *c.budget_host = h.budget;
     GWAM_CUDA(cudaMemcpyAsync(c.ctl, c.ctl_host, sizeof(Ctl), cudaMemcpyHostToDevice, c.stream));
     GWAM_CUDA(cudaMemcpyAsync(c.budget, c.budget_host, sizeof(DevBudget), cudaMemcpyHostToDevice, c.stream));

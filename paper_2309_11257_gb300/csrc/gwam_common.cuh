@@ -145,6 +145,32 @@ __device__ __forceinline__ bool warp_run_interior(int key)
     return start > 0 && end < 31;
 }
 
+// The cell offsets of a step: before the cap, and after it.  The second scan runs only when a column
+// was over the cap; otherwise the first one's offsets stand.
+struct CellOffsets {
+    const int *before, *after;
+    __device__ __forceinline__ const int* live(const Ctl* ctl) const { return ctl->n_over ? after : before; }
+};
+
+// All threads: zero part m of `parts` of n ints (a 16-byte aligned array), grid-stride within the part
+__device__ __forceinline__ void clear_ints(int* p, int n, int m, int parts)
+{
+    const int per = (n / 4 + parts - 1) / parts, end = min((m + 1) * per, n / 4);
+    for (int i = m * per + blockIdx.x * blockDim.x + threadIdx.x; i < end; i += gridDim.x * blockDim.x)
+        reinterpret_cast<int4*>(p)[i] = make_int4(0, 0, 0, 0);
+    if (m == 0 && blockIdx.x == 0 && (int)threadIdx.x < n % 4) p[n - 1 - threadIdx.x] = 0;
+}
+
+// First entry of this warp in pass m of a loop over n entries (n or more: none): consecutive entries
+// block by block, except that fewer entries than the grid has threads go a warp to every block before
+// the second of any (2600 ray volumes kept 11 of 152 SMs busy).
+__device__ __forceinline__ int64_t loop_warp(int m, int n)
+{
+    const int T = gridDim.x * blockDim.x, w = threadIdx.x >> 5;
+    if (n < T) return m ? n : ((int64_t)w * gridDim.x + blockIdx.x) * 32;
+    return (int64_t)m * T + (int64_t)blockIdx.x * blockDim.x + w * 32;
+}
+
 // ---------------------------------------------------------------------------- per-column cap (App. B.5)
 
 // Doubles as unsigned integers of the same order (-0 = +0, NaN above everything): comparisons on the

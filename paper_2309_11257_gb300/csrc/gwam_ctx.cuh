@@ -80,8 +80,9 @@ struct Context {
 
     // per-ray scratch
     int* info = nullptr;            // split code | children << 4 | status << 8
-    int4* ccell = nullptr;          // child cells (-1 = left the domain)
-    int4* cslot = nullptr;          // child slot inside its cell
+    int2* child0 = nullptr;         // first child: its cell (-1 = left the domain) and its slot there
+    int4* ccell = nullptr;          // all children's cells and slots, written for ray volumes that split
+    int4* cslot = nullptr;
     int* newid = nullptr;           // ids needed per ray -> exclusive prefix
     long long* ent_id = nullptr;    // entry id (in cell-offset order)
     int* ent_src = nullptr;         // entry source: parent * 4 + child, < 0 removed by the cap
@@ -226,7 +227,7 @@ void prof_harvest(Context& c);
 void launch_gather_rays(Context& c, double* state13, long long* ids, int* cells, int64_t cap);
 void launch_field_to_caller(Context& c, const double* src, double* dst, int nlev);
 void launch_gamma_to_caller(Context& c, double* dst);
-void exclusive_scan(Context& c, const int* in, int* out, int64_t n, const int* n_dev);
+void exclusive_scan(Context& c, const int* in, int* out, int64_t n, const int* n_dev, const int* run_if = nullptr);
 // two independent exclusive scans in one pair of launches
 void exclusive_scan2(Context& c, const int* in0, int* out0, int64_t n0, const int* n_dev0, const int* in1,
                      int* out1, int64_t n1, const int* n_dev1);
@@ -234,6 +235,26 @@ int scan_block_count(int64_t n);
 // histogram of the cells + exclusive scan (the two offsets entry points); each launch's own status
 cudaError_t launch_cell_offsets(const int32_t* cells, int64_t n, int32_t ncell, int* counts, int* scratch, int* flag,
                                 cudaStream_t s);
-void finalize_tallies(Context& c, int slot_mask, int mode);
+void finalize_step(Context& c, int slot_mask);
+void finalize_launch(Context& c, int blocks, const int* launched, int total);
+
+// Columns a smoothing warp slides over: `most` where `rows` row groups x levels x fields give at least
+// 16 warps per SM, halved (down to 4: a span reads two columns beside its own) while they do not.  On
+// a small grid the time is that of one warp's chain of columns.
+inline int smooth_span(const Context& c, long long rows, int most)
+{
+    int span = most;
+    while (span > 4 && rows * ((c.G.nx + span - 1) / span) < 16LL * c.num_sms) span /= 2;
+    return span;
+}
+
+// Columns of a divergence block: 32 (16 for more than 96 levels: shared memory), halved while the
+// grid gives fewer than two blocks per SM, down to 4 (a 16 x 16 box ran on 16 SMs)
+inline int divergence_tile(const Context& c)
+{
+    int tw = c.G.nz <= 96 ? 32 : 16;
+    while (tw > 4 && (long long)((c.G.nx + tw - 1) / tw) * c.G.ny * c.G.members < 2LL * c.num_sms) tw /= 2;
+    return tw;
+}
 
 }  // namespace gwam

@@ -60,20 +60,20 @@ struct FieldSet32 {
 };
 
 // separable 1-2-1 x 1-2-1 smoothing (periodic in lambda, edge row reused at the poles).  A warp
-// owns 32 consecutive levels of kRows32 rows over a run of kSpan columns and slides a 3 x 3 window
+// owns 32 consecutive levels of kRows32 rows over a span of columns and slides a 3 x 3 window
 // along the rows: each new column costs kRows32 + 2 loads (the rows and their two neighbours) for
 // kRows32 outputs, and the column sums of the previous two columns stay in registers.  All loads of
 // a pass (two columns) are issued before any of them is converted.  Three rows over spans of 32
 // columns, reading the FP64 fields: 5/3 loads per output, measured faster than two, four or six
-// rows or spans of 16 (more rows hold more registers).  Warp item = (field, member, row group,
+// rows or spans of 16 (more rows hold more registers); small grids take shorter spans
+// (smooth_span).  Warp item = (field, member, row group,
 // level group, span).
-constexpr int kSpan = 32;
 constexpr int kRows32 = 3;
-__global__ void __launch_bounds__(256) k_smooth_fields32(Grid G, FieldSet32 fs, int f0, int nf)
+__global__ void __launch_bounds__(256) k_smooth_fields32(Grid G, FieldSet32 fs, int f0, int nf, int span)
 {
     const int lane = threadIdx.x & 31;
     const int nlg = (G.nz + 1 + 31) / 32;                   // level groups (interface fields have nz + 1)
-    const int nsp = (G.nx + kSpan - 1) / kSpan;
+    const int nsp = (G.nx + span - 1) / span;
     const int nrg = (G.ny + kRows32 - 1) / kRows32;
     const long long per_field = (long long)G.members * nrg * nlg * nsp;
     const long long items = per_field * nf;
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) k_smooth_fields32(Grid G, FieldSet32 fs, 
         loadcol(i, raw);
         sums(raw, cs);
     };
-    const int i0 = sp * kSpan, i1 = min(G.nx, i0 + kSpan);
+    const int i0 = sp * span, i1 = min(G.nx, i0 + span);
     float cm[kRows32], c0[kRows32], cp[kRows32], cq[kRows32];
     colsums(i0 == 0 ? G.nx - 1 : i0 - 1, cm);
     colsums(i0, c0);
@@ -275,11 +275,22 @@ __device__ __forceinline__ void sat_run32(int p, int b, int c, const double* __r
                                           const double* __restrict__ pj, const float* __restrict__ k2, float dt,
                                           float* __restrict__ kappa)
 {
+    // four terms at a time, their loads issued before they are added (in order), as in sat_run
     double Pc = 0.0, Q = 0.0;
-    for (int q = p; q < b; ++q) {
-        const double v = pj[q];
-        Pc += v;
-        Q = fma(v, widen(k2[q]), Q);
+    for (int q = p; q < b; q += 4) {
+        double v[4];
+        float k[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            v[u] = q + u < b ? pj[q + u] : 0.0;
+            k[u] = q + u < b ? k2[q + u] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (q + u < b) {
+                Pc += v[u];
+                Q = fma(v[u], widen(k[u]), Q);
+            }
     }
     const double d = fma(-0.5, rho[c], Pc);
     float kap = 0.0f;
@@ -288,11 +299,12 @@ __device__ __forceinline__ void sat_run32(int p, int b, int c, const double* __r
 }
 
 // the listed runs (k_sat_heads of the FP64 form lists them), one per lane
-__global__ void k_sat_kappa32(const Ctl* ctl, const int* __restrict__ off2, const int* __restrict__ runlist,
+__global__ void k_sat_kappa32(const Ctl* ctl, CellOffsets cell, const int* __restrict__ runlist,
                               const double* __restrict__ rho, const double* __restrict__ pj,
                               const float* __restrict__ k2, float dt, float* __restrict__ kappa)
 {
     const int nl = ctl->status ? 0 : ctl->n_big;
+    const int* __restrict__ off2 = cell.live(ctl);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nl; t += gridDim.x * blockDim.x) {
         const int c = runlist[t];
         sat_run32(off2[c], off2[c + 1], c, rho, pj, k2, dt, kappa);
@@ -321,9 +333,11 @@ static void smooth32(Context& c, int f0, int f1)
         fs.in[f] = c.field[f];
         fs.out[f] = c.sm32[f];
     }
-    const long long warps = (long long)(f1 - f0) * c.G.members * ((c.G.ny + kRows32 - 1) / kRows32) *
-                            ((c.G.nz + 1 + 31) / 32) * ((c.G.nx + kSpan - 1) / kSpan);
-    k_smooth_fields32<<<(unsigned)((warps + 7) / 8), 256, 0, c.stream>>>(c.G, fs, f0, f1 - f0);
+    const long long rows = (long long)(f1 - f0) * c.G.members * ((c.G.ny + kRows32 - 1) / kRows32) *
+                           ((c.G.nz + 1 + 31) / 32);
+    const int span = smooth_span(c, rows, 32);
+    const long long warps = rows * ((c.G.nx + span - 1) / span);
+    k_smooth_fields32<<<(unsigned)((warps + 7) / 8), 256, 0, c.stream>>>(c.G, fs, f0, f1 - f0, span);
 }
 
 void smooth_field32(Context& c, int f)
@@ -347,21 +361,22 @@ static void grid_phase32(Context& c, double* du, double* dv, int mask)
         narrow_fields(c, 0, F_WAD);
         fl = c.nar32;
     }
-    const int TW = G.nz <= 96 ? 32 : 16;
+    const int TW = divergence_tile(c);
     const size_t shm = sizeof(float) * (2 * (size_t)TW * G.nz + G.nz);
     if (shm > 48 * 1024) cudaFuncSetAttribute(k_divergence32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     const int ntx = (G.nx + TW - 1) / TW;
     k_divergence32<<<ntx * G.ny * G.members, kThreads, shm, s>>>(G, TW, fl[F_ZL], fl[F_ZP], fl[F_LL], fl[F_LP],
                                                                  fl[F_PL], fl[F_PP], fl[F_EL], fl[F_EP], c.rho_inv32,
                                                                  out_u, out_v);
-    finalize_tallies(c, mask, 1);
+    finalize_step(c, mask);
 }
 
 // RK3 advance in FP32 (the ray-step kernel of the precision form): state read and written in
 // place, exits, split decisions, child cells and slots as in k_advance.
 __global__ void __launch_bounds__(kThreads) k_advance32(Grid G, Params P, Ray32SoA A, const Node32* __restrict__ bg,
                                                           Ctl* ctl, float dt, int* __restrict__ info,
-                                                          int4* __restrict__ ccell, int4* __restrict__ cslot,
+                                                          int2* __restrict__ child0, int4* __restrict__ ccell,
+                                                        int4* __restrict__ cslot,
                                                           int* __restrict__ newid, int* __restrict__ cnt,
                                                           double* __restrict__ partials, int pstride, ClearSet zs)
 {
@@ -413,8 +428,11 @@ __global__ void __launch_bounds__(kThreads) k_advance32(Grid G, Params P, Ray32S
             store32(G, A, i, s);
         }
         info[i] = code | (nch << 4) | (st << 8);
-        ccell[i] = make_int4(cc[0], cc[1], cc[2], cc[3]);
-        cslot[i] = make_int4(sl[0], sl[1], sl[2], sl[3]);
+        child0[i] = make_int2(cc[0], sl[0]);
+        if (nch > 1) {   // few ray volumes split in a step
+            ccell[i] = make_int4(cc[0], cc[1], cc[2], cc[3]);
+            cslot[i] = make_int4(sl[0], sl[1], sl[2], sl[3]);
+        }
         newid[i] = nch > 0 ? nch - 1 : 0;
     }
     clear_finish(zs, cs);
@@ -438,7 +456,8 @@ __device__ __forceinline__ long long id32(const Ray32SoA& A, int64_t i)
 }
 
 __global__ void k_scatter32(Grid G, Ray32SoA A, Ctl* ctl, int64_t max_rays, const int* __restrict__ info,
-                            const int4* __restrict__ ccell, const int4* __restrict__ cslot,
+                            const int2* __restrict__ child0, const int4* __restrict__ ccell,
+                            const int4* __restrict__ cslot,
                             const int* __restrict__ newid, const int* __restrict__ off,
                             long long* __restrict__ ent_id, int* __restrict__ ent_src, int* __restrict__ ent_cell)
 {
@@ -454,11 +473,17 @@ __global__ void k_scatter32(Grid G, Ray32SoA A, Ctl* ctl, int64_t max_rays, cons
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int nch = (info[i] >> 4) & 7;
         if (!nch) continue;
-        const int4 cc = ccell[i], sl = cslot[i];
-        const int cs[4] = {cc.x, cc.y, cc.z, cc.w}, ss[4] = {sl.x, sl.y, sl.z, sl.w};
+        const int2 first = child0[i];
+        int cs[4] = {first.x, -1, -1, -1}, ss[4] = {first.y, 0, 0, 0};
+        if (nch > 1) {
+            const int4 cc = ccell[i], sl = cslot[i];
+            cs[1] = cc.y; cs[2] = cc.z; cs[3] = cc.w;
+            ss[1] = sl.y; ss[2] = sl.z; ss[3] = sl.w;
+        }
         const long long pid = id32(A, i);
-        for (int c = 0; c < nch; ++c) {
-            if (cs[c] < 0) continue;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (c >= nch || cs[c] < 0) continue;
             const int64_t pos = (int64_t)off[cs[c]] + ss[c];
             if (pos >= max_rays) continue;
             ent_id[pos] = c == 0 ? pid : with_member(member_of(pid), next + newid[i] + c - 1);
@@ -516,15 +541,14 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_apply32(Grid G, Params P, R
 
 __global__ void __launch_bounds__(kThreads) k_materialize32(Grid G, Params P, Ray32SoA A, Ray32SoA B,
                                                               const Node32* __restrict__ bg, Ctl* ctl,
-                                                              const int* __restrict__ off2,
-                                                              const int* __restrict__ sorted_src,
+                                                              CellOffsets cell, const int* __restrict__ sorted_src,
                                                               const int* __restrict__ info,
                                                               const int* __restrict__ newid,
                                                               double* __restrict__ pj, float* __restrict__ k2,
                                                               int* __restrict__ raycell)
 {
     if (ctl->status) return;
-    const int n_new = off2[G.ncell_all];
+    const int n_new = cell.live(ctl)[G.ncell_all];
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->n_new = n_new;   // the live count k_finalize closes the step with
     const int n_old = ctl->n;
     const long long next = ctl->next_id;
@@ -561,7 +585,7 @@ __global__ void __launch_bounds__(kThreads) k_materialize32(Grid G, Params P, Ra
 // THETA: also the potential-temperature flux integrals of Eq. fluxes:temperature (fields F_TL, F_TP)
 template <bool THETA>
 __global__ void __launch_bounds__(kThreads) k_project32(Grid G, Params P, Ray32SoA B, const Node32* __restrict__ bg,
-                                                          const Ctl* ctl, const int* __restrict__ off2,
+                                                          const Ctl* ctl, CellOffsets cell, int* __restrict__ cnt,
                                                           const float* __restrict__ kappa,
                                                           const float* __restrict__ k2, double dt,
                                                           double* __restrict__ fz_l, double* __restrict__ fz_p,
@@ -576,12 +600,15 @@ __global__ void __launch_bounds__(kThreads) k_project32(Grid G, Params P, Ray32S
     // FP64 work is kept out of the per-ray path (GB300's FP64 rate is 1/72 of FP32): the action
     // and the budget terms in double-float, float -> double by integer widening, FP64 only in the
     // grid atomics (L2) and one addition per thread for the budget
-    const int n = ctl->status ? 0 : off2[G.ncell_all];
+    const int n = ctl->status ? 0 : cell.live(ctl)[G.ncell_all];
     DF w_sat{0.0f, 0.0f}, w_tot{0.0f, 0.0f};
     const float dtf = (float)dt;
-    const int stride = gridDim.x * blockDim.x;
-    for (int p0 = blockIdx.x * blockDim.x; p0 < n; p0 += stride) {
-        const int p = p0 + threadIdx.x;
+    const int passes = loop_passes(n);
+    for (int m = 0; m < passes; ++m) {
+        clear_ints(cnt, G.ncell_all + 1, m, passes);   // the cells' counters, for the next step
+        const int64_t p0 = loop_warp(m, n);
+        if (p0 >= n) continue;
+        const int p = (int)p0 + (threadIdx.x & 31);
         const bool act = p < n;
         int key = -1;
         DF hv[NH];
@@ -719,12 +746,11 @@ void launch_gather_rays32(Context& c, double* state13, long long* ids, int* cell
 }
 
 // kernels shared with the FP64 step (gwam_step.cu)
-__global__ void k_step_begin(Ctl* ctl);
 __global__ void k_cap_find(Grid G, Params P, Ctl* ctl, const int* __restrict__ off, int* __restrict__ overlist);
-__global__ void k_segsort(Grid G, Ctl* ctl, const int* __restrict__ off, const int* __restrict__ off2,
+__global__ void k_segsort(Grid G, Ctl* ctl, CellOffsets cell,
                           const long long* __restrict__ ent_id, const int* __restrict__ ent_src,
                           const int* __restrict__ ent_cell, int* __restrict__ sorted_src);
-__global__ void __launch_bounds__(kThreads) k_sat_heads(Ctl* ctl, const int* __restrict__ off2, int ncell_all,
+__global__ void __launch_bounds__(kThreads) k_sat_heads(Ctl* ctl, CellOffsets cell, int ncell_all,
                                                           const int* __restrict__ raycell, int* __restrict__ runlist);
 
 void run_step32(Context& c, double dt, double* du, double* dv)
@@ -739,39 +765,35 @@ void run_step32(Context& c, double dt, double* du, double* dv)
     const LaunchCfg& la = c.lcfg[0];
     const LaunchCfg& lm = c.lcfg[1];
     const LaunchCfg& lp = c.lcfg[2];
-    k_step_begin<<<1, 1, 0, s>>>(c.ctl);
-    cudaMemsetAsync(c.cnt, 0, sizeof(int) * (size_t)(G.ncell_all + 1), s);
-    cudaMemsetAsync(c.partials, 0, sizeof(double) * NTALLY * (size_t)c.max_blocks, s);
     prof_mark(c, 0);
     tune_mark(c, 0);
-    k_advance32<<<la.blocks, la.threads, 0, s>>>(G, P, c.A32, c.bg32, c.ctl, (float)dt, c.info, c.ccell, c.cslot,
+    k_advance32<<<la.blocks, la.threads, 0, s>>>(G, P, c.A32, c.bg32, c.ctl, (float)dt, c.info, c.child0, c.ccell, c.cslot,
                                                  c.newid, c.cnt, c.partials, c.max_blocks, clear_set(c));
     tune_mark(c, 1);
     prof_mark(c, 1);
     exclusive_scan2(c, c.newid, c.newid, c.max_rays, &c.ctl->n, c.cnt, c.off, G.ncell_all, nullptr);
-    k_scatter32<<<nb, kThreads, 0, s>>>(G, c.A32, c.ctl, c.max_rays, c.info, c.ccell, c.cslot, c.newid, c.off,
+    k_scatter32<<<nb, kThreads, 0, s>>>(G, c.A32, c.ctl, c.max_rays, c.info, c.child0, c.ccell, c.cslot, c.newid, c.off,
                                         c.ent_id, c.ent_src, c.ent_cell);
     int mask = (1 << T_EXIT) | (1 << T_INVALID) | (1 << T_SAT) | (1 << T_TOTAL);
-    const int* off2 = c.off;
+    const CellOffsets cell{c.off, c.off2};
     if (P.cap > 0) {
         k_cap_find<<<col_blocks, kThreads, 0, s>>>(G, P, c.ctl, c.off, c.overlist);
         k_cap_apply32<<<c.max_blocks, kCapThreads, 0, s>>>(G, P, c.A32, c.bg32, c.ctl, c.info, c.off, c.overlist, c.ent_id,
                                                            c.ent_src, c.ent_cell, c.ecap, c.cnt, c.partials, c.max_blocks);
-        exclusive_scan(c, c.cnt, c.off2, G.ncell_all, nullptr);
-        off2 = c.off2;
+        exclusive_scan(c, c.cnt, c.off2, G.ncell_all, nullptr, &c.ctl->n_over);
         mask |= 1 << T_CAP;
     }
-    k_segsort<<<nb, kThreads, 0, s>>>(G, c.ctl, c.off, off2, c.ent_id, c.ent_src, c.ent_cell, c.sorted_src);
+    k_segsort<<<nb, kThreads, 0, s>>>(G, c.ctl, cell, c.ent_id, c.ent_src, c.ent_cell, c.sorted_src);
     tune_mark(c, 2);
-    k_materialize32<<<lm.blocks, lm.threads, 0, s>>>(G, P, c.A32, c.B32, c.bg32, c.ctl, off2, c.sorted_src, c.info,
+    k_materialize32<<<lm.blocks, lm.threads, 0, s>>>(G, P, c.A32, c.B32, c.bg32, c.ctl, cell, c.sorted_src, c.info,
                                                      c.newid, c.pj, reinterpret_cast<float*>(c.k2), c.raycell);
     tune_mark(c, 3);
     prof_mark(c, 2);
     if (P.saturation) {
         // both saturation passes on the largest grid (eight blocks per SM, all resident): shorter
         // chains of per-block passes (saturation 0.070 -> 0.060 ms on the 512 x 256 sphere)
-        k_sat_heads<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, off2, G.ncell_all, c.raycell, c.biglist);
-        k_sat_kappa32<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, off2, c.biglist, c.rho, c.pj,
+        k_sat_heads<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, cell, G.ncell_all, c.raycell, c.biglist);
+        k_sat_kappa32<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, cell, c.biglist, c.rho, c.pj,
                                               reinterpret_cast<const float*>(c.k2), (float)dt,
                                               reinterpret_cast<float*>(c.kappa));
     }
@@ -780,13 +802,13 @@ void run_step32(Context& c, double dt, double* du, double* dv)
     tune_mark(c, 4);
     if (P.theta_flux)
         k_project32<true><<<lp.blocks, lp.threads, 0, s>>>(
-            G, P, c.B32, c.bg32, c.ctl, off2, reinterpret_cast<const float*>(c.kappa),
+            G, P, c.B32, c.bg32, c.ctl, cell, c.cnt, reinterpret_cast<const float*>(c.kappa),
             reinterpret_cast<const float*>(c.k2), dt, c.field[F_ZL], c.field[F_ZP], c.field[F_LL], c.field[F_LP],
             c.field[F_PL], c.field[F_PP], c.field[F_EL], c.field[F_EP], c.field[F_WAD], c.field[F_TL], c.field[F_TP],
             c.partials, c.max_blocks);
     else
         k_project32<false><<<lp.blocks, lp.threads, 0, s>>>(
-            G, P, c.B32, c.bg32, c.ctl, off2, reinterpret_cast<const float*>(c.kappa),
+            G, P, c.B32, c.bg32, c.ctl, cell, c.cnt, reinterpret_cast<const float*>(c.kappa),
             reinterpret_cast<const float*>(c.k2), dt, c.field[F_ZL], c.field[F_ZP], c.field[F_LL], c.field[F_LP],
             c.field[F_PL], c.field[F_PP], c.field[F_EL], c.field[F_EP], c.field[F_WAD], nullptr, nullptr,
             c.partials, c.max_blocks);

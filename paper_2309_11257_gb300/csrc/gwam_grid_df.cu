@@ -22,21 +22,20 @@ struct FieldSetDF {
 };
 
 // 1-2-1 x 1-2-1 smoothing (periodic in lambda, edge row reused at the poles): a warp owns 32
-// consecutive levels of kRowsDF rows over kSpanDF columns.  For every column it loads and splits the
+// consecutive levels of kRowsDF rows over a span of columns.  For every column it loads and splits the
 // kRowsDF + 2 values of its rows and their two neighbours once (2 loads and splits per output
 // instead of 3 for two rows: measured faster than 1, 4 or 8 rows), forms the vertical 1-2-1 sums
 // of its rows, and slides a window of three such sums along the row (spans of 16 columns: measured
-// faster than 8 or 32).  The raw values of the column after next are loaded while the next one is
+// faster than 8 or 32; small grids take shorter ones: smooth_span).  The raw values of the column after next are loaded while the next one is
 // summed, so every warp keeps two columns' loads in flight (grid phase 0.291 -> 0.228 ms on the
 // 256 x 128 x 90 sphere; a distance of two columns gained nothing more).  Warp item = (field,
 // member, row group, level group, span).
-constexpr int kSpanDF = 16;
 constexpr int kRowsDF = 2;
-__global__ void __launch_bounds__(256) k_smooth_df(Grid G, FieldSetDF fs, int f0, int nf)
+__global__ void __launch_bounds__(256) k_smooth_df(Grid G, FieldSetDF fs, int f0, int nf, int span)
 {
     const int lane = threadIdx.x & 31;
     const int nlg = (G.nz + 1 + 31) / 32;
-    const int nsp = (G.nx + kSpanDF - 1) / kSpanDF;
+    const int nsp = (G.nx + span - 1) / span;
     const int nrg = (G.ny + kRowsDF - 1) / kRowsDF;
     const long long per_field = (long long)G.members * nrg * nlg * nsp;
     const long long w = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -111,7 +110,7 @@ __global__ void __launch_bounds__(256) k_smooth_df(Grid G, FieldSetDF fs, int f0
             }
         }
     };
-    const int i0 = sp * kSpanDF, i1 = min(G.nx, i0 + kSpanDF);
+    const int i0 = sp * span, i1 = min(G.nx, i0 + span);
     DF cm[kRowsDF], c0[kRowsDF], cp[kRowsDF];
     double ra[kRowsDF + 2], rb[kRowsDF + 2];
     loadraw(i0 - 1, true, ra);
@@ -290,9 +289,11 @@ void grid_phase_df(Context& c, double* du, double* dv, int mask)
             fs.in[f] = c.field[f];
             fs.out[f] = sm[f];
         }
-        const long long warps = (long long)F_WAD * G.members * ((G.ny + kRowsDF - 1) / kRowsDF) *
-                                ((G.nz + 1 + 31) / 32) * ((G.nx + kSpanDF - 1) / kSpanDF);
-        k_smooth_df<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(G, fs, 0, F_WAD);
+        const long long rows =
+            (long long)F_WAD * G.members * ((G.ny + kRowsDF - 1) / kRowsDF) * ((G.nz + 1 + 31) / 32);
+        const int span = smooth_span(c, rows, 16);
+        const long long warps = rows * ((G.nx + span - 1) / span);
+        k_smooth_df<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(G, fs, 0, F_WAD, span);
         for (int f = 0; f < NFIELD; ++f) fl[f] = sm[f];
     } else {
         // unsmoothed: split in place into the same buffers (one pass per field)
@@ -309,14 +310,14 @@ void grid_phase_df(Context& c, double* du, double* dv, int mask)
     K.h2y = host_split(0.5 * G.inv_dY);
     K.idz = host_split(G.inv_dz);
     K.ig = host_split(G.inv_g);
-    const int TW = G.nz <= 96 ? 32 : 16;
+    const int TW = divergence_tile(c);
     const size_t shm = sizeof(double) * 2 * (size_t)TW * G.nz;
     if (shm > 48 * 1024) cudaFuncSetAttribute(k_divergence_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     const int ntx = (G.nx + TW - 1) / TW;
     k_divergence_df<<<ntx * G.ny * G.members, kThreads, shm, s>>>(
         G, TW, K, c.tables_df, fl[F_ZL], fl[F_ZP], fl[F_LL], fl[F_LP], fl[F_PL], fl[F_PP], fl[F_EL], fl[F_EP],
         c.rho_inv, out_u, out_v);
-    finalize_tallies(c, mask, 1);
+    finalize_step(c, mask);
 }
 
 }  // namespace gwam

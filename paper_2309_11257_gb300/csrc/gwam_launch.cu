@@ -327,15 +327,6 @@ __global__ void k_add_rays(Grid G, RaySoA A, Ray32SoA A32, bool f32, Ctl* ctl, i
     if (threadIdx.x == 0 && pass == 1) partials[T_LAUNCH * pstride + blockIdx.x] = wb;
 }
 
-__global__ void k_append_close(Ctl* ctl, int64_t max_rays, int added)
-{
-    int n = ctl->n + added;
-    if ((int64_t)n > max_rays) n = (int)max_rays;
-    ctl->n = n;
-    ctl->next_id += added;
-    ctl->n_launched += added;
-}
-
 void launch_add_rays(Context& c, const double* const in[13], int64_t n)
 {
     RayInputPtrs d_in;
@@ -349,11 +340,9 @@ void launch_add_rays(Context& c, const double* const in[13], int64_t n)
         c.err = "gwam_add_rays: a ray volume lies outside the domain or is invalid";
         throw (int)GWAM_EINVAL;
     }
-    cudaMemsetAsync(c.partials, 0, sizeof(double) * NTALLY * (size_t)c.max_blocks, c.stream);
     k_add_rays<<<c.grid_blocks, kThreads, 0, c.stream>>>(c.G, c.A, c.A32, c.f32, c.ctl, c.max_rays, d_in, (int)n, 1,
                                                          c.flag_dev, c.partials, c.max_blocks);
-    finalize_tallies(c, 1 << T_LAUNCH, 0);
-    k_append_close<<<1, 1, 0, c.stream>>>(c.ctl, c.max_rays, (int)n);
+    finalize_launch(c, c.grid_blocks, nullptr, (int)n);
 }
 
 // ----------------------------------------------------------------------------- sources (Sec. 3c)
@@ -491,7 +480,7 @@ __device__ __forceinline__ int ghost_emit(const Grid& G, const NodeDF* __restric
 // member alone) staged at position t of S / S32, filtered bins counted; k_launch_place then moves the
 // launched ones behind the live rays.  (While both passes computed the states, a ghost-layer launch
 // into 8192 columns took 2 x 390 us.)  kGhost: what left the ghost layer over ghost_dt instead of
-// the launch state itself.  Dynamic shared memory: the ghost's kRkSmem, then the source's sines and cosines
+// the launch state itself.  Dynamic shared memory: the ghost's kRkWarp a warp, then the source's sines and cosines
 // of the azimuths and its phase speeds (2 n_az + n_c doubles).
 template <bool kSpec, bool kGhost>
 __global__ void __launch_bounds__(kThreads, 2) k_launch(Grid G, const Node* __restrict__ bg,
@@ -502,7 +491,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_launch(Grid G, const Node* __re
                                                         int* __restrict__ flag)
 {
     extern __shared__ float4 sh_launch[];
-    double* const az = reinterpret_cast<double*>(sh_launch + (kGhost ? kRkSmem / sizeof(float4) : 0));
+    double* const az = reinterpret_cast<double*>(sh_launch + (kGhost ? kRkWarp * (blockDim.x / 32) : 0));
     double* const speed = az + 2 * src.n_az;
     const int nbins = kSpec ? 1 : src.n_az * src.n_c;
     if (!kSpec) {
@@ -608,16 +597,6 @@ void configure_launch_kernels()
     cudaFuncSetAttribute(k_launch<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRkSmem);
 }
 
-__global__ void k_launch_close(Ctl* ctl, int64_t max_rays, const int* off, int total)
-{
-    const int added = off[total];
-    int n = ctl->n + added;
-    if ((int64_t)n > max_rays) n = (int)max_rays;
-    ctl->n = n;
-    ctl->next_id += added;
-    ctl->n_launched += added;
-}
-
 static void launch_common(Context& c, const gwam_bg_source* src, const gwam_spec* specs, int64_t total,
                           double ghost_dt = 0.0)
 {
@@ -647,22 +626,25 @@ static void launch_common(Context& c, const gwam_bg_source* src, const gwam_spec
     // the ghost layer propagates vertically only: the single-column equations on this grid copy
     Grid G = c.G;
     if (ghost) G.columnar = 1;
-    const size_t shm = (ghost ? kRkSmem : 0) + (specs ? 0 : (2 * s0.n_az + s0.n_c) * sizeof(double));
+    // one wave of two blocks per SM; few bins in blocks of a warp, spread over the SMs (the bins' FP64
+    // chains share an SM's FP64 pipe: 200 bins in one block took 16 us)
+    const int threads = total >= 2 * (int64_t)c.num_sms * kThreads ? kThreads : 32;
+    const int blocks = (int)std::min<int64_t>((int64_t)nb * (kThreads / threads), (total + threads - 1) / threads);
+    const size_t shm = (ghost ? kRkSmem / (kThreads / threads) : 0) + (specs ? 0 : (2 * s0.n_az + s0.n_c) * sizeof(double));
     if (!specs) {
-        const int cb = std::min((c.G.ncol_all + 63) / 64, 32 * c.num_sms);
-        k_launch_columns<<<cb, 64, 0, c.stream>>>(c.G, c.bg, s0, reinterpret_cast<LaunchColumn*>(c.launch_cols));
+        const int cb = std::min((c.G.ncol_all + 31) / 32, 32 * c.num_sms);
+        k_launch_columns<<<cb, 32, 0, c.stream>>>(c.G, c.bg, s0, reinterpret_cast<LaunchColumn*>(c.launch_cols));
     }
     auto* kernel = specs ? (ghost ? k_launch<true, true> : k_launch<true, false>)
                          : (ghost ? k_launch<false, true> : k_launch<false, false>);
-    kernel<<<std::min<int>(nb, (int)((total + kThreads - 1) / kThreads)), kThreads, shm, c.stream>>>(
+    kernel<<<blocks, threads, shm, c.stream>>>(
         G, c.bg, c.bgdf, S, S32s, c.f32, c.ctl, s0, reinterpret_cast<const LaunchColumn*>(c.launch_cols), specs,
         (int)total, ghost_dt, flag);
     exclusive_scan(c, flag, flag, total, nullptr);
-    cudaMemsetAsync(c.partials, 0, sizeof(double) * NTALLY * (size_t)c.max_blocks, c.stream);
-    k_launch_place<<<nb, kThreads, 0, c.stream>>>(c.G, S, S32s, c.A, c.A32, c.f32, c.ctl, c.max_rays, (int)total, flag,
+    const int pb = std::min<int>(nb, (int)((total + kThreads - 1) / kThreads));
+    k_launch_place<<<pb, kThreads, 0, c.stream>>>(c.G, S, S32s, c.A, c.A32, c.f32, c.ctl, c.max_rays, (int)total, flag,
                                                   c.partials, c.max_blocks);
-    finalize_tallies(c, 1 << T_LAUNCH, 0);
-    k_launch_close<<<1, 1, 0, c.stream>>>(c.ctl, c.max_rays, flag, (int)total);
+    finalize_launch(c, pb, flag, (int)total);
     if (own) cudaFreeAsync(own, c.stream);
 }
 

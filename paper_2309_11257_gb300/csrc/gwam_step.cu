@@ -178,8 +178,10 @@ __device__ __forceinline__ const ScanJob& scan_job(const ScanJob& j0, const Scan
     return j1;
 }
 
-__global__ void __launch_bounds__(kThreads) k_part_sums(ScanJob j0, ScanJob j1)
+// run_if: nothing to do while this device int is zero (null: always run)
+__global__ void __launch_bounds__(kThreads) k_part_sums(ScanJob j0, ScanJob j1, const int* run_if)
 {
+    if (run_if && !*run_if) return;
     int part;
     const ScanJob& j = scan_job(j0, j1, part);
     const int len = scan_len(j.n, j.n_dev);
@@ -198,8 +200,9 @@ __global__ void __launch_bounds__(kThreads) k_part_sums(ScanJob j0, ScanJob j1)
     if (threadIdx.x == 0) j.psum[part] = (int)t;
 }
 
-__global__ void __launch_bounds__(kThreads) k_part_scan(ScanJob j0, ScanJob j1)
+__global__ void __launch_bounds__(kThreads) k_part_scan(ScanJob j0, ScanJob j1, const int* run_if)
 {
+    if (run_if && !*run_if) return;
     __shared__ int wsum[kPartGroup][kThreads / 32];
     __shared__ int base;
     int part;
@@ -274,13 +277,13 @@ static ScanJob scan_job_for(const Context& c, const int* in, int* out, int64_t n
 
 // Exclusive prefix of in[0..len) into out[0..len], out[len] = total; len = *n_dev if given
 // (then n is its upper bound).  in == out is allowed (every part reads its items before writing
-// them, and out[len] lies outside every part).
-void exclusive_scan(Context& c, const int* in, int* out, int64_t n, const int* n_dev)
+// them, and out[len] lies outside every part).  run_if: see k_part_sums.
+void exclusive_scan(Context& c, const int* in, int* out, int64_t n, const int* n_dev, const int* run_if)
 {
     const ScanJob j0 = scan_job_for(c, in, out, n, n_dev, c.scan_tmp, c.scan_tmp_cap);
     const ScanJob none{nullptr, nullptr, 0, nullptr, nullptr, 0};
-    k_part_sums<<<j0.nparts, kThreads, 0, c.stream>>>(j0, none);
-    k_part_scan<<<j0.nparts, kThreads, 0, c.stream>>>(j0, none);
+    k_part_sums<<<j0.nparts, kThreads, 0, c.stream>>>(j0, none, run_if);
+    k_part_scan<<<j0.nparts, kThreads, 0, c.stream>>>(j0, none, run_if);
 }
 
 // Two independent exclusive scans in the same two launches (the part sums of the second one
@@ -291,8 +294,8 @@ void exclusive_scan2(Context& c, const int* in0, int* out0, int64_t n0, const in
     const int64_t half = c.scan_tmp_cap / 2;
     const ScanJob j0 = scan_job_for(c, in0, out0, n0, n_dev0, c.scan_tmp, half);
     const ScanJob j1 = scan_job_for(c, in1, out1, n1, n_dev1, c.scan_tmp + j0.nparts, c.scan_tmp_cap - j0.nparts);
-    k_part_sums<<<j0.nparts + j1.nparts, kThreads, 0, c.stream>>>(j0, j1);
-    k_part_scan<<<j0.nparts + j1.nparts, kThreads, 0, c.stream>>>(j0, j1);
+    k_part_sums<<<j0.nparts + j1.nparts, kThreads, 0, c.stream>>>(j0, j1, nullptr);
+    k_part_scan<<<j0.nparts + j1.nparts, kThreads, 0, c.stream>>>(j0, j1, nullptr);
 }
 
 // ============================================================================ advance
@@ -303,7 +306,8 @@ constexpr size_t kAdvanceSmem = kRkSmem + 6 * kThreads * sizeof(double);
 
 __global__ void __launch_bounds__(kThreads, 2) k_advance(Grid G, Params P, RaySoA A, const NodeDF* __restrict__ bg,
                                                         Ctl* ctl, double dt, int* __restrict__ info,
-                                                        int4* __restrict__ ccell, int4* __restrict__ cslot,
+                                                        int2* __restrict__ child0, int4* __restrict__ ccell,
+                                                        int4* __restrict__ cslot,
                                                         int* __restrict__ newid, int* __restrict__ cnt,
                                                         double* __restrict__ partials, int pstride, ClearSet zs)
 {
@@ -385,8 +389,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_advance(Grid G, Params P, RaySo
             store_ray(A, i, s, id);
         }
         info[i] = code | (nch << 4) | (st << 8);
-        ccell[i] = make_int4(cc[0], cc[1], cc[2], cc[3]);
-        cslot[i] = make_int4(sl[0], sl[1], sl[2], sl[3]);
+        child0[i] = make_int2(cc[0], sl[0]);
+        if (nch > 1) {   // few ray volumes split in a step
+            ccell[i] = make_int4(cc[0], cc[1], cc[2], cc[3]);
+            cslot[i] = make_int4(sl[0], sl[1], sl[2], sl[3]);
+        }
         newid[i] = nch > 0 ? nch - 1 : 0;
     }
     const double we = block_sum(tw[0]);
@@ -406,7 +413,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_advance(Grid G, Params P, RaySo
 // ============================================================================ re-binning
 
 __global__ void k_scatter(Grid G, RaySoA A, Ctl* ctl, int64_t max_rays, const int* __restrict__ info,
-                          const int4* __restrict__ ccell, const int4* __restrict__ cslot,
+                          const int2* __restrict__ child0, const int4* __restrict__ ccell,
+                            const int4* __restrict__ cslot,
                           const int* __restrict__ newid, const int* __restrict__ off, long long* __restrict__ ent_id,
                           int* __restrict__ ent_src, int* __restrict__ ent_cell)
 {
@@ -422,11 +430,17 @@ __global__ void k_scatter(Grid G, RaySoA A, Ctl* ctl, int64_t max_rays, const in
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int nch = (info[i] >> 4) & 7;
         if (!nch) continue;
-        const int4 cc = ccell[i], sl = cslot[i];
-        const int cs[4] = {cc.x, cc.y, cc.z, cc.w}, ss[4] = {sl.x, sl.y, sl.z, sl.w};
+        const int2 first = child0[i];
+        int cs[4] = {first.x, -1, -1, -1}, ss[4] = {first.y, 0, 0, 0};
+        if (nch > 1) {
+            const int4 cc = ccell[i], sl = cslot[i];
+            cs[1] = cc.y; cs[2] = cc.z; cs[3] = cc.w;
+            ss[1] = sl.y; ss[2] = sl.z; ss[3] = sl.w;
+        }
         const long long pid = __double_as_longlong(A.a[6][i].y);
-        for (int c = 0; c < nch; ++c) {
-            if (cs[c] < 0) continue;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (c >= nch || cs[c] < 0) continue;
             const int64_t pos = (int64_t)off[cs[c]] + ss[c];
             if (pos >= max_rays) continue;
             ent_id[pos] = c == 0 ? pid : with_member(member_of(pid), next + newid[i] + c - 1);
@@ -512,11 +526,13 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_apply(Grid G, Params P, Ray
 // there.  No thread idles on the many empty cells, no per-thread arrays; cell segments are short
 // (a few entries, tens in the launch slab and above the ghost layer), so the count per entry is
 // cheap, and every entry of a warp reads the same few cells.
-__global__ void k_segsort(Grid G, Ctl* ctl, const int* __restrict__ off, const int* __restrict__ off2,
+__global__ void k_segsort(Grid G, Ctl* ctl, CellOffsets cell,
                           const long long* __restrict__ ent_id, const int* __restrict__ ent_src,
                           const int* __restrict__ ent_cell, int* __restrict__ sorted_src)
 {
     if (ctl->status) return;
+    const int* __restrict__ off = cell.before;
+    const int* __restrict__ off2 = cell.live(ctl);
     const int total = off[G.ncell_all];
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
         const int src = ent_src[e];
@@ -548,24 +564,24 @@ __global__ void k_segsort(Grid G, Ctl* ctl, const int* __restrict__ off, const i
 // and K_j^2 (Eq. instability-threshold).
 __global__ void __launch_bounds__(kThreads) k_materialize(Grid G, Params P, RaySoA A, RaySoA B,
                                                             const NodeDF* __restrict__ bg, Ctl* ctl,
-                                                            const int* __restrict__ off2,
-                                                            const int* __restrict__ sorted_src,
+                                                            CellOffsets cell, const int* __restrict__ sorted_src,
                                                             const int* __restrict__ info,
                                                             const int* __restrict__ newid, double* __restrict__ pj,
                                                             double* __restrict__ k2, int* __restrict__ raycell)
 {
     if (ctl->status) return;
-    const int n_new = off2[G.ncell_all];
+    const int n_new = cell.live(ctl)[G.ncell_all];
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->n_new = n_new;   // the live count k_finalize closes the step with
     const int n_old = ctl->n;
     const long long next = ctl->next_id;
-    const int stride = gridDim.x * blockDim.x;
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
+    int64_t p = loop_warp(0, n_new) + (threadIdx.x & 31);
     int src_next = p < n_new ? sorted_src[p] : 0;
-    for (; p < n_new; p += stride) {
+    for (int m = 0; p < n_new; ++m) {
+        const int64_t at = p;
         const int src = src_next;
         // the next source index loaded a pass ahead (the parent's record load waits on it)
-        if (p + stride < n_new) src_next = sorted_src[p + stride];
+        p = loop_warp(m + 1, n_new) + (threadIdx.x & 31);
+        if (p < n_new) src_next = sorted_src[p];
         const int i = src >> 2, c = src & 3;
         if (src < 0 || i >= n_old) {   // inconsistent re-binning: never read past the parents
             set_status(ctl, GWAM_ECUDA);
@@ -576,8 +592,8 @@ __global__ void __launch_bounds__(kThreads) k_materialize(Grid G, Params P, RayS
         load_ray(A, i, s, id);
         make_child(G, s, info[i] & 7, c, ch);
         const long long cid = c == 0 ? id : with_member(member_of(id), next + newid[i] + c - 1);
-        store_ray(B, p, ch, cid);
-        raycell[p] = member_of(id) * G.ncell + cell_of(G, ch);
+        store_ray(B, at, ch, cid);
+        raycell[at] = member_of(id) * G.ncell + cell_of(G, ch);
         if (P.saturation) {
             IntrDF in;
             intrinsic_df(G, bg + (int64_t)member_of(id) * G.ncell, ch, in);
@@ -585,8 +601,8 @@ __global__ void __launch_bounds__(kThreads) k_materialize(Grid G, Params P, RayS
             cell_ijk(G, ch, ci, cj, ck);
             const float2 iv = G.ivol_df[cj * G.nz + ck];
             const DF av = df_mul2(df_split(ray_action(ch)), DF{iv.x, iv.y});
-            pj[p] = df_to_double(df_mul2(df_mul2(df_mul2(in.m2, in.kh2), df_mul2(in.d.iw, in.d.iK2)), av));
-            k2[p] = df_to_double(in.d.K2);
+            pj[at] = df_to_double(df_mul2(df_mul2(df_mul2(in.m2, in.kh2), df_mul2(in.d.iw, in.d.iK2)), av));
+            k2[at] = df_to_double(in.d.K2);
         }
     }
 }
@@ -600,12 +616,12 @@ __global__ void __launch_bounds__(kThreads) k_materialize(Grid G, Params P, RayS
 // skips the many empty cells) and k_sat_kappa sums the listed runs one per lane: the FP64 additions of 32
 // runs share one warp instruction, where a thread per ray left all but the runs' first lanes idle.
 // The list order varies from run to run; every run's sum does not.
-__global__ void __launch_bounds__(kThreads) k_sat_heads(Ctl* ctl, const int* __restrict__ off2, int ncell_all,
+__global__ void __launch_bounds__(kThreads) k_sat_heads(Ctl* ctl, CellOffsets cell, int ncell_all,
                                                           const int* __restrict__ raycell, int* __restrict__ runlist)
 {
     __shared__ int wcount[kThreads / 32], wbase[kThreads / 32];
     if (ctl->status) return;
-    const int n = off2[ncell_all];
+    const int n = cell.live(ctl)[ncell_all];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // one atomic per block and pass: the block's warps take consecutive slices of the list
     for (int p0 = blockIdx.x * blockDim.x; p0 < n; p0 += gridDim.x * blockDim.x) {
@@ -637,10 +653,22 @@ __device__ __forceinline__ void sat_run(int p, int b, int c, const double* __res
                                         const double* __restrict__ pj, const double* __restrict__ k2, double dt,
                                         double* __restrict__ kappa)
 {
+    // four terms at a time, their loads issued before they are added (in order): a run of n terms
+    // waited for n loads one after the other
     double Pc = 0.0, Q = 0.0;
-    for (int q = p; q < b; ++q) {
-        Pc += pj[q];
-        Q += pj[q] * k2[q];
+    for (int q = p; q < b; q += 4) {
+        double a[4], k[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            a[u] = q + u < b ? pj[q + u] : 0.0;
+            k[u] = q + u < b ? k2[q + u] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (q + u < b) {
+                Pc += a[u];
+                Q += a[u] * k[u];
+            }
     }
     // Newton-refined reciprocal instead of an IEEE division (<= 2 ulp; FP64 division is a long
     // instruction sequence at GB300's FP64 rate)
@@ -648,12 +676,13 @@ __device__ __forceinline__ void sat_run(int p, int b, int c, const double* __res
     for (int q = p; q < b; ++q) kappa[q] = kap;
 }
 
-// the listed runs, counted in ctl->n_big (cleared by k_step_begin; k_sat_heads lists them)
-__global__ void k_sat_kappa(const Ctl* ctl, const int* __restrict__ off2, const int* __restrict__ runlist,
+// the listed runs, counted in ctl->n_big (cleared by k_finalize; k_sat_heads lists them)
+__global__ void k_sat_kappa(const Ctl* ctl, CellOffsets cell, const int* __restrict__ runlist,
                             const double* __restrict__ rho, const double* __restrict__ pj,
                             const double* __restrict__ k2, double dt, double* __restrict__ kappa)
 {
     const int nl = ctl->status ? 0 : ctl->n_big;
+    const int* __restrict__ off2 = cell.live(ctl);
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nl; t += gridDim.x * blockDim.x) {
         const int c = runlist[t];
         sat_run(off2[c], off2[c + 1], c, rho, pj, k2, dt, kappa);
@@ -670,7 +699,7 @@ __global__ void k_sat_kappa(const Ctl* ctl, const int* __restrict__ off2, const 
 // Interface fields (z = kk dz, 1 <= kk < nz): staggered-cell overlap, weight w_h * overlap / dz.
 template <bool THETA>
 __global__ void __launch_bounds__(kThreads, THETA ? 3 : 4) k_project(Grid G, Params P, RaySoA B, const NodeDF* __restrict__ bg,
-                                                        const Ctl* ctl, const int* __restrict__ off2,
+                                                        const Ctl* ctl, CellOffsets cell, int* __restrict__ cnt,
                                                         const double* __restrict__ kappa,
                                                         const double* __restrict__ k2, double dt,
                                                         double* __restrict__ fz_l, double* __restrict__ fz_p,
@@ -682,11 +711,14 @@ __global__ void __launch_bounds__(kThreads, THETA ? 3 : 4) k_project(Grid G, Par
                                                         int pstride)
 {
     constexpr int NH = THETA ? 9 : 7;   // centre fields of the segmented sums
-    const int n = ctl->status ? 0 : off2[G.ncell_all];
+    const int n = ctl->status ? 0 : cell.live(ctl)[G.ncell_all];
     double w_sat = 0.0, w_tot = 0.0;
-    const int stride = gridDim.x * blockDim.x;
-    for (int p0 = blockIdx.x * blockDim.x; p0 < n; p0 += stride) {
-        const int p = p0 + threadIdx.x;
+    const int passes = loop_passes(n);
+    for (int m = 0; m < passes; ++m) {
+        clear_ints(cnt, G.ncell_all + 1, m, passes);   // the cells' counters, for the next step
+        const int64_t p0 = loop_warp(m, n);
+        if (p0 >= n) continue;
+        const int p = (int)p0 + (threadIdx.x & 31);
         const bool act = p < n;
         int key = -1;
         DF hv[NH];
@@ -926,38 +958,49 @@ void launch_smooth(Context& c, int nf)
 // ============================================================================ budget, control
 
 // Fold the per-block partials of the slots in `mask` into the budget (a fixed order:
-// deterministic); mode 1 also closes a step (live count, ids, step counter).  One warp per slot,
-// the slots side by side: lane l sums partials l, l + 32, ... of its slot, kFinUnroll loads issued
-// before they are added, then the lane sums by a fixed shuffle tree.  (A block looping over the
-// slots one after another, each ending in a block reduction, chained about 30 memory latencies:
-// 20 us a step.)
-constexpr int kFinUnroll = 16;
-static_assert(NTALLY * 32 <= kThreads, "k_finalize runs one warp per tally slot");
-__global__ void k_finalize(Ctl* ctl, DevBudget* bud, const double* __restrict__ partials, int nb, int mask, int mode)
+// deterministic).  kFinWarps warps per slot, the slots side by side: a lane takes every
+// (32 kFinWarps)-th partial, kFinUnroll loads issued before they are added, then a fixed shuffle tree
+// and the warps' sums in order.  (A block looping over the slots one after another, each ending in a
+// block reduction, chained about 30 memory latencies: 20 us a step; one warp a slot 5.7 us.)
+// Mode 1 also closes a step: live count, ids, step counters, and the step's own counts back to zero;
+// mode 2 closes a launch of `launched[total]` ray volumes.
+constexpr int kFinUnroll = 8;
+constexpr int kFinWarps = 5;
+struct TallyBlocks {
+    int n[NTALLY];   // blocks that wrote a partial
+};
+__global__ void __launch_bounds__(NTALLY * kFinWarps * 32)
+    k_finalize(Ctl* ctl, DevBudget* bud, const double* __restrict__ partials, int stride, TallyBlocks nb, int mask,
+               int mode, const int* launched, int total, int64_t max_rays)
 {
-    __shared__ double acc[NTALLY];
+    __shared__ double sum[NTALLY][kFinWarps];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < NTALLY) {
-        double v = 0.0;
-        if (mask & (1 << w)) {
-            const double* __restrict__ p = partials + (int64_t)w * nb;
-            for (int b0 = 0; b0 < nb; b0 += 32 * kFinUnroll) {
-                double t[kFinUnroll];
+    const int slot = w / kFinWarps, part = w % kFinWarps;
+    double v = 0.0;
+    if (mask & (1 << slot)) {
+        const double* __restrict__ p = partials + (int64_t)slot * stride;
+        const int n = nb.n[slot];
+        for (int b0 = 32 * part + lane; b0 < n; b0 += 32 * kFinWarps * kFinUnroll) {
+            double t[kFinUnroll];
 #pragma unroll
-                for (int u = 0; u < kFinUnroll; ++u) {
-                    const int b = b0 + u * 32 + lane;
-                    t[u] = b < nb ? p[b] : 0.0;
-                }
-#pragma unroll
-                for (int u = 0; u < kFinUnroll; ++u) v += t[u];
+            for (int u = 0; u < kFinUnroll; ++u) {
+                const int b = b0 + u * 32 * kFinWarps;
+                t[u] = b < n ? p[b] : 0.0;
             }
+#pragma unroll
+            for (int u = 0; u < kFinUnroll; ++u) v += t[u];
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) acc[w] = v;
     }
+    if (lane == 0) sum[slot][part] = v;
     __syncthreads();
     if (threadIdx.x != 0) return;
+    double acc[NTALLY];
+    for (int q = 0; q < NTALLY; ++q) {
+        acc[q] = 0.0;
+        for (int u = 0; u < kFinWarps; ++u) acc[q] += sum[q][u];
+    }
     if (mask & (1 << T_EXIT)) bud->w_exited += acc[T_EXIT];
     if (mask & (1 << T_INVALID)) bud->w_invalid += acc[T_INVALID];
     if (mask & (1 << T_CAP)) bud->w_capped += acc[T_CAP];
@@ -968,20 +1011,22 @@ __global__ void k_finalize(Ctl* ctl, DevBudget* bud, const double* __restrict__ 
     }
     if (mask & (1 << T_TOTAL)) bud->w_total = acc[T_TOTAL];
     if (mode == 1) {
+        ctl->ray_steps += ctl->n;
         // after a device failure the population is not trustworthy: drop it (the status stays set)
         ctl->n = ctl->status ? 0 : ctl->n_new;
         ctl->next_id += ctl->new_ids;
         ctl->n_steps += 1;
+        ctl->n_over = 0;
+        ctl->n_big = 0;
+        ctl->n_children = 0;
+        ctl->new_ids = 0;
+    } else if (mode == 2) {
+        const int added = launched ? launched[total] : total;
+        const int64_t n = (int64_t)ctl->n + added;
+        ctl->n = (int)(n > max_rays ? max_rays : n);
+        ctl->next_id += added;
+        ctl->n_launched += added;
     }
-}
-
-__global__ void k_step_begin(Ctl* ctl)
-{
-    ctl->n_over = 0;
-    ctl->n_big = 0;
-    ctl->n_children = 0;
-    ctl->new_ids = 0;
-    ctl->ray_steps += ctl->n;
 }
 
 // ============================================================================ orchestration
@@ -995,9 +1040,24 @@ void smooth_field(Context& c, int f)
     k_smooth<<<blocks, kThreads, 0, c.stream>>>(c.G, c.field[f], c.smooth[f], nlev);
 }
 
-void finalize_tallies(Context& c, int mask, int mode)
+// close a step: the blocks of its tally kernels are those of run_step / run_step32
+void finalize_step(Context& c, int mask)
 {
-    k_finalize<<<1, kThreads, 0, c.stream>>>(c.ctl, c.budget, c.partials, c.max_blocks, mask, mode);
+    TallyBlocks nb{};
+    nb.n[T_EXIT] = nb.n[T_INVALID] = c.lcfg[0].blocks;
+    nb.n[T_CAP] = c.max_blocks;
+    nb.n[T_SAT] = nb.n[T_TOTAL] = c.lcfg[2].blocks;
+    k_finalize<<<1, NTALLY * kFinWarps * 32, 0, c.stream>>>(c.ctl, c.budget, c.partials, c.max_blocks, nb, mask, 1,
+                                                            nullptr, 0, c.max_rays);
+}
+
+// close a launch: launched[total] ray volumes (or, without it, all `total`) by a kernel of `blocks` blocks
+void finalize_launch(Context& c, int blocks, const int* launched, int total)
+{
+    TallyBlocks nb{};
+    nb.n[T_LAUNCH] = blocks;
+    k_finalize<<<1, NTALLY * kFinWarps * 32, 0, c.stream>>>(c.ctl, c.budget, c.partials, c.max_blocks, nb,
+                                                            1 << T_LAUNCH, 2, launched, total, c.max_rays);
 }
 
 void tune_mark(Context& c, int idx)
@@ -1057,51 +1117,47 @@ void run_step(Context& c, double dt, double* du, double* dv)
     const LaunchCfg& la = c.lcfg[0];
     const LaunchCfg& lm = c.lcfg[1];
     const LaunchCfg& lp = c.lcfg[2];
-    k_step_begin<<<1, 1, 0, s>>>(c.ctl);
-    cudaMemsetAsync(c.cnt, 0, sizeof(int) * (size_t)(G.ncell_all + 1), s);
-    cudaMemsetAsync(c.partials, 0, sizeof(double) * NTALLY * (size_t)c.max_blocks, s);
     prof_mark(c, 0);
     tune_mark(c, 0);
-    k_advance<<<la.blocks, la.threads, kAdvanceSmem, s>>>(G, P, c.A, c.bgdf, c.ctl, dt, c.info, c.ccell, c.cslot, c.newid, c.cnt,
+    k_advance<<<la.blocks, la.threads, kAdvanceSmem, s>>>(G, P, c.A, c.bgdf, c.ctl, dt, c.info, c.child0, c.ccell, c.cslot, c.newid, c.cnt,
                                                c.partials, c.max_blocks, clear_set(c));
     tune_mark(c, 1);
     prof_mark(c, 1);
     exclusive_scan2(c, c.newid, c.newid, c.max_rays, &c.ctl->n, c.cnt, c.off, G.ncell_all, nullptr);
-    k_scatter<<<nb, kThreads, 0, s>>>(G, c.A, c.ctl, c.max_rays, c.info, c.ccell, c.cslot, c.newid, c.off, c.ent_id,
+    k_scatter<<<nb, kThreads, 0, s>>>(G, c.A, c.ctl, c.max_rays, c.info, c.child0, c.ccell, c.cslot, c.newid, c.off, c.ent_id,
                                       c.ent_src, c.ent_cell);
     int mask = (1 << T_EXIT) | (1 << T_INVALID) | (1 << T_SAT) | (1 << T_TOTAL);
-    const int* off2 = c.off;
+    const CellOffsets cell{c.off, c.off2};
     if (P.cap > 0) {
         k_cap_find<<<col_blocks, kThreads, 0, s>>>(G, P, c.ctl, c.off, c.overlist);
         k_cap_apply<<<c.max_blocks, kCapThreads, 0, s>>>(G, P, c.A, c.bgdf, c.ctl, c.info, c.off, c.overlist, c.ent_id,
                                                          c.ent_src, c.ent_cell, c.ecap, c.cnt, c.partials, c.max_blocks);
-        exclusive_scan(c, c.cnt, c.off2, G.ncell_all, nullptr);
-        off2 = c.off2;
+        exclusive_scan(c, c.cnt, c.off2, G.ncell_all, nullptr, &c.ctl->n_over);
         mask |= 1 << T_CAP;
     }
-    k_segsort<<<nb, kThreads, 0, s>>>(G, c.ctl, c.off, off2, c.ent_id, c.ent_src, c.ent_cell, c.sorted_src);
+    k_segsort<<<nb, kThreads, 0, s>>>(G, c.ctl, cell, c.ent_id, c.ent_src, c.ent_cell, c.sorted_src);
     tune_mark(c, 2);
-    k_materialize<<<lm.blocks, lm.threads, 0, s>>>(G, P, c.A, c.B, c.bgdf, c.ctl, off2, c.sorted_src, c.info, c.newid,
+    k_materialize<<<lm.blocks, lm.threads, 0, s>>>(G, P, c.A, c.B, c.bgdf, c.ctl, cell, c.sorted_src, c.info, c.newid,
                                                    c.pj, c.k2, c.raycell);
     tune_mark(c, 3);
     prof_mark(c, 2);
     if (P.saturation) {
         // both saturation passes on the largest grid (eight blocks per SM, all resident): shorter
         // chains of per-block passes (saturation 0.070 -> 0.060 ms on the 512 x 256 sphere)
-        k_sat_heads<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, off2, G.ncell_all, c.raycell, c.biglist);
-        k_sat_kappa<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, off2, c.biglist, c.rho, c.pj, c.k2, dt, c.kappa);
+        k_sat_heads<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, cell, G.ncell_all, c.raycell, c.biglist);
+        k_sat_kappa<<<c.max_blocks, kThreads, 0, s>>>(c.ctl, cell, c.biglist, c.rho, c.pj, c.k2, dt, c.kappa);
     }
     prof_mark(c, 3);
     // (the projected fields were cleared by k_advance)
     tune_mark(c, 4);
     if (P.theta_flux)
-        k_project<true><<<lp.blocks, lp.threads, 0, s>>>(G, P, c.B, c.bgdf, c.ctl, off2, c.kappa, c.k2, dt,
+        k_project<true><<<lp.blocks, lp.threads, 0, s>>>(G, P, c.B, c.bgdf, c.ctl, cell, c.cnt, c.kappa, c.k2, dt,
                                                          c.field[F_ZL], c.field[F_ZP], c.field[F_LL], c.field[F_LP],
                                                          c.field[F_PL], c.field[F_PP], c.field[F_EL], c.field[F_EP],
                                                          c.field[F_WAD], c.field[F_TL], c.field[F_TP], c.partials,
                                                          c.max_blocks);
     else
-        k_project<false><<<lp.blocks, lp.threads, 0, s>>>(G, P, c.B, c.bgdf, c.ctl, off2, c.kappa, c.k2, dt,
+        k_project<false><<<lp.blocks, lp.threads, 0, s>>>(G, P, c.B, c.bgdf, c.ctl, cell, c.cnt, c.kappa, c.k2, dt,
                                                           c.field[F_ZL], c.field[F_ZP], c.field[F_LL], c.field[F_LP],
                                                           c.field[F_PL], c.field[F_PP], c.field[F_EL], c.field[F_EP],
                                                           c.field[F_WAD], nullptr, nullptr, c.partials, c.max_blocks);
