@@ -3,6 +3,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "gwam_df.cuh"
 #include "gwam_gemm.cuh"
@@ -27,16 +28,25 @@ __device__ __forceinline__ uint64_t gtime()
 
 // bounded wait for completion of the mbarrier phase with the given parity; false if it gave up
 // (after limit_ns of %globaltimer time, or 2^31 polls)
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit_ns)
 {
     uint64_t t0 = 0;
     for (uint32_t it = 0; it < 0x7fffffffu; ++it) {
         uint32_t done;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
+        if (CLUSTER)   // arrivals of another CTA of the cluster
+            asm volatile(
+                "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+                " selp.u32 %0, 1, 0, p;\n}"
+                : "=r"(done)
+                : "r"(bar), "r"(parity)
+                : "memory");
+        else
+            asm volatile(
+                "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                : "=r"(done)
+                : "r"(bar), "r"(parity)
+                : "memory");
         if (done) return true;
         if ((it & 63u) == 0) {
             const uint64_t t = gtime();
@@ -96,12 +106,20 @@ __device__ __forceinline__ float erf_abs(float z, float& e)
 }
 
 // GELU(z) = z Phi(z) = z / 2 + |z| erf(|z| / sqrt 2) / 2
-__device__ __forceinline__ float gelu(float z)
+// GELU of two values, z (1 + erf(z / sqrt 2)) / 2, in packed instructions (half the issue slots); the steps
+// of erf_abs, with the polynomial's coefficients negated for its negated value.
+__device__ __forceinline__ float2 gelu2(float2 z)
 {
-    float e;
-    const float r = erf_abs(z, e);
-    const float h = 0.5f * z;
-    return fmaf(fabsf(h), r, h);
+    const float2 az = make_float2(fabsf(z.x), fabsf(z.y));
+    const float2 d = fma2(dup2(0.23164189961f), az, dup2(1.0f));
+    const float2 t = make_float2(rcp_approx(d.x), rcp_approx(d.y));
+    float2 p = fma2(t, dup2(-1.061405429f), dup2(1.453152027f));
+    p = fma2(t, p, dup2(-1.421413741f));
+    p = fma2(t, p, dup2(0.284496736f));
+    p = fma2(t, p, dup2(-0.254829592f));
+    const float2 q = mul2(mul2(z, z), dup2(-0.72134752044f));
+    const float2 r = fma2(mul2(t, p), make_float2(ex2_approx(q.x), ex2_approx(q.y)), dup2(1.0f));
+    return fma2(mul2(az, dup2(0.5f)), r, mul2(z, dup2(0.5f)));
 }
 
 // GELU'(z) = Phi(z) + z phi(z), phi(z) = exp(-z^2 / 2) / sqrt(2 pi)
@@ -112,13 +130,13 @@ __device__ __forceinline__ float gelu_grad(float z)
     return fmaf(z * 0.39894228040143268f, e, fmaf(0.5f, copysignf(r, z), 0.5f));
 }
 
-// Epilogue of 32 consecutive accumulator columns n = nb .. nb+31 of one row.  Per-column
-// parameters arrive one per lane (lane j holds column nb + j) and are broadcast with shuffles, so
-// every lane of the warp must call this (rows >= M only skip the stores).  zz: the prefetched
+// Epilogue of 32 consecutive accumulator columns n = nb .. nb+31 of one row.  Per-column parameters come
+// from shared memory (sbias: the bias of npad columns; EPI_DRAG: then sigma and mu).  Rows >= M only skip
+// the stores.  zz: the prefetched
 // pre-activations of EPI_BWD.
 template <int MODE>
 __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, float (&v)[32], const float* sbias,
-                                      float ps, float pm, const float (&zz)[32], int rowmask, gwam::DF& sq,
+                                      int npad, const float (&zz)[32], int rowmask, gwam::DF& sq,
                                       uint32_t stg, int cc0)
 {
     const bool live = row < e.M;
@@ -143,14 +161,21 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
             // de-normalised in FP32 (one FMA, relative error 6e-8, far below the BF16 network's) and
             // widened exactly by integer operations: FP64 arithmetic and float -> double conversions
             // run at 1/64 of the FP32 rate on GB300
+            if (!live || rowmask != 0) return;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float sj = __shfl_sync(0xffffffffu, ps, j), mj = __shfl_sync(0xffffffffu, pm, j);
-                const int n = nb + j;
-                if (live && rowmask == 0 && n < e.n_true) {
-                    const double y = gwam::widen(__fmaf_rn(v[j], sj, mj));
-                    if (n < e.nlev) e.du[(size_t)n * e.ncol + row] = y;
-                    else e.dv[(size_t)(n - e.nlev) * e.ncol + row] = y;
+            for (int j = 0; j < 32; j += 4) {
+                // sigma and mu behind the bias in shared memory, broadcast four at a time
+                const float4 s4 = *reinterpret_cast<const float4*>(sbias + npad + nb + j);
+                const float4 m4 = *reinterpret_cast<const float4*>(sbias + 2 * npad + nb + j);
+                const float sj[4] = {s4.x, s4.y, s4.z, s4.w}, mj[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int n = nb + j + u;
+                    if (n < e.n_true) {
+                        const double y = gwam::widen(__fmaf_rn(v[j + u], sj[u], mj[u]));
+                        if (n < e.nlev) e.du[(size_t)n * e.ncol + row] = y;
+                        else e.dv[(size_t)(n - e.nlev) * e.ncol + row] = y;
+                    }
                 }
             }
             return;
@@ -171,7 +196,11 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
             }
             if (e.act) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) v[j] = gelu(v[j]);
+                for (int j = 0; j < 32; j += 2) {
+                    const float2 g = gelu2(make_float2(v[j], v[j + 1]));
+                    v[j] = g.x;
+                    v[j + 1] = g.y;
+                }
             }
         } else {  // EPI_LOSS
             if (e.cf) {
@@ -350,9 +379,15 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     // (the set-up above touched only shared and tensor memory and the kernel parameters)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int npad = (e.N + 31) & ~31;
     if (e.bias) {
-        const int npad = (e.N + 31) & ~31;
-        for (int i = tid; i < npad; i += blockDim.x) sbias[i] = i < e.N ? e.bias[i] : 0.0f;
+        for (int i = tid; i < npad; i += blockDim.x) {
+            sbias[i] = i < e.N ? e.bias[i] : 0.0f;
+            if (MODE == EPI_DRAG) {
+                sbias[npad + i] = i < e.n_true ? e.ysig[i] : 0.0f;
+                sbias[2 * npad + i] = i < e.n_true ? e.ymu[i] : 0.0f;
+            }
+        }
     }
     tc_before();
     __syncthreads();
@@ -465,14 +500,6 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
             const int m0 = (r / n_tiles) * kBM, n0 = (r % n_tiles) * BN;
             const int row = m0 + q * 32 + lane;
             const int cbeg = n0 + part * kColsPerWarp;
-            // de-normalisation of this warp's columns, one per lane, fetched before the wait
-            float ps[kChunks], pm[kChunks];
-#pragma unroll
-            for (int k = 0; k < kChunks; ++k) {
-                const int n = cbeg + 32 * k + lane;
-                ps[k] = (MODE == EPI_DRAG && n < e.n_true) ? e.ysig[n] : 0.0f;
-                pm[k] = (MODE == EPI_DRAG && n < e.n_true) ? e.ymu[n] : 0.0f;
-            }
             const int rowmask = (MODE == EPI_DRAG && row < e.M) ? e.mask[row] : 0;
             const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((tl / 2) & 1), wlim);
             if (!__all_sync(0xffffffffu, got) || abort_flag) {
@@ -522,15 +549,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rr[j]);
                 const uint32_t stg =
                     e.tstore ? stg_warp + (uint32_t)((32 * k) / 64) * 4096u + (uint32_t)lane * 128u : 0u;
-                // this chunk's de-normalisation, selected rather than indexed (stays in registers)
-                float psk = ps[0], pmk = pm[0];
-#pragma unroll
-                for (int u = 1; u < kChunks; ++u)
-                    if (k == u) {
-                        psk = ps[u];
-                        pmk = pm[u];
-                    }
-                epi32<MODE>(e, z, row, nb, v, sbias, psk, pmk, zz, rowmask, sq, stg, ((32 * k) % 64) / 8);
+                epi32<MODE>(e, z, row, nb, v, sbias, npad, zz, rowmask, sq, stg, ((32 * k) % 64) / 8);
             }
             tc_before();
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&acce_bar[acc])) : "memory");
@@ -569,6 +588,296 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     if (!__syncthreads_and(ok && fin) && tid == 0 && e.err) atomicOr(e.err, 1);
     tc_after();
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
+}
+
+// All hidden layers of the inference (gemm_hidden_launch).  Layer by layer in k_gemm_bf16 a layer of
+// 32 768 x 512 x 512 reads 197 MB from L2 (8 TB/s) and takes 26 us where the tensor cores need 9.  Here a
+// cluster of C = N / 128 CTAs owns the same rows through all layers, so that a layer needs nothing from other
+// clusters and the layers follow one another without a launch between them.  Two CTAs are a pair
+// (cta_group::2): 256 rows x 256 columns a tile, each CTA holding its 128 rows of A and 128 of the pair's 256
+// rows of W, half of the shared-memory reads that the tile would cost one CTA.  W stays in shared memory
+// through a layer (blocks of the next one replace it as the last tile releases them): 94 MB a layer.
+// Inference of 32 768 columns through 4 x 512: 121 us, 137 layer by layer.  What bounds it: a tile takes 5 us,
+// of them 3.6 the round trips of the four A stages that fit beside W (without any epilogue), the rest
+// the epilogue and the wait for the previous layer's stores; multicast of A between the pairs changed nothing.
+//
+// Warps as in k_gemm_bf16, sixteen of them epilogue (eight: 12 us more).  full, in the pair's first CTA: A (and
+// in a layer's first tile W) of a stage has landed in both CTAs; empty: the MMAs have released the stage;
+// accf, acce: the accumulator is complete, drained by both CTAs.  done[w]: tiles that an epilogue warp of this
+// CTA (or of its counterpart in the other pair) has finished writing to global memory, which the next layer's
+// loads wait for.  Every wait is bounded; a CTA that gives up still meets the others at the end.
+constexpr int kHidStages = 4;
+constexpr int kHidMaxK = 512;
+constexpr int kHidEpi = 16;                          // epilogue warps
+constexpr uint32_t kHidStgWarp = 32u * 32u * 2u;
+
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, int rank)
+{
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int C>
+__global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_constant__ HiddenSet h, int M, int* err)
+{
+    constexpr int kRows = 2 * kBM, kStages = kHidStages;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], accf_bar[2], acce_bar[2], done_bar;
+    __shared__ uint32_t done[kHidEpi * C / 2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_flag;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x % C, cluster = blockIdx.x / C, clusters = gridDim.x / C;
+    const int pair = rank >> 1, half = rank & 1, lead = rank & ~1;
+    const int tiles = ((M + kRows - 1) / kRows - cluster + clusters - 1) / clusters;   // >= 1 of this cluster
+    // W (up to 8 blocks of 16 KB), A stages, staging boxes of the epilogue warps
+    const uint32_t wbase = (saddr(smem_raw) + 1023u) & ~1023u;
+    const uint32_t abase = wbase + (kHidMaxK / kBK) * kABytes, sbase = abase + kStages * kABytes;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&full_bar[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&empty_bar[s])));
+        }
+        for (int a = 0; a < 2; ++a) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&accf_bar[a])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(&acce_bar[a])), "r"(2 * kHidEpi));
+        }
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&done_bar)));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        abort_flag = 0;
+    }
+    if (tid < kHidEpi * C / 2) done[tid] = 0u;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(saddr(&tmem_slot)));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+    }
+    tc_before();
+    __syncthreads();
+    cluster_sync();
+    tc_after();
+    const uint32_t tmem = tmem_slot;
+    // a 64 x 128 box of W or A; its bytes are counted by the barrier of the pair's first CTA
+    auto load = [](uint32_t dst, const CUtensorMap& map, int x, int y, uint32_t bar) {
+        asm volatile(
+            "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, "
+            "%3}], [%4];" ::"r"(dst),
+            "l"(reinterpret_cast<uint64_t>(&map)), "r"(x), "r"(y), "r"(bar)
+            : "memory");
+    };
+    auto expect = [&](int s, uint32_t bytes) {
+        if (half == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(&full_bar[s])), "r"(bytes) : "memory");
+    };
+    // the first blocks of W, while the previous kernel still runs
+    const int pre = min(kStages, h.nk[0]);
+    if (tid == 0)
+        for (int i = 0; i < pre; ++i) {
+            expect(i, 4 * kABytes);
+            load(wbase + (uint32_t)i * kABytes, h.b[0], i * kBK, rank * 128, cluster_addr(saddr(&full_bar[i]), lead));
+        }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    bool ok = true;
+
+    if (warp == 0) {
+        int it = 0;
+        for (int l = 0; l < h.n && ok; ++l) {
+            const int nk = h.nk[l], nkp = l ? h.nk[l - 1] : kStages;
+            for (int j = 0; j < tiles && ok; ++j) {
+                if (l > 0) {
+                    // this tile's rows of the previous layer are in global memory
+                    const uint32_t want = (uint32_t)((l - 1) * tiles + j + 1);
+                    uint64_t t0 = 0;
+                    for (;;) {
+                        uint32_t v = want;
+                        if (lane < kHidEpi * C / 2)
+                            asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(saddr(&done[lane])) : "memory");
+                        if (__all_sync(0xffffffffu, v >= want)) break;
+                        const uint64_t t = __shfl_sync(0xffffffffu, gtime(), 0);
+                        if (t0 == 0) t0 = t;
+                        else if (t - t0 > kWaitNs) {
+                            ok = false;
+                            break;
+                        }
+                    }
+                    if (!ok) break;
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                }
+                if (lane == 0) {
+                    const int row = (cluster + j * clusters) * kRows + half * kBM;
+                    for (int i = 0; i < nk; ++i) {
+                        const int q = it + i, s = q % kStages, p = q - nkp;
+                        const uint32_t fb = cluster_addr(saddr(&full_bar[s]), lead);
+                        if ((q >= kStages && !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((q / kStages - 1) & 1), kWaitNs)) ||
+                            // the block of W that this one replaces may be read by a later stage than that
+                            (l > 0 && j == 0 && nkp < kStages && i < nkp &&
+                             !mbar_wait(saddr(&empty_bar[p % kStages]), (uint32_t)((p / kStages) & 1), kWaitNs)) ||
+                            abort_flag) {
+                            ok = false;
+                            break;
+                        }
+                        if (j > 0) expect(s, 2 * kABytes);
+                        else if (l > 0 || i >= pre) {
+                            expect(s, 4 * kABytes);
+                            load(wbase + (uint32_t)i * kABytes, h.b[l], i * kBK, rank * 128, fb);
+                        }
+                        load(abase + (uint32_t)s * kABytes, h.a[l], i * kBK, row, fb);
+                    }
+                }
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                it += nk;
+            }
+        }
+        if (lane == 0) {
+            if (!ok) abort_flag = 1;
+            // the last stages' copies have landed and their release has arrived
+            for (int i = it > kStages ? it - kStages : 0; i < it && ok; ++i)
+                ok = mbar_wait(saddr(&empty_bar[i % kStages]), (uint32_t)((i / kStages) & 1), kWaitNs);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (lane == 0 && half == 0) {
+            constexpr uint32_t idesc = idesc_bf16(kRows, 256);
+            auto commit = [](uint64_t* bar, uint16_t mask) {
+                asm volatile(
+                    "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+                        saddr(bar)),
+                    "h"(mask)
+                    : "memory");
+            };
+            const uint16_t mine = (uint16_t)(3u << lead);
+            int it = 0, tl = 0;
+            for (int l = 0; l < h.n && ok; ++l) {
+                const int nk = h.nk[l];
+                for (int j = 0; j < tiles && ok; ++j, ++tl) {
+                    const int acc = tl & 1;
+                    if (tl >= 2 && !mbar_wait<true>(saddr(&acce_bar[acc]), (uint32_t)((tl / 2 - 1) & 1), kWaitNs)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_after();
+                    for (int i = 0; i < nk; ++i, ++it) {
+                        const int s = it % kStages;
+                        const uint32_t ph = (uint32_t)((it / kStages) & 1);
+                        if (abort_flag || !mbar_wait<true>(saddr(&full_bar[s]), ph, kWaitNs)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_after();
+                        const uint32_t a0 = abase + (uint32_t)s * kABytes, b0 = wbase + (uint32_t)i * kABytes;
+#pragma unroll
+                        for (int kk = 0; kk < kBK / 16; ++kk) {
+                            const uint64_t ad = desc_sw128(a0 + 32u * kk), bd = desc_sw128(b0 + 32u * kk);
+                            const uint32_t accum = (i > 0 || kk > 0) ? 1u : 0u;
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)acc * 256u),
+                                "l"(ad), "l"(bd), "r"(idesc), "r"(accum)
+                                : "memory");
+                        }
+                        commit(&empty_bar[s], mine);
+                    }
+                    if (!ok) break;
+                    commit(&accf_bar[acc], mine);
+                }
+            }
+            if (!ok) abort_flag = 1;
+            commit(&done_bar, mine);
+        }
+        __syncwarp();
+    } else {
+        // epilogue: 32 rows x 64 columns a warp and tile
+        const int w = warp - 2, q = warp & 3, part = w >> 2;
+        const uint32_t stg = sbase + (uint32_t)w * kHidStgWarp;
+        const uint32_t slot = saddr(&done[kHidEpi * pair + w]);
+        auto finished = [&](int n) {   // lane 0: the first n tiles of this warp are written
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+            asm volatile("fence.acq_rel.cluster;" ::: "memory");
+            asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(slot, rank)), "r"(n) : "memory");
+            if (C == 4)
+                asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr(slot, rank ^ 2)), "r"(n)
+                             : "memory");
+        };
+        const int n0 = pair * 256 + part * 64;
+        int tl = 0;
+        for (int l = 0; l < h.n && ok; ++l) {
+            const float4* bias = reinterpret_cast<const float4*>(h.bias[l] + n0);
+            for (int j = 0; j < tiles; ++j, ++tl) {
+                const int acc = tl & 1, row0 = (cluster + j * clusters) * kRows + half * kBM + q * 32;
+                const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((tl / 2) & 1), kWaitNs);
+                if (!__all_sync(0xffffffffu, got) || abort_flag) {
+                    ok = false;
+                    break;
+                }
+                tc_after();
+                if (lane == 0) finished(tl);
+                const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * 256 + part * 64);
+#pragma unroll 1
+                for (int b = 0; b < 2; ++b) {
+                    uint32_t rr[32];
+                    tmem_ld32(tacc + (uint32_t)(32 * b), rr);
+                    // the first box has been read from the staging memory
+                    if (b == 1 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                    __syncwarp();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t o[4];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const float4 bb = __ldg(bias + 8 * b + 2 * c + u);
+                            const uint32_t* r = rr + 8 * c + 4 * u;
+                            const float2 g0 = gelu2(add2(make_float2(__uint_as_float(r[0]), __uint_as_float(r[1])), make_float2(bb.x, bb.y)));
+                            const float2 g1 = gelu2(add2(make_float2(__uint_as_float(r[2]), __uint_as_float(r[3])), make_float2(bb.z, bb.w)));
+                            const __nv_bfloat162 p0 = __floats2bfloat162_rn(g0.x, g0.y), p1 = __floats2bfloat162_rn(g1.x, g1.y);
+                            o[2 * u] = *reinterpret_cast<const uint32_t*>(&p0);
+                            o[2 * u + 1] = *reinterpret_cast<const uint32_t*>(&p1);
+                        }
+                        // 64-byte-swizzled box: 16-byte chunk c of row r at r * 64 + ((c ^ (r / 2 % 4)) * 16)
+                        const uint32_t a = stg + (uint32_t)lane * 64u + ((uint32_t)(c ^ ((lane >> 1) & 3)) << 4);
+                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                                     "r"(o[3])
+                                     : "memory");
+                    }
+                    if (b == 1) tc_before();
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (row0 < M)
+                            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                                             reinterpret_cast<uint64_t>(&h.c[l])),
+                                         "r"(n0 + 32 * b), "r"(row0), "r"(stg)
+                                         : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                }
+                if (lane == 0) {
+                    arrive_cluster(cluster_addr(saddr(&acce_bar[acc]), lead));
+                    // with one or two tiles a layer the next layer's loads are due before the next tile's epilogue
+                    if (tiles <= 2) finished(tl + 1);
+                }
+                __syncwarp();
+            }
+        }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        __syncwarp();
+        if (!ok) abort_flag = 1;
+    }
+    const bool fin = mbar_wait(saddr(&done_bar), 0u, kWaitNs);
+    if (!__syncthreads_and(ok && fin) && tid == 0 && err) atomicOr(err, 1);
+    tc_before();
+    cluster_sync();   // nobody reads the accumulators or writes to another CTA's shared memory any more
+    tc_after();
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+    cluster_sync();
 }
 
 // Weight gradients and weight updates of all layers (GradSet), the roles of the warps as in k_gemm_bf16:
@@ -836,7 +1145,7 @@ bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap
     constexpr size_t kMaxShm = 232448 - 256;   // 227 KB opt-in per block, less the static part
     constexpr size_t kStg = (size_t)32 * BN / (EPW / 4) * 2 * EPW;
     const size_t shm = (size_t)ST * (kABytes + BN * kBK * 2) + 1024 + (e.tstore ? kStg : 0) +
-                       (e.bias ? (size_t)((e.N + 31) & ~31) * 4 : 0);
+                       (e.bias ? (size_t)((e.N + 31) & ~31) * 4 * (MODE == EPI_DRAG ? 3 : 1) : 0);
     if (shm > kMaxShm) return false;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -897,18 +1206,20 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 
 }  // namespace
 
-bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows)
+bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t box_rows,
+                    uint32_t box_cols)
 {
     auto fn = encode_fn();
     if (!fn || !map || !base || rows == 0 || cols == 0 || ld < cols || (ld * 2) % 16 || box_rows == 0 ||
-        box_rows > 256 || (reinterpret_cast<uintptr_t>(base) & 15))
+        box_rows > 256 || (box_cols != 64 && box_cols != 32) || (reinterpret_cast<uintptr_t>(base) & 15))
         return false;
     const cuuint64_t dims[2] = {cols, rows};
     const cuuint64_t strides[1] = {ld * 2};
-    const cuuint32_t box[2] = {64, box_rows};
+    const cuuint32_t box[2] = {box_cols, box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -940,6 +1251,77 @@ int gemm_pick_bn(int M, int N)
         }
     }
     return best;
+}
+
+namespace {
+
+constexpr size_t kHidSmem = (size_t)(kHidMaxK / kBK + kHidStages) * kABytes + kHidEpi * kHidStgWarp + 1024;
+
+template <int C>
+cudaLaunchConfig_t hidden_config(int clusters, cudaLaunchAttribute (&attr)[2], cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(clusters * C));
+    cfg.blockDim = dim3(64 + 32 * kHidEpi);
+    cfg.dynamicSmemBytes = kHidSmem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+// clusters of C CTAs that can be resident at once (0: the kernel cannot run)
+template <int C>
+int hidden_clusters()
+{
+    static std::atomic<int> n[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 0;
+    if (!n[dev]) {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = hidden_config<C>(1, attr, nullptr);
+        cfg.numAttrs = 1;
+        int c = 0;
+        if (cudaFuncSetAttribute(k_hidden<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHidSmem) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&c, k_hidden<C>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            c = 0;
+        }
+        n[dev] = c > 0 ? c : -1;
+    }
+    return std::max(n[dev].load(), 0);
+}
+
+template <int C>
+bool hidden_launch(const HiddenSet& h, int M, int* err, cudaStream_t s)
+{
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = hidden_config<C>(std::min(hidden_clusters<C>(), (M + 2 * kBM - 1) / (2 * kBM)), attr, s);
+    return cudaLaunchKernelEx(&cfg, k_hidden<C>, h, M, err) == cudaSuccess;
+}
+
+}  // namespace
+
+bool gemm_hidden_fits(int M, int N, int K0)
+{
+    if ((N != 256 && N != 512) || M < 1 || K0 < kBK || K0 > kHidMaxK || K0 % kBK) return false;
+    // With fewer row tiles than 0.6 of the clusters the smaller tiles of k_gemm_bf16 spread better over the SMs
+    // (4 x 512: 5000 rows 53.7 us here, 53.1 there; 9000 rows 58 and 63; 18 000 rows 74 and 89; 4 x 256: 9500
+    // rows 50 and 47, 12 000 rows 59 and 62; the whole inference each time).
+    const int clusters = N == 256 ? hidden_clusters<2>() : hidden_clusters<4>();
+    return clusters > 0 && 5LL * ((M + 2 * kBM - 1) / (2 * kBM)) >= 3LL * clusters;
+}
+
+bool gemm_hidden_launch(const HiddenSet& h, int M, int N, int* err, cudaStream_t s)
+{
+    if (h.n < 1 || h.n > kHiddenMax || !gemm_hidden_fits(M, N, h.nk[0] * kBK)) return false;
+    return N == 256 ? hidden_launch<2>(h, M, err, s) : hidden_launch<4>(h, M, err, s);
 }
 
 bool gemm_bf16_grad_launch(GradSet& g, int K, int* err, cudaStream_t s)

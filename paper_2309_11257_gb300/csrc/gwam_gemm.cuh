@@ -62,9 +62,9 @@ struct GemmEpi {
 };
 
 // 2-D BF16 tensor map of a row-major [rows][cols] matrix with leading dimension ld (elements),
-// box = 64 columns x box_rows rows, 128-byte swizzle.  false if the driver refuses it.
+// box = box_cols (64, or 32) columns x box_rows rows, swizzled over 128 (64) bytes.  false if the driver refuses it.
 bool make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
-                    uint32_t box_rows);
+                    uint32_t box_rows, uint32_t box_cols = 64);
 
 // One Adam update (Kingma & Ba 2015) of a parameter w with gradient g; returns the new value
 struct Adam {
@@ -103,6 +103,21 @@ bool gemm_bf16_grad_launch(GradSet& set, int K, int* err, cudaStream_t s);
 // shape.
 bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ksplit,
                       const GemmEpi& e, cudaStream_t s);
+
+// All hidden layers of the inference, act_l = GELU(act_(l-1) . W_l^T + bias_l) in BF16, in one kernel with the
+// weights in shared memory: N = 256 or 512 outputs a layer, 64 nk <= 512 inputs.  a: act_(l-1) and
+// b: W_l with box rows 128; c: act_l in boxes of 32 rows x 32 columns.  The kernel reads the weights
+// before the previous kernel of the stream has completed (programmatic dependent launch): they must be
+// older than that.  gemm_hidden_fits says whether M rows should run here rather than layer by layer.
+constexpr int kHiddenMax = 8;
+struct HiddenSet {
+    CUtensorMap a[kHiddenMax], b[kHiddenMax], c[kHiddenMax];
+    const float* bias[kHiddenMax];
+    int nk[kHiddenMax];
+    int n;
+};
+bool gemm_hidden_fits(int M, int N, int K0);
+bool gemm_hidden_launch(const HiddenSet& h, int M, int N, int* err, cudaStream_t s);
 
 // The tile width gemm_bf16_launch uses when bn = 0 (the caller builds tb with this box): the one with
 // the least waves x (width + 48) over the GPU's SMs -- a tile's time grows with its width, 48 columns

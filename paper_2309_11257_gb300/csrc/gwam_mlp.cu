@@ -136,9 +136,9 @@ __global__ void __launch_bounds__(256) k_bias_update(const __grid_constant__ Bia
     if (u.adam.lr > 0.0f && o < u.n_o[q]) u.b[q][o] = u.adam(u.b[q][o], g, u.mb[q][o], u.vb[q][o]);
 }
 
-// launch with programmatic stream serialisation (the kernel begins with pdl_enter)
+// launch with programmatic stream serialisation (the kernel begins with pdl_enter), if early is set
 template <class... P, class... A>
-bool launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args)
+bool launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, bool early, A... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -146,7 +146,7 @@ bool launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... arg
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = early;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k, args...) == cudaSuccess;
@@ -318,6 +318,7 @@ struct gwam_mlp {
     CUtensorMap tf_a[kMaxL + 1], tx_a[kMaxL + 1], tw_a[kMaxL + 1], tw_b[kMaxL + 1];
     CUtensorMap tf_b[kMaxL + 1][4], tx_b[kMaxL + 1][4];   // by tile width (64, 128, 192, 256)
     CUtensorMap to_act[kMaxL + 1], to_dz[kMaxL + 1];      // BF16 outputs written by TMA stores
+    gwam::HiddenSet hidden{};
     std::vector<void*> allocs;
     std::string last_error;
     // inference timing: events before the pack kernel, before the first GEMM, after the last GEMM
@@ -428,7 +429,11 @@ bool gemm(gwam_mlp* m, const CUtensorMap& ta, const CUtensorMap& tb, const CUten
 // forward through every layer for B rows of act[0]; last layer per `last`
 bool forward(gwam_mlp* m, int B, bool train, const gwam::GemmEpi& last)
 {
-    for (int l = 1; l < m->nl; ++l) {
+    // (inference only: a training step's weights may still be in the making when its forward pass is
+    // launched, and it needs more than the activations)
+    const bool fused = !train && m->nl > 1 && gwam::gemm_hidden_fits(B, m->D[1], m->D[0]);
+    if (fused && !gwam::gemm_hidden_launch(m->hidden, B, m->D[1], m->err, m->s)) return false;
+    for (int l = 1; l < m->nl && !fused; ++l) {
         gwam::GemmEpi e{};
         e.mode = gwam::EPI_STORE;
         e.act = 1;
@@ -516,9 +521,17 @@ int gwam_mlp_create(gwam_mlp** out, const gwam_mlp_config* cfg, void* stream)
              gwam::make_tmap_bf16(&m->tw_b[l], m->actT[l - 1], Di, Bm, Bm, gwam::kGradBN) &&
              gwam::make_tmap_bf16(&m->to_dz[l], m->dz[l], Bm, Do, Do, 32) &&
              (l == m->nl || gwam::make_tmap_bf16(&m->to_act[l], m->act[l], Bm, Do, Do, 32));
+        if (l < m->nl) {
+            ok = ok && gwam::make_tmap_bf16(&m->hidden.c[l - 1], m->act[l], Bm, Do, Do, 32, 32);
+            m->hidden.a[l - 1] = m->tf_a[l];
+            m->hidden.bias[l - 1] = m->b[l];
+            m->hidden.nk[l - 1] = Di / 64;
+            m->hidden.n = l;
+        }
         for (int w = 0; w < 4 && ok; ++w)
             ok = gwam::make_tmap_bf16(&m->tf_b[l][w], m->Wb[l], Do, Di, Di, 64 * (w + 1)) &&
                  gwam::make_tmap_bf16(&m->tx_b[l][w], m->WbT[l], Di, Do, Do, 64 * (w + 1));
+        if (l < m->nl) m->hidden.b[l - 1] = m->tf_b[l][1];
     }
     if (!ok) {
         gwam_mlp_destroy(m);
@@ -665,7 +678,7 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
     if (!m->has_norm) return fail(m, GWAM_ESTATE, "normalisation not set");
     const int B = batch, L = m->nl, Dn = m->D[L];
     cudaMemsetAsync(m->loss, 0, 2 * sizeof(double), m->s);   // and err
-    bool ok = launch_pdl(k_batch, dim3((m->D[0] + Dn) / 32, B / 32), dim3(32, 8), m->s, X, Y, n, m->N[0], m->D[0],
+    bool ok = launch_pdl(k_batch, dim3((m->D[0] + Dn) / 32, B / 32), dim3(32, 8), m->s, true, X, Y, n, m->N[0], m->D[0],
                          m->N[L], Dn, rows, seed, (const float*)m->xmu, (const float*)m->xisig, (const float*)m->ymu,
                          (const float*)m->yisig, m->act[0], m->actT[0], m->max_batch, m->T, m->err);
     gwam::GemmEpi last{};
@@ -733,7 +746,7 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
         u.B = B;
         g.adam = u.adam = adam;
         ok = gwam::gemm_bf16_grad_launch(g, B, m->err, m->s) &&
-             launch_pdl(k_bias_update, dim3((outputs + 7) / 8), dim3(256), m->s, u);
+             launch_pdl(k_bias_update, dim3((outputs + 7) / 8), dim3(256), m->s, true, u);
     }
     if (!ok || cudaPeekAtLastError() != cudaSuccess) return fail(m, GWAM_ECUDA, "kernel launch failed");
     if (lr > 0) ++m->t;
@@ -777,7 +790,8 @@ int gwam_mlp_infer(gwam_mlp* m, const float* X, int64_t ncol, double* dudt, doub
         const int rows = (int)std::min<int64_t>(m->max_batch, ncol - c0);
         if (m->prof && m->prof_used + 3 > 3 * 64) prof_harvest(m);
         if (m->prof) prof_mark(m);
-        if (!launch_pdl(k_pack_infer, dim3((rows + 7) / 8), dim3(256), m->s, X, ncol, c0, rows, m->N[0], m->D[0],
+        // the first one waits for all that came before it: the layers read the weights ahead of their turn
+        if (!launch_pdl(k_pack_infer, dim3((rows + 7) / 8), dim3(256), m->s, c0 > 0, X, ncol, c0, rows, m->N[0], m->D[0],
                         (const float*)m->xmu, (const float*)m->xisig, (const float*)m->lo, (const float*)m->hi,
                         m->act[0], fallback_mask, n_fallback))
             return fail(m, GWAM_ECUDA, "kernel launch failed");

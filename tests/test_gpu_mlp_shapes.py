@@ -77,3 +77,26 @@ def test_inference_column_counts(gw, ncol):
     Yo, _ = mlp.forward([(_bf16(W), b.astype(np.float64)) for W, b in par], _bf16(X))
     got = np.concatenate([du.cpu().numpy(), dv.cpu().numpy()]).T
     assert int(nfb.item()) == 0 and _rel(got, Yo) <= 1e-2
+
+
+@pytest.mark.parametrize("n_in,hidden,layers,ncol", [(5, 256, 2, 11265), (5, 512, 3, 5889), (70, 512, 2, 10001), (130, 256, 7, 20480), (512, 512, 1, 24673)])
+def test_inference_many_columns(gw, n_in, hidden, layers, ncol):
+    """Column counts that run all hidden layers in one kernel, with one, two and three row tiles a cluster, inputs
+    of one to eight K blocks; the last case in two chunks, the second one short and layer by layer.  Right behind
+    a training step the new weights are used."""
+    import torch
+    S, _ = _network(gw, n_in, hidden, layers, 3, 20480, seed=n_in + hidden)
+    r = np.random.default_rng(ncol)
+    X, Y = r.standard_normal((ncol, n_in)).astype(np.float32), r.standard_normal((ncol, 6)).astype(np.float32)
+    Xd, Yd = torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda()
+    out = [torch.zeros((6, ncol), dtype=torch.float64, device="cuda") for _ in range(2)]
+    mask, nfb = torch.zeros(ncol, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    for o in out:
+        if o is out[0]:
+            S.train_step(Xd, Yd, 1024, lr=1e-2)
+        S.infer(Xd, o[:3], o[3:], mask, nfb)
+    S.status()
+    assert torch.equal(out[0], out[1]) and int(nfb.item()) == 0
+    Yo, _ = mlp.forward([(_bf16(W), b.astype(np.float64)) for W, b in S.params()], _bf16(X))
+    assert _rel(out[0].cpu().numpy().T, Yo) <= 1e-2
