@@ -130,13 +130,14 @@ __device__ __forceinline__ float gelu_grad(float z)
     return fmaf(z * 0.39894228040143268f, e, fmaf(0.5f, copysignf(r, z), 0.5f));
 }
 
-// Epilogue of 32 consecutive accumulator columns n = nb .. nb+31 of one row.  Per-column parameters come
-// from shared memory (sbias: the bias of npad columns; EPI_DRAG: then sigma and mu).  Rows >= M only skip
-// the stores.  zz: the prefetched
+// Epilogue of 32 consecutive accumulator columns n = nb .. nb+31 of one row.  The columns' bias comes from
+// shared memory (sbias), behind it EPI_DRAG's sigma and mu where they fit beside the stages (not at 8192
+// outputs); EPI_DRAG_WIDE loads them from global memory (inference of 32 768 columns 121
+// and 124 us).  Rows >= M only skip the stores.  zz: the prefetched
 // pre-activations of EPI_BWD.
 template <int MODE>
 __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, float (&v)[32], const float* sbias,
-                                      int npad, const float (&zz)[32], int rowmask, gwam::DF& sq,
+                                      const float (&zz)[32], int rowmask, gwam::DF& sq,
                                       uint32_t stg, int cc0)
 {
     const bool live = row < e.M;
@@ -157,16 +158,18 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
                 v[4 * qq + 3] += b.w;
             }
         }
-        if (MODE == EPI_DRAG) {
+        if (MODE == EPI_DRAG || MODE == EPI_DRAG_WIDE) {
+            const int npad = (e.N + 31) & ~31;
             // de-normalised in FP32 (one FMA, relative error 6e-8, far below the BF16 network's) and
             // widened exactly by integer operations: FP64 arithmetic and float -> double conversions
             // run at 1/64 of the FP32 rate on GB300
             if (!live || rowmask != 0) return;
 #pragma unroll
             for (int j = 0; j < 32; j += 4) {
-                // sigma and mu behind the bias in shared memory, broadcast four at a time
-                const float4 s4 = *reinterpret_cast<const float4*>(sbias + npad + nb + j);
-                const float4 m4 = *reinterpret_cast<const float4*>(sbias + 2 * npad + nb + j);
+                const float4 s4 = MODE == EPI_DRAG ? *reinterpret_cast<const float4*>(sbias + npad + nb + j)
+                                                   : __ldg(reinterpret_cast<const float4*>(e.ysig + nb + j));
+                const float4 m4 = MODE == EPI_DRAG ? *reinterpret_cast<const float4*>(sbias + 2 * npad + nb + j)
+                                                   : __ldg(reinterpret_cast<const float4*>(e.ymu + nb + j));
                 const float sj[4] = {s4.x, s4.y, s4.z, s4.w}, mj[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -379,8 +382,8 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     // (the set-up above touched only shared and tensor memory and the kernel parameters)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int npad = (e.N + 31) & ~31;
     if (e.bias) {
+        const int npad = (e.N + 31) & ~31;
         for (int i = tid; i < npad; i += blockDim.x) {
             sbias[i] = i < e.N ? e.bias[i] : 0.0f;
             if (MODE == EPI_DRAG) {
@@ -500,7 +503,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
             const int m0 = (r / n_tiles) * kBM, n0 = (r % n_tiles) * BN;
             const int row = m0 + q * 32 + lane;
             const int cbeg = n0 + part * kColsPerWarp;
-            const int rowmask = (MODE == EPI_DRAG && row < e.M) ? e.mask[row] : 0;
+            const int rowmask = ((MODE == EPI_DRAG || MODE == EPI_DRAG_WIDE) && row < e.M) ? e.mask[row] : 0;
             const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((tl / 2) & 1), wlim);
             if (!__all_sync(0xffffffffu, got) || abort_flag) {
                 ok = false;
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rr[j]);
                 const uint32_t stg =
                     e.tstore ? stg_warp + (uint32_t)((32 * k) / 64) * 4096u + (uint32_t)lane * 128u : 0u;
-                epi32<MODE>(e, z, row, nb, v, sbias, npad, zz, rowmask, sq, stg, ((32 * k) % 64) / 8);
+                epi32<MODE>(e, z, row, nb, v, sbias, zz, rowmask, sq, stg, ((32 * k) % 64) / 8);
             }
             tc_before();
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&acce_bar[acc])) : "memory");
@@ -1146,7 +1149,9 @@ bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap
     constexpr size_t kStg = (size_t)32 * BN / (EPW / 4) * 2 * EPW;
     const size_t shm = (size_t)ST * (kABytes + BN * kBK * 2) + 1024 + (e.tstore ? kStg : 0) +
                        (e.bias ? (size_t)((e.N + 31) & ~31) * 4 * (MODE == EPI_DRAG ? 3 : 1) : 0);
-    if (shm > kMaxShm) return false;
+    if (shm > kMaxShm)
+        return MODE == EPI_DRAG ? launch_mode<BN, ST, EPW, MODE == EPI_DRAG ? (int)EPI_DRAG_WIDE : MODE>(ta, tb, tc, K, ksplit, e, s)
+                                : false;
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 64) return false;

@@ -7,9 +7,9 @@
 // K-major layout, written by cp.async.bulk.tensor) and signals a "full" mbarrier per stage with
 // the transaction byte count.  Thread 32 issues four 128 x BN x 16 tcgen05.mma per K block into
 // the TMEM accumulator and commits them to the stage's "empty" mbarrier, which hands the stage
-// back to the producer; a final commit signals the accumulator.  All four warps then read the
-// accumulator with tcgen05.ld (warp w owns TMEM lanes = tile rows 32w..32w+31) and run the
-// epilogue.  Every mbarrier wait is bounded in time; a wait that gives up sets the error word,
+// back to the producer; a final commit signals the accumulator (two of them, so that a tile's
+// epilogue overlaps the next tile's MMAs).  4 to 16 warps read it with tcgen05.ld (a warp owns 32 TMEM
+// lanes = tile rows) and run the epilogue.  Every mbarrier wait is bounded in time; a wait that gives up sets the error word,
 // the kernel still waits (bounded) for its own copies and MMAs and releases its TMEM.
 #pragma once
 
@@ -28,6 +28,7 @@ enum GemmEpiMode {
                     // y -> cf; sum of e^2 added to *loss
     EPI_DRAG = 3,   // y = acc + bias; for n < n_true and mask[row] == 0: y * ysig[n] + ymu[n]
                     // -> du[n * ncol + row] (n < nlev) or dv[(n - nlev) * ncol + row]
+    EPI_DRAG_WIDE = 4,   // the launch's form of EPI_DRAG for outputs too many for shared memory
 };
 
 struct GemmEpi {
@@ -48,8 +49,8 @@ struct GemmEpi {
     int ldt;
     int n_true;               // EPI_LOSS / EPI_DRAG: number of real outputs (N may be padded)
     float gscale;             // EPI_LOSS: dL/dy = gscale * (y - t)
-    double* loss;             // EPI_LOSS: sum of squared errors (FP64 atomic per warp)
-    const float* ysig;        // EPI_DRAG: de-normalisation
+    double* loss;             // EPI_LOSS: sum of squared errors (double-float in the warp, one FP64 atomic)
+    const float* ysig;        // EPI_DRAG: de-normalisation (N entries, N a multiple of 32, 16-byte aligned)
     const float* ymu;
     const int* mask;          // EPI_DRAG: 1 = column goes to the ray tracer
     double* du;

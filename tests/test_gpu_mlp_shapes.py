@@ -100,3 +100,19 @@ def test_inference_many_columns(gw, n_in, hidden, layers, ncol):
     assert torch.equal(out[0], out[1]) and int(nfb.item()) == 0
     Yo, _ = mlp.forward([(_bf16(W), b.astype(np.float64)) for W, b in S.params()], _bf16(X))
     assert _rel(out[0].cpu().numpy().T, Yo) <= 1e-2
+
+
+@pytest.mark.parametrize("nlev,ncol", [(1, 130), (1500, 130), (4096, 130), (4096, 20000)])
+def test_inference_output_widths(gw, nlev, ncol):
+    """Output layers up to the widest one accepted: the epilogue's per-column parameters fit at every tile width."""
+    import torch
+    S, par = _network(gw, 40, 64, 1, nlev, 20480, seed=nlev)
+    X = np.random.default_rng(ncol).standard_normal((ncol, 40)).astype(np.float32)
+    du = torch.zeros((nlev, ncol), dtype=torch.float64, device="cuda")
+    dv, mask, nfb = torch.zeros_like(du), torch.zeros(ncol, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    S.infer(torch.from_numpy(X).cuda(), du, dv, mask, nfb)
+    S.status()
+    rows = np.r_[0:65, ncol - 65:ncol]
+    Yo, _ = mlp.forward([(_bf16(W), b.astype(np.float64)) for W, b in par], _bf16(X[rows]))
+    got = np.concatenate([du[:, rows].cpu().numpy(), dv[:, rows].cpu().numpy()]).T
+    assert int(nfb.item()) == 0 and _rel(got, Yo) <= 1e-2
