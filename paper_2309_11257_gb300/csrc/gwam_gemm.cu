@@ -1244,6 +1244,8 @@ int gemm_sm_count()
 
 int gemm_pick_bn(int M, int N)
 {
+    // (beyond 8192 columns the bias does not fit beside the eight stages of the narrowest tiles)
+    if (N > 8192) return 256;
     const int sms = gemm_sm_count();
     int best = 256;
     long long cost = -1;

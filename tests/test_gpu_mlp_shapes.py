@@ -116,3 +116,19 @@ def test_inference_output_widths(gw, nlev, ncol):
     Yo, _ = mlp.forward([(_bf16(W), b.astype(np.float64)) for W, b in par], _bf16(X[rows]))
     got = np.concatenate([du[:, rows].cpu().numpy(), dv[:, rows].cpu().numpy()]).T
     assert int(nfb.item()) == 0 and _rel(got, Yo) <= 1e-2
+
+
+@pytest.mark.parametrize("N", [8192, 8704, 16320])
+def test_gemm_wide_with_bias(gw, N):
+    """The tile width picked for few rows and many columns leaves room for the bias (bar of test_gpu_gemm.py)."""
+    import ctypes as C
+    import torch
+    g = torch.Generator().manual_seed(N)
+    A, B = torch.randn(100, 64, generator=g).to(torch.bfloat16), (torch.randn(N, 64, generator=g) / 8).to(torch.bfloat16)
+    b = torch.randn(N, generator=g).float()
+    Ad, Bd, bd, Cd = A.cuda(), B.cuda(), b.cuda(), torch.full((100, N), float("nan"), dtype=torch.float32, device="cuda")
+    p = lambda t: C.c_void_p(t.data_ptr())
+    assert gw.lib().gwam_gemm_bf16(p(Ad), p(Bd), 100, N, 64, p(bd), 0, 0, 0, p(Cd),
+                                   C.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    z, S = A.double() @ B.double().T + b.double(), A.double().abs() @ B.double().abs().T
+    assert ((Cd.cpu().double() - z).abs() <= 2e-5 * S + 1e-6 * z.abs()).all()
