@@ -69,13 +69,11 @@ def clear_bytes(nx, ny, nz, theta=False):
 
 # DRAM bytes (read + write) of one launch in the ncu captures in profiles/, as a fraction of that
 # launch's algorithmic bytes (ray bytes x 253 952 rays + the clearing of the 128 x 64 x 90 fields):
-# k_advance 67.75 MB of 134.48 MB, k_advance32 40.77 MB of 85.72 MB (written field lines still in L2
+# k_advance 60.96 MB of 134.48 MB, k_advance32 36.69 MB of 85.72 MB (written field lines still in L2
 # when the kernel ends are not counted).  The bench's traffic is that fraction of its own launch's
-# algorithmic bytes; None while the kernel has changed since its counters were taken: k_advance has
-# (narrow, which its double-float splits call on their out-of-range path, changed after the capture;
-# its loads and stores did not), so its traffic is null until the next capture.
-ADV_TRAFFIC_FRACTION = None     # was 67.75 / 134.48
-ADV32_TRAFFIC_FRACTION = 40.77 / 85.72
+# algorithmic bytes; None while a kernel has changed since its counters were taken.
+ADV_TRAFFIC_FRACTION = 60.96 / 134.48
+ADV32_TRAFFIC_FRACTION = 36.69 / 85.72
 
 
 def measured_peaks():
@@ -467,8 +465,7 @@ def gpu_arm(args, rank, world, local_rank):
                                        "k_advance_sphere_half_fp64.md) as a fraction of that launch's algorithmic "
                                        "bytes (ray state, gathers, field clearing), times this launch's")
                     if ADV_TRAFFIC_FRACTION is not None else
-                    "null: k_advance changed after its ncu capture (profiles/k_advance_sphere_half_fp64.md: "
-                    "DRAM 50 % of the algorithmic bytes then)",
+                    "null: k_advance changed after its ncu capture",
                     "peak_source": "modelled (not measured) from unit counts and the 2.07 GHz clock: "
                                    "FP64-precision operations as double-float on the FP32 pipes (5.37 T/s at 7.5 "
                                    "instructions each) plus the FP64 pipe (0.63 T/s)",
@@ -691,7 +688,7 @@ def surrogate_arm(args):
     peaks = measured_peaks()
     peak = peaks.get("bf16_tflops", 1900.0)
     achieved = SUR_FLOPS_PER_COLUMN * B / (gemm_ms / 1000.0) / 1e12
-    roofline = {"bound": "tensor", "kernel": "k_gemm_bf16 (tcgen05, 5 launches per pass)", "achieved": achieved,
+    roofline = {"bound": "tensor", "kernel": "k_hidden + k_gemm_bf16 (tcgen05: the hidden layers in one launch, the output layer)", "achieved": achieved,
                 "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                 "peak_source": "measured burst bf16 (MEASURED_PEAKS.json bf16_tflops)",
                 "gemm_ms_per_pass": gemm_ms, "pack_ms_per_pass": prof["pack_ms"] / max(passes, 1),
@@ -748,7 +745,7 @@ def surrogate_arm(args):
                        if infos else None,
                        "generation_seconds": gen_s, "prep_seconds": prep_s, "fallback_in_batch": int(nfb.item()),
                        "l2": "256 MB buffer written between timed passes"},
-            "gpu_launches": args.steps * 6, "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
+            "gpu_launches": args.steps * 3, "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
             "clocks": clocks}
     print(json.dumps(line), flush=True)
     return 0
