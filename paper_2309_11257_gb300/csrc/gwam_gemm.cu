@@ -130,6 +130,36 @@ __device__ __forceinline__ float gelu_grad(float z)
     return fmaf(z * 0.39894228040143268f, e, fmaf(0.5f, copysignf(r, z), 0.5f));
 }
 
+// Sum of the squares of 32 errors, as accurate as the FP64 sum and over its whole range.  FP64 additions and
+// conversions of every element (1/64 of the FP32 rate) had made this kernel 55 us: the exact products
+// (hi, lo) go into an unevaluated sum of three FP32 numbers, the errors of the two larger ones carried into the
+// next, and only the three results are added in FP64 (relative error about 2^-53; a double-float sum, 48 bits, was
+// 1e-14 off after 64 elements).  Products that FP32 cannot hold exactly -- a non-zero error outside 2^-50 .. 2^60,
+// infinities -- take FP64 throughout.
+__device__ __forceinline__ double sum_squares(const float (&d)[32])
+{
+    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, most = 0.0f, least = 1.0f;
+    auto two_sum = [](float& s, float x) {
+        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+        s = t;
+        return e;
+    };
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const DF p = df_prod(d[j], d[j]);
+        const float e0 = two_sum(s0, p.hi);
+        s2 = __fadd_rn(s2, __fadd_rn(two_sum(s1, e0), two_sum(s1, p.lo)));
+        most = fmaxf(most, fabsf(d[j]));
+        least = fminf(least, d[j] == 0.0f ? 1.0f : fabsf(d[j]));
+    }
+    if (most <= 0x1p60f && least >= 0x1p-50f) return widen(s0) + (widen(s1) + widen(s2));
+    double q = 0.0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) q = fma((double)d[j], (double)d[j], q);
+    return q;
+}
+
 // Epilogue of 32 consecutive accumulator columns n = nb .. nb+31 of one row.  The columns' bias comes from
 // shared memory (sbias), behind it EPI_DRAG's sigma and mu where they fit beside the stages (not at 8192
 // outputs); EPI_DRAG_WIDE loads them from global memory (inference of 32 768 columns 121
@@ -137,8 +167,8 @@ __device__ __forceinline__ float gelu_grad(float z)
 // pre-activations of EPI_BWD.
 template <int MODE>
 __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, float (&v)[32], const float* sbias,
-                                      const float (&zz)[32], int rowmask, gwam::DF& sq,
-                                      uint32_t stg, int cc0)
+                                      const float (&zz)[32], int rowmask, double& sq, uint32_t stg,
+                                      int cc0)
 {
     const bool live = row < e.M;
     const bool full = nb + 32 <= e.N;
@@ -234,13 +264,10 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
                 for (int j = 0; j < 32; ++j) tp[j] = nb + j < e.n_true ? tg[j] : 0.0f;
             }
 #pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                // the squares (exact products) summed in double-float: FP64 additions and conversions
-                // had made this kernel 55 us
-                const float d = nb + j < e.n_true ? v[j] - tp[j] : 0.0f;
-                sq = gwam::df_add(sq, gwam::df_prod(d, d));
-                v[j] = e.gscale * d;
-            }
+            for (int j = 0; j < 32; ++j) v[j] = nb + j < e.n_true ? v[j] - tp[j] : 0.0f;
+            sq += sum_squares(v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = e.gscale * v[j];
         }
     }
     if (!live) return;
@@ -398,7 +425,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     const uint32_t tmem = tmem_slot;
     const unsigned long long wlim = e.wait_ns ? e.wait_ns : kWaitNs;
     bool ok = true;
-    DF sq{0.0f, 0.0f};
+    double sq = 0.0;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -580,10 +607,9 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
         __syncwarp();
         if (!ok) abort_flag = 1;
         if (MODE == EPI_LOSS) {
-            double sum = df_to_double(sq);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane == 0 && sum != 0.0) atomicAdd(e.loss, sum);
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if (lane == 0 && sq != 0.0) atomicAdd(e.loss, sq);
         }
     }
     // every MMA has finished before the TMEM is released (bounded wait; immediate normally)

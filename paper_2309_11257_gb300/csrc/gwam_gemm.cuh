@@ -49,7 +49,7 @@ struct GemmEpi {
     int ldt;
     int n_true;               // EPI_LOSS / EPI_DRAG: number of real outputs (N may be padded)
     float gscale;             // EPI_LOSS: dL/dy = gscale * (y - t)
-    double* loss;             // EPI_LOSS: sum of squared errors (double-float in the warp, one FP64 atomic)
+    double* loss;             // EPI_LOSS: sum of squared errors, to FP64 accuracy and range
     const float* ysig;        // EPI_DRAG: de-normalisation (N entries, N a multiple of 32, 16-byte aligned)
     const float* ymu;
     const int* mask;          // EPI_DRAG: 1 = column goes to the ray tracer
