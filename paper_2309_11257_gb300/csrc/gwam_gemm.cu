@@ -1167,15 +1167,26 @@ __global__ void __launch_bounds__(64 + 32 * kGradEpi, 1) k_grad_update(const __g
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
+// Shared memory of k_gemm_bf16: the stages, with TMA stores 4 KB of staging boxes (32 rows x 64 columns) an
+// epilogue warp, and the bias of all columns (in EPI_DRAG with sigma and mu behind it)
+constexpr size_t gemm_smem(int bn, int stages, int warps, int N, int columns, bool staged)
+{
+    return (size_t)stages * (kABytes + bn * kBK * 2) + 1024 + (staged ? (size_t)warps * 4096 : 0) +
+           (size_t)columns * ((N + 31) & ~31) * 4;
+}
+constexpr size_t kGemmMaxSmem = 232448 - 256;   // 227 KB opt-in per block, less the static part
+struct GemmShape {
+    int bn, stages, warps;
+};
+constexpr GemmShape kGemmShapes[] = {{256, 3, 16}, {192, 4, 12}, {128, 5, 8}, {64, 8, 4}};
+
 template <int BN, int ST, int EPW, int MODE>
 bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int K, int ksplit,
                  const GemmEpi& e, cudaStream_t s)
 {
-    constexpr size_t kMaxShm = 232448 - 256;   // 227 KB opt-in per block, less the static part
-    constexpr size_t kStg = (size_t)32 * BN / (EPW / 4) * 2 * EPW;
-    const size_t shm = (size_t)ST * (kABytes + BN * kBK * 2) + 1024 + (e.tstore ? kStg : 0) +
-                       (e.bias ? (size_t)((e.N + 31) & ~31) * 4 * (MODE == EPI_DRAG ? 3 : 1) : 0);
-    if (shm > kMaxShm)
+    static_assert(BN / (EPW / 4) == 64, "a warp's staging box");
+    const size_t shm = gemm_smem(BN, ST, EPW, e.N, e.bias ? (MODE == EPI_DRAG ? 3 : 1) : 0, e.tstore);
+    if (shm > kGemmMaxSmem)
         return MODE == EPI_DRAG ? launch_mode<BN, ST, EPW, MODE == EPI_DRAG ? (int)EPI_DRAG_WIDE : MODE>(ta, tb, tc, K, ksplit, e, s)
                                 : false;
     int dev = 0;
@@ -1208,15 +1219,16 @@ bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap
 
 // one kernel per epilogue mode: each holds only its own epilogue code (a smaller instruction
 // footprint for the epilogue warps, whose instruction fetch otherwise stalls them)
-template <int BN, int ST, int EPW>
+template <int SHAPE>
 bool launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int K, int ksplit, const GemmEpi& e,
             cudaStream_t s)
 {
+    constexpr GemmShape g = kGemmShapes[SHAPE];
     switch (e.mode) {
-    case EPI_STORE: return launch_mode<BN, ST, EPW, EPI_STORE>(ta, tb, tc, K, ksplit, e, s);
-    case EPI_BWD: return launch_mode<BN, ST, EPW, EPI_BWD>(ta, tb, tc, K, ksplit, e, s);
-    case EPI_LOSS: return launch_mode<BN, ST, EPW, EPI_LOSS>(ta, tb, tc, K, ksplit, e, s);
-    case EPI_DRAG: return launch_mode<BN, ST, EPW, EPI_DRAG>(ta, tb, tc, K, ksplit, e, s);
+    case EPI_STORE: return launch_mode<g.bn, g.stages, g.warps, EPI_STORE>(ta, tb, tc, K, ksplit, e, s);
+    case EPI_BWD: return launch_mode<g.bn, g.stages, g.warps, EPI_BWD>(ta, tb, tc, K, ksplit, e, s);
+    case EPI_LOSS: return launch_mode<g.bn, g.stages, g.warps, EPI_LOSS>(ta, tb, tc, K, ksplit, e, s);
+    case EPI_DRAG: return launch_mode<g.bn, g.stages, g.warps, EPI_DRAG>(ta, tb, tc, K, ksplit, e, s);
     default: return false;
     }
 }
@@ -1268,19 +1280,18 @@ int gemm_sm_count()
     return sms[dev];
 }
 
-int gemm_pick_bn(int M, int N)
+int gemm_pick_bn(int M, int N, bool bias, bool staged)
 {
-    // (beyond 8192 columns the bias does not fit beside the eight stages of the narrowest tiles)
-    if (N > 8192) return 256;
     const int sms = gemm_sm_count();
     int best = 256;
     long long cost = -1;
-    for (int bn : {256, 192, 128, 64}) {
-        const long long tiles = (long long)((M + kBM - 1) / kBM) * ((N + bn - 1) / bn);
-        const long long c = (tiles + sms - 1) / sms * (bn + 48);
+    for (const GemmShape& g : kGemmShapes) {
+        if (gemm_smem(g.bn, g.stages, g.warps, N, bias, staged) > kGemmMaxSmem) continue;
+        const long long tiles = (long long)((M + kBM - 1) / kBM) * ((N + g.bn - 1) / g.bn);
+        const long long c = (tiles + sms - 1) / sms * (g.bn + 48);
         if (cost < 0 || c < cost) {
             cost = c;
-            best = bn;
+            best = g.bn;
         }
     }
     return best;
@@ -1399,12 +1410,13 @@ bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtens
     e.tstore = (tc && e.cb) ? 1 : 0;
     static const CUtensorMap none{};
     const CUtensorMap& tcm = e.tstore ? *tc : none;
-    if (bn == 0) bn = gemm_pick_bn(e.M, e.N);
+    if (bn == 0) bn = gemm_pick_bn(e.M, e.N, e.bias != nullptr, e.tstore != 0);
+    static_assert(kGemmShapes[0].bn == 256 && kGemmShapes[1].bn == 192 && kGemmShapes[2].bn == 128 && kGemmShapes[3].bn == 64);
     switch (bn) {
-    case 64: return launch<64, 8, 4>(ta, tb, tcm, K, ksplit, e, s);
-    case 128: return launch<128, 5, 8>(ta, tb, tcm, K, ksplit, e, s);
-    case 192: return launch<192, 4, 12>(ta, tb, tcm, K, ksplit, e, s);
-    case 256: return launch<256, 3, 16>(ta, tb, tcm, K, ksplit, e, s);
+    case 256: return launch<0>(ta, tb, tcm, K, ksplit, e, s);
+    case 192: return launch<1>(ta, tb, tcm, K, ksplit, e, s);
+    case 128: return launch<2>(ta, tb, tcm, K, ksplit, e, s);
+    case 64: return launch<3>(ta, tb, tcm, K, ksplit, e, s);
     default: return false;
     }
 }
@@ -1420,7 +1432,7 @@ int gemm_selftest(const void* A, const void* B, int M, int N, int K, const float
                                                                   bn != 256))
         return -1;
     cudaStream_t s = (cudaStream_t)stream;
-    const int use_bn = bn ? bn : gwam::gemm_pick_bn(M, N);
+    const int use_bn = bn ? bn : gwam::gemm_pick_bn(M, N, bias != nullptr, out_bf16 && N % 8 == 0);
     CUtensorMap ta, tb, tc;
     if (!gwam::make_tmap_bf16(&ta, A, (uint64_t)M, (uint64_t)K, (uint64_t)K, 128) ||
         !gwam::make_tmap_bf16(&tb, B, (uint64_t)N, (uint64_t)K, (uint64_t)K, (uint32_t)use_bn))

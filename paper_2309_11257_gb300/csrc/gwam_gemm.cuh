@@ -100,7 +100,7 @@ bool gemm_bf16_grad_launch(GradSet& set, int K, int* err, cudaStream_t s);
 // Launch: A described by ta (box rows 128), B by tb (box rows bn); K a multiple of 64, split into
 // ksplit slices along K (K / 64 must be divisible by ksplit).  tc (or null): tensor map of the BF16
 // output cb (box 64 columns x 32 rows) -- the epilogue then stages each warp's rows in shared memory
-// and writes them with TMA stores.  bn = 0 picks the tile width from N.  false on an unsupported
+// and writes them with TMA stores.  bn = 0 picks the tile width (gemm_pick_bn).  false on an unsupported
 // shape.
 bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ksplit,
                       const GemmEpi& e, cudaStream_t s);
@@ -123,8 +123,10 @@ bool gemm_hidden_launch(const HiddenSet& h, int M, int N, int* err, cudaStream_t
 // The tile width gemm_bf16_launch uses when bn = 0 (the caller builds tb with this box): the one with
 // the least waves x (width + 48) over the GPU's SMs -- a tile's time grows with its width, 48 columns
 // stand for its fixed part.  Wide tiles for large M (32 768 x 512: 256), narrow ones where wide ones
-// would leave SMs idle (4096 x 512: 128 instead of 64 tiles of 256; 1000 x 512: 64).
-int gemm_pick_bn(int M, int N);
+// would leave SMs idle (4096 x 512: 128 instead of 64 tiles of 256; 1000 x 512: 64).  Only widths whose
+// shared memory holds the bias of all N columns (if there is one) and the staging boxes of TMA stores (`staged`)
+// beside the stages: with both, 64, 192 and 256 do up to 4544 columns, 128 up to 8640.
+int gemm_pick_bn(int M, int N, bool bias, bool staged);
 // compute units of the current device
 int gemm_sm_count();
 

@@ -448,14 +448,14 @@ bool forward(gwam_mlp* m, int B, bool train, const gwam::GemmEpi& last)
             e.ct = m->actT[l];
             e.ldct = m->max_batch;
         }
-        const int bn = gwam::gemm_pick_bn(B, m->D[l]);
+        const int bn = gwam::gemm_pick_bn(B, m->D[l], true, true);
         if (!gemm(m, m->tf_a[l], m->tf_b[l][bn / 64 - 1], &m->to_act[l], m->D[l - 1], bn, 1, e)) return false;
     }
     gwam::GemmEpi e = last;
     e.M = B;
     e.N = m->D[m->nl];
     e.bias = m->b[m->nl];
-    const int bn = gwam::gemm_pick_bn(B, e.N);
+    const int bn = gwam::gemm_pick_bn(B, e.N, true, e.cb != nullptr);
     return gemm(m, m->tf_a[m->nl], m->tf_b[m->nl][bn / 64 - 1], e.cb ? &m->to_dz[m->nl] : nullptr, m->D[m->nl - 1],
                 bn, 1, e);
 }
@@ -707,7 +707,7 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
         x.ldcb = m->D[l - 1];
         x.ct = m->dzT[l - 1];
         x.ldct = m->max_batch;
-        const int bn = gwam::gemm_pick_bn(B, x.N);
+        const int bn = gwam::gemm_pick_bn(B, x.N, false, true);
         ok = gemm(m, m->tx_a[l], m->tx_b[l][bn / 64 - 1], &m->to_dz[l - 1], m->D[l], bn, 1, x);
     }
     // then the weight gradients of all layers, dW_l = dz_l^T act_{l-1}, with the weight updates in one
