@@ -191,7 +191,7 @@ __device__ __forceinline__ unsigned long long key_scaled(unsigned long long key,
 
 constexpr int kCapThreads = 128;
 constexpr int kCapKeys = 1024;   // keys held in shared memory; longer columns keep theirs in global scratch
-constexpr double kCapDelta = 1.0 / (1ll << 36);
+constexpr double kCapDelta = 1.0 / (1 << 24);
 
 // The entries [a, a + count) that the cap removes from an over-full column: the `drop` with the lowest
 // energies, ties by the larger id first, as one block (kCapThreads).  energy(e) may be off by kCapDelta / 2

@@ -535,6 +535,7 @@ struct GeoDF {
 // (|d| <= half a row): sin(p0 + d) = s0 cos d + c0 sin d, cos(p0 + d) = c0 cos d - s0 sin d, with
 // sin d and cos d from their Taylor series -- the terms up to d^3 and d^4 in DF, the smaller ones
 // (below 3e-8 for rows of up to 9 degrees) in FP32, truncated after d^7 and d^8
+constexpr double kLatSeriesRow = 9.0 * kPi / 180.0;
 __device__ __forceinline__ void lat_sincos_row_df(const Grid& G, int j, DF Y, DF& sphi, DF& cphi)
 {
     const float2 rl = G.row_lat_df[j];

@@ -463,7 +463,11 @@ __global__ void k_cap_find(Grid G, Params P, Ctl* ctl, const int* __restrict__ o
 // Remove the lowest-energy ray volumes of each over-full column (energy w_hat * N Px Py Pz;
 // ties: the larger id goes first), a block per column: w_hat in double-float, in FP64 for the few
 // volumes around the cut, so that the choice is the FP64 energies' (8192 columns of 128 volumes: 407 us
-// while every energy was formed in FP64 and ranked by FP64 comparisons).
+// while every energy was formed in FP64 and ranked by FP64 comparisons).  The double-float w_hat^2 = f^2 +
+// (N^2 - f^2) k_h^2 / K^2 is a sum of positive terms (a background has N^2 > f^2), good to 2^-44, and kCapDelta
+// leaves a factor of 2^19 for f close to the equator.  On rows wider than the latitude's series is for (kSeries
+// false; two rows: 3e-7 off, which changed the choice) every energy is the FP64 one.
+template <bool kSeries>
 __global__ void __launch_bounds__(kCapThreads) k_cap_apply(Grid G, Params P, RaySoA A, const NodeDF* __restrict__ bg,
                                                              Ctl* ctl, const int* __restrict__ info,
                                                              const int* __restrict__ off,
@@ -481,12 +485,22 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_apply(Grid G, Params P, Ray
         load_ray(A, src >> 2, s, id);
         make_child(G, s, info[src >> 2] & 7, src & 3, ch);
     };
+    auto exact = [&](int e) {
+        double ch[NSTATE];
+        long long id;
+        child(e, ch, id);
+        Geo g;
+        Intr in;
+        intrinsic_at(G, bg + (int64_t)member_of(id) * G.ncell, ch, g, in);
+        return in.w * ray_action(ch);
+    };
     for (int w = blockIdx.x; w < nover; w += gridDim.x) {
         const int col = overlist[w];
         const int a = off[col * G.nz], count = off[(col + 1) * G.nz] - a;
         cap_column(
             a, count, count - P.cap, ent_id, ecap,
             [&](int e) {
+                if (!kSeries) return exact(e);
                 double ch[NSTATE];
                 long long id;
                 child(e, ch, id);
@@ -494,15 +508,7 @@ __global__ void __launch_bounds__(kCapThreads) k_cap_apply(Grid G, Params P, Ray
                 intrinsic_df(G, bg + (int64_t)member_of(id) * G.ncell, ch, in);
                 return df_to_double(df_mul2(in.d.w2, in.d.iw)) * ray_action(ch);
             },
-            [&](int e) {
-                double ch[NSTATE];
-                long long id;
-                child(e, ch, id);
-                Geo g;
-                Intr in;
-                intrinsic_at(G, bg + (int64_t)member_of(id) * G.ncell, ch, g, in);
-                return in.w * ray_action(ch);
-            },
+            exact,
             [&](int e) {
                 double ch[NSTATE];
                 long long id;
@@ -1130,8 +1136,9 @@ void run_step(Context& c, double dt, double* du, double* dv)
     const CellOffsets cell{c.off, c.off2};
     if (P.cap > 0) {
         k_cap_find<<<col_blocks, kThreads, 0, s>>>(G, P, c.ctl, c.off, c.overlist);
-        k_cap_apply<<<c.max_blocks, kCapThreads, 0, s>>>(G, P, c.A, c.bgdf, c.ctl, c.info, c.off, c.overlist, c.ent_id,
-                                                         c.ent_src, c.ent_cell, c.ecap, c.cnt, c.partials, c.max_blocks);
+        auto* cap = G.geometry != 1 || G.dY <= kLatSeriesRow ? k_cap_apply<true> : k_cap_apply<false>;
+        cap<<<c.max_blocks, kCapThreads, 0, s>>>(G, P, c.A, c.bgdf, c.ctl, c.info, c.off, c.overlist, c.ent_id, c.ent_src,
+                                                 c.ent_cell, c.ecap, c.cnt, c.partials, c.max_blocks);
         exclusive_scan(c, c.cnt, c.off2, G.ncell_all, nullptr, &c.ctl->n_over);
         mask |= 1 << T_CAP;
     }
