@@ -480,15 +480,16 @@ __device__ __forceinline__ int ghost_emit(const Grid& G, const NodeDF* __restric
 // member alone) staged at position t of S / S32, filtered bins counted; k_launch_place then moves the
 // launched ones behind the live rays.  (While both passes computed the states, a ghost-layer launch
 // into 8192 columns took 2 x 390 us.)  kGhost: what left the ghost layer over ghost_dt instead of
-// the launch state itself.  Dynamic shared memory: the ghost's kRkWarp a warp, then the source's sines and cosines
-// of the azimuths and its phase speeds (2 n_az + n_c doubles).
+// the launch state itself.  The source's bins are counted from bin0 of column col0 on.  Dynamic shared
+// memory: the ghost's kRkWarp a warp, then the source's sines and cosines of the azimuths and its phase speeds
+// (2 n_az + n_c doubles).
 template <bool kSpec, bool kGhost>
 __global__ void __launch_bounds__(kThreads, 2) k_launch(Grid G, const Node* __restrict__ bg,
                                                         const NodeDF* __restrict__ bgdf, RaySoA S, Ray32SoA S32s, bool f32,
                                                         Ctl* ctl, gwam_bg_source src,
                                                         const LaunchColumn* __restrict__ cols,
-                                                        const gwam_spec* __restrict__ specs, int total, double ghost_dt,
-                                                        int* __restrict__ flag)
+                                                        const gwam_spec* __restrict__ specs, int col0, int bin0, int total,
+                                                        double ghost_dt, int* __restrict__ flag)
 {
     extern __shared__ float4 sh_launch[];
     double* const az = reinterpret_cast<double*>(sh_launch + (kGhost ? kRkWarp * (blockDim.x / 32) : 0));
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_launch(Grid G, const Node* __re
                                   sp.spectral_frac, s);
             }
         } else if (eligible) {
-            const int g = t / nbins, bin = t - g * nbins;
+            const int q = (bin0 + t) / nbins, g = col0 + q, bin = bin0 + t - q * nbins;
             const LaunchColumn col = cols[g];
             eligible = col.hY != 0.0;
             if (eligible) {
@@ -597,6 +598,10 @@ void configure_launch_kernels()
     cudaFuncSetAttribute(k_launch<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRkSmem);
 }
 
+// Launches of more bins than the context holds ray volumes (most bins filtered, or an overflow to be reported)
+// go in parts: of this many bins, or of max_rays, whichever is more
+constexpr int64_t kLaunchPart = 1 << 18;
+
 static void launch_common(Context& c, const gwam_bg_source* src, const gwam_spec* specs, int64_t total,
                           double ghost_dt = 0.0)
 {
@@ -604,47 +609,55 @@ static void launch_common(Context& c, const gwam_bg_source* src, const gwam_spec
     const int nb = c.grid_blocks;
     const bool ghost = ghost_dt > 0.0;
     // The re-binned ray buffer is free between steps: launch states of up to max_rays bins are staged
-    // there, their flags in the per-ray scratch.  Larger launches (most bins filtered, or an overflow
-    // to be reported) bring their own.
+    // there, their flags in the per-ray scratch.  A part of more bins than that brings its own (30 MB; for
+    // all bins at once it would be 116 bytes each, gigabytes on a large grid with many bins), or, where that
+    // cannot be had, is cut down until it can or fits the free buffer.
     RaySoA S = c.B;
     Ray32SoA S32s = c.B32;
     int* flag = c.newid;
     char* own = nullptr;
-    if (total > c.max_rays) {
-        const size_t rec = c.f32 ? 4 * sizeof(float4) : 7 * sizeof(double2);
-        if (cudaMallocAsync((void**)&own, rec * (size_t)total + sizeof(int) * (size_t)(total + 1), c.stream) != cudaSuccess) {
-            cudaGetLastError();
-            c.err = "launch: scratch allocation failed";
-            throw (int)GWAM_ENOMEM;
+    int64_t part = std::min(total, std::max(c.max_rays, kLaunchPart));
+    const size_t rec = c.f32 ? 4 * sizeof(float4) : 7 * sizeof(double2);
+    while (part > c.max_rays) {
+        if (cudaMallocAsync((void**)&own, rec * (size_t)part + sizeof(int) * (size_t)(part + 1), c.stream) == cudaSuccess) {
+            for (int q = 0; q < 7; ++q) S.a[q] = reinterpret_cast<double2*>(own) + q * part;
+            for (int q = 0; q < 4; ++q) S32s.q[q] = reinterpret_cast<float4*>(own) + q * part;
+            flag = reinterpret_cast<int*>(own + rec * (size_t)part);
+            break;
         }
-        for (int q = 0; q < 7; ++q) S.a[q] = reinterpret_cast<double2*>(own) + q * total;
-        for (int q = 0; q < 4; ++q) S32s.q[q] = reinterpret_cast<float4*>(own) + q * total;
-        flag = reinterpret_cast<int*>(own + rec * (size_t)total);
+        cudaGetLastError();
+        own = nullptr;
+        part = std::max(c.max_rays, part / 2);
     }
     gwam_bg_source s0{};
     if (src) s0 = *src;
     // the ghost layer propagates vertically only: the single-column equations on this grid copy
     Grid G = c.G;
     if (ghost) G.columnar = 1;
-    // one wave of two blocks per SM; few bins in blocks of a warp, spread over the SMs (the bins' FP64
-    // chains share an SM's FP64 pipe: 200 bins in one block took 16 us)
-    const int threads = total >= 2 * (int64_t)c.num_sms * kThreads ? kThreads : 32;
-    const int blocks = (int)std::min<int64_t>((int64_t)nb * (kThreads / threads), (total + threads - 1) / threads);
-    const size_t shm = (ghost ? kRkSmem / (kThreads / threads) : 0) + (specs ? 0 : (2 * s0.n_az + s0.n_c) * sizeof(double));
     if (!specs) {
         const int cb = std::min((c.G.ncol_all + 31) / 32, 32 * c.num_sms);
         k_launch_columns<<<cb, 32, 0, c.stream>>>(c.G, c.bg, s0, reinterpret_cast<LaunchColumn*>(c.launch_cols));
     }
+    const int nbins = specs ? 1 : s0.n_az * s0.n_c;
     auto* kernel = specs ? (ghost ? k_launch<true, true> : k_launch<true, false>)
                          : (ghost ? k_launch<false, true> : k_launch<false, false>);
-    kernel<<<blocks, threads, shm, c.stream>>>(
-        G, c.bg, c.bgdf, S, S32s, c.f32, c.ctl, s0, reinterpret_cast<const LaunchColumn*>(c.launch_cols), specs,
-        (int)total, ghost_dt, flag);
-    exclusive_scan(c, flag, flag, total, nullptr);
-    const int pb = std::min<int>(nb, (int)((total + kThreads - 1) / kThreads));
-    k_launch_place<<<pb, kThreads, 0, c.stream>>>(c.G, S, S32s, c.A, c.A32, c.f32, c.ctl, c.max_rays, (int)total, flag,
-                                                  c.partials, c.max_blocks);
-    finalize_launch(c, pb, flag, (int)total);
+    for (int64_t first = 0; first < total; first += part) {
+        const int64_t n = std::min(part, total - first);
+        // one wave of two blocks per SM; few bins in blocks of a warp, spread over the SMs (the bins' FP64
+        // chains share an SM's FP64 pipe: 200 bins in one block took 16 us)
+        const int threads = n >= 2 * (int64_t)c.num_sms * kThreads ? kThreads : 32;
+        const int blocks = (int)std::min<int64_t>((int64_t)nb * (kThreads / threads), (n + threads - 1) / threads);
+        const size_t shm =
+            (ghost ? kRkSmem / (kThreads / threads) : 0) + (specs ? 0 : (2 * s0.n_az + s0.n_c) * sizeof(double));
+        kernel<<<blocks, threads, shm, c.stream>>>(
+            G, c.bg, c.bgdf, S, S32s, c.f32, c.ctl, s0, reinterpret_cast<const LaunchColumn*>(c.launch_cols),
+            specs ? specs + first : nullptr, (int)(first / nbins), (int)(first % nbins), (int)n, ghost_dt, flag);
+        exclusive_scan(c, flag, flag, n, nullptr);
+        const int pb = std::min<int>(nb, (int)((n + kThreads - 1) / kThreads));
+        k_launch_place<<<pb, kThreads, 0, c.stream>>>(c.G, S, S32s, c.A, c.A32, c.f32, c.ctl, c.max_rays, (int)n, flag,
+                                                      c.partials, c.max_blocks);
+        finalize_launch(c, pb, flag, (int)n);
+    }
     if (own) cudaFreeAsync(own, c.stream);
 }
 
