@@ -664,10 +664,14 @@ int gwam_mlp_get_params_host(gwam_mlp* m, int layer, int which, float* W, float*
     // which: 0 master weights, 1 gradients of the last train step
     if (!m || layer < 1 || layer > m->nl || (which != 0 && which != 1)) return fail(m, GWAM_EINVAL, "bad arguments");
     const size_t Di = m->D[layer - 1], no = m->N[layer], ni = m->N[layer - 1];
+    // (straight into the caller's arrays: a copy that the runtime refuses there leaves no error behind for the wait)
+    cudaError_t rc = cudaSuccess;
     if (W)
-        cudaMemcpy2DAsync(W, ni * 4, which ? m->gW[layer] : m->W[layer], Di * 4, ni * 4, no, cudaMemcpyDeviceToHost, m->s);
-    if (b) cudaMemcpyAsync(b, which ? m->gb[layer] : m->b[layer], no * 4, cudaMemcpyDeviceToHost, m->s);
-    return cudaStreamSynchronize(m->s) == cudaSuccess ? GWAM_OK : fail(m, GWAM_ECUDA, "copy failed");
+        rc = cudaMemcpy2DAsync(W, ni * 4, which ? m->gW[layer] : m->W[layer], Di * 4, ni * 4, no, cudaMemcpyDeviceToHost, m->s);
+    if (b && rc == cudaSuccess) rc = cudaMemcpyAsync(b, which ? m->gb[layer] : m->b[layer], no * 4, cudaMemcpyDeviceToHost, m->s);
+    if (rc != cudaSuccess) cudaGetLastError();
+    const cudaError_t wait = cudaStreamSynchronize(m->s);
+    return rc == cudaSuccess && wait == cudaSuccess ? GWAM_OK : fail(m, GWAM_ECUDA, "copy failed");
 }
 
 int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, const int32_t* rows, int batch,
