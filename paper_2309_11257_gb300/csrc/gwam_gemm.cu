@@ -739,6 +739,9 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
                         }
                     }
                     if (!ok) break;
+                    // every lane has acquired its flag; a vote does not order memory, so the warp barrier makes
+                    // the rows behind all of them visible to lane 0, whose loads read them
+                    __syncwarp();
                     asm volatile("fence.proxy.async;" ::: "memory");
                 }
                 if (lane == 0) {
