@@ -432,6 +432,19 @@ int gwam_mlp_profile_enable(gwam_mlp *m, int enable);
 int gwam_mlp_profile_read(gwam_mlp *m, double *ms_host, int64_t *passes);
 /* Pending device status of the surrogate (synchronises). */
 int gwam_mlp_status(gwam_mlp *m);
+/* Self-tests of the surrogate's kernels (not in the paper).  gwam_selftest_hidden_plan: 1 when an inference chunk
+ * of `rows` rows runs all hidden layers in one kernel, 0 when every layer is a launch; *clusters (or NULL)
+ * receives the clusters of that kernel that are resident at once (256 rows a cluster at a time; 0: the
+ * width is not one of its own).  GWAM_EINVAL for bad arguments. */
+int gwam_selftest_hidden_plan(const gwam_mlp *m, int rows, int *clusters);
+/* The bounded device waits of that kernel (kernel = 0; rows as above, the plan must be 1) and of the weight gradients
+ * (kernel = 1; rows a multiple of 64), as gwam_selftest_gemm_timeout: launched on whatever the buffers hold with every
+ * wait limited to wait_us microseconds (1 .. 2 000 000) and the producers told to issue no copies (skip_copies = 1;
+ * for kernel 0: 1 the first, 2 the second, 3 both CTAs of each pair) or all (0).  A kernel that gives up waits
+ * (bounded) for the copies and MMAs that it issued and frees its tensor memory; the call returns GWAM_ETIMEOUT, or
+ * GWAM_OK when no wait ran out, and the context stays usable.  Activations and the stored gradients are
+ * overwritten, weights are not.  Synchronises. */
+int gwam_selftest_mlp_timeout(gwam_mlp *m, int kernel, int rows, int skip_copies, unsigned int wait_us);
 /* Fallback routing: copy the ray tracer's drag into the columns with mask[c] != 0 (device arrays,
  * [nlev][ncol] FP64). */
 int gwam_mlp_merge_fallback(const int32_t *mask, int64_t ncol, int nlev, const double *dudt_tracer,

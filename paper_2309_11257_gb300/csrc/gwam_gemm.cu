@@ -634,7 +634,9 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
 // in a layer's first tile W) of a stage has landed in both CTAs; empty: the MMAs have released the stage;
 // accf, acce: the accumulator is complete, drained by both CTAs.  done[w]: tiles that an epilogue warp of this
 // CTA (or of its counterpart in the other pair) has finished writing to global memory, which the next layer's
-// loads wait for.  Every wait is bounded; a CTA that gives up still meets the others at the end.
+// loads wait for.  Every wait is bounded; a CTA that gives up still meets the others at the end.  A pair may then
+// have issued different stages: sent tells the first CTA how far each came, which accounts for the bytes that
+// never left and waits (bounded) for the others before either leaves.
 constexpr int kHidStages = 4;
 constexpr int kHidMaxK = 512;
 constexpr int kHidEpi = 16;                          // epilogue warps
@@ -662,6 +664,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kStages], empty_bar[kStages], accf_bar[2], acce_bar[2], done_bar;
     __shared__ uint32_t done[kHidEpi * C / 2];
+    __shared__ int sent[3];   // blocks of W loaded ahead; stages; whether all of them have been released
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -671,6 +674,8 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
     // W (up to 8 blocks of 16 KB), A stages, staging boxes of the epilogue warps
     const uint32_t wbase = (saddr(smem_raw) + 1023u) & ~1023u;
     const uint32_t abase = wbase + (kHidMaxK / kBK) * kABytes, sbase = abase + kStages * kABytes;
+    const unsigned long long wlim = h.wait_ns ? h.wait_ns : kWaitNs;
+    const bool mute = (h.skip_copies >> half) & 1;   // self-test: this CTA of the pair issues no copies
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -708,7 +713,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(saddr(&full_bar[s])), "r"(bytes) : "memory");
     };
     // the first blocks of W, while the previous kernel still runs
-    const int pre = min(kStages, h.nk[0]);
+    const int pre = mute ? 0 : min(kStages, h.nk[0]);
     if (tid == 0)
         for (int i = 0; i < pre; ++i) {
             expect(i, 4 * kABytes);
@@ -718,8 +723,8 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
     bool ok = true;
 
     if (warp == 0) {
-        int it = 0;
-        for (int l = 0; l < h.n && ok; ++l) {
+        int it = 0, issued = 0;
+        for (int l = 0; l < h.n && ok && !mute; ++l) {
             const int nk = h.nk[l], nkp = l ? h.nk[l - 1] : kStages;
             for (int j = 0; j < tiles && ok; ++j) {
                 if (l > 0) {
@@ -733,7 +738,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
                         if (__all_sync(0xffffffffu, v >= want)) break;
                         const uint64_t t = __shfl_sync(0xffffffffu, gtime(), 0);
                         if (t0 == 0) t0 = t;
-                        else if (t - t0 > kWaitNs) {
+                        if (t - t0 > wlim || __any_sync(0xffffffffu, abort_flag != 0)) {
                             ok = false;
                             break;
                         }
@@ -749,10 +754,10 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
                     for (int i = 0; i < nk; ++i) {
                         const int q = it + i, s = q % kStages, p = q - nkp;
                         const uint32_t fb = cluster_addr(saddr(&full_bar[s]), lead);
-                        if ((q >= kStages && !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((q / kStages - 1) & 1), kWaitNs)) ||
+                        if ((q >= kStages && !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((q / kStages - 1) & 1), wlim)) ||
                             // the block of W that this one replaces may be read by a later stage than that
                             (l > 0 && j == 0 && nkp < kStages && i < nkp &&
-                             !mbar_wait(saddr(&empty_bar[p % kStages]), (uint32_t)((p / kStages) & 1), kWaitNs)) ||
+                             !mbar_wait(saddr(&empty_bar[p % kStages]), (uint32_t)((p / kStages) & 1), wlim)) ||
                             abort_flag) {
                             ok = false;
                             break;
@@ -763,6 +768,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
                             load(wbase + (uint32_t)i * kABytes, h.b[l], i * kBK, rank * 128, fb);
                         }
                         load(abase + (uint32_t)s * kABytes, h.a[l], i * kBK, row, fb);
+                        issued = q + 1;
                     }
                 }
                 ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
@@ -773,7 +779,10 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
             if (!ok) abort_flag = 1;
             // the last stages' copies have landed and their release has arrived
             for (int i = it > kStages ? it - kStages : 0; i < it && ok; ++i)
-                ok = mbar_wait(saddr(&empty_bar[i % kStages]), (uint32_t)((i / kStages) & 1), kWaitNs);
+                ok = mbar_wait(saddr(&empty_bar[i % kStages]), (uint32_t)((i / kStages) & 1), wlim);
+            sent[0] = pre;
+            sent[1] = issued;
+            sent[2] = ok;
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -792,7 +801,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
                 const int nk = h.nk[l];
                 for (int j = 0; j < tiles && ok; ++j, ++tl) {
                     const int acc = tl & 1;
-                    if (tl >= 2 && !mbar_wait<true>(saddr(&acce_bar[acc]), (uint32_t)((tl / 2 - 1) & 1), kWaitNs)) {
+                    if (tl >= 2 && !mbar_wait<true>(saddr(&acce_bar[acc]), (uint32_t)((tl / 2 - 1) & 1), wlim)) {
                         ok = false;
                         break;
                     }
@@ -800,7 +809,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
                     for (int i = 0; i < nk; ++i, ++it) {
                         const int s = it % kStages;
                         const uint32_t ph = (uint32_t)((it / kStages) & 1);
-                        if (abort_flag || !mbar_wait<true>(saddr(&full_bar[s]), ph, kWaitNs)) {
+                        if (abort_flag || !mbar_wait<true>(saddr(&full_bar[s]), ph, wlim)) {
                             ok = false;
                             break;
                         }
@@ -845,7 +854,7 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
             const float4* bias = reinterpret_cast<const float4*>(h.bias[l] + n0);
             for (int j = 0; j < tiles; ++j, ++tl) {
                 const int acc = tl & 1, row0 = (cluster + j * clusters) * kRows + half * kBM + q * 32;
-                const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((tl / 2) & 1), kWaitNs);
+                const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((tl / 2) & 1), wlim);
                 if (!__all_sync(0xffffffffu, got) || abort_flag) {
                     ok = false;
                     break;
@@ -903,11 +912,45 @@ __global__ void __launch_bounds__(64 + 32 * kHidEpi, 1) k_hidden(const __grid_co
         __syncwarp();
         if (!ok) abort_flag = 1;
     }
+    // (what is in flight is waited for with the full limit, also when a test has cut the others short)
     const bool fin = mbar_wait(saddr(&done_bar), 0u, kWaitNs);
     if (!__syncthreads_and(ok && fin) && tid == 0 && err) atomicOr(err, 1);
     tc_before();
     cluster_sync();   // nobody reads the accumulators or writes to another CTA's shared memory any more
     tc_after();
+    if (half == 0 && tid == 0) {
+        auto theirs = [&](int q) {
+            int v;
+            asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cluster_addr(saddr(&sent[q]), lead + 1)) : "memory");
+            return v;
+        };
+        if (!sent[2] || !theirs(2)) {
+            // copies may be in flight: stage q's barrier completes once the bytes of both CTAs have arrived, those
+            // that a CTA did not get to (A from stage[r] on, W in a layer's first tile unless loaded ahead) counted
+            // as arrived here.  A CTA is at most kStages stages ahead of the other, so no earlier one is open.
+            const int ahead[2] = {sent[0], theirs(0)}, stage[2] = {sent[1], theirs(1)};
+            auto first_tile = [&](int q) {
+                int l = 0;
+                for (; l + 1 < h.n && q >= h.nk[l] * tiles; ++l) q -= h.nk[l] * tiles;
+                return q < h.nk[l];
+            };
+            const int end = max(max(stage[0], stage[1]), max(ahead[0], ahead[1]));
+            for (int q = min(stage[0], stage[1]); q < end; ++q) {
+                const bool w = first_tile(q);
+                uint32_t missing = 0;
+                for (int r = 0; r < 2; ++r)
+                    if (q >= stage[r]) missing += w && q >= ahead[r] ? 2 * kABytes : kABytes;
+                if (q >= stage[0] && q >= ahead[0]) expect(q % kStages, (w ? 4 : 2) * kABytes);
+                asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(
+                                 cluster_addr(saddr(&full_bar[q % kStages]), lead)),
+                             "r"(missing)
+                             : "memory");
+            }
+            for (int q = max(0, end - kStages); q < end; ++q)
+                mbar_wait<true>(saddr(&full_bar[q % kStages]), (uint32_t)((q / kStages) & 1), kWaitNs);
+        }
+    }
+    __syncwarp();
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
     cluster_sync();
 }
@@ -960,6 +1003,7 @@ __global__ void __launch_bounds__(64 + 32 * kGradEpi, 1) k_grad_update(const __g
     tc_after();
     const uint32_t tmem = tmem_slot;
     const int total = G.end[G.n - 1], kb = K / kBK;
+    const unsigned long long wlim = G.wait_ns ? G.wait_ns : kWaitNs;
     float* const tile = reinterpret_cast<float*>(smem_raw + (base - saddr(smem_raw)) + kGradStages * kGradStage);
     auto epi_sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(32 * kGradEpi) : "memory"); };   // the epilogue warps
     bool ok = true;
@@ -976,13 +1020,13 @@ __global__ void __launch_bounds__(64 + 32 * kGradEpi, 1) k_grad_update(const __g
     if (warp == 0) {
         if (lane == 0) {
             int it = 0;
-            for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+            for (int t = blockIdx.x; t < total && ok && !G.skip_copies; t += gridDim.x) {
                 int j, m0, n0;
                 decode(t, j, m0, n0);
                 for (int i = 0; i < kb; ++i, ++it) {
                     const int s = it % kGradStages;
                     if ((it >= kGradStages &&
-                         !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((it / kGradStages - 1) & 1), kWaitNs)) ||
+                         !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((it / kGradStages - 1) & 1), wlim)) ||
                         abort_flag) {
                         ok = false;
                         break;
@@ -1020,14 +1064,14 @@ __global__ void __launch_bounds__(64 + 32 * kGradEpi, 1) k_grad_update(const __g
                 for (int z = 0; z < G.S[j] && ok; ++z, ++sl) {
                     const int acc = sl % kGradAcc;
                     if (sl >= kGradAcc &&
-                        !mbar_wait(saddr(&acce_bar[acc]), (uint32_t)((sl / kGradAcc - 1) & 1), kWaitNs)) {
+                        !mbar_wait(saddr(&acce_bar[acc]), (uint32_t)((sl / kGradAcc - 1) & 1), wlim)) {
                         ok = false;
                         break;
                     }
                     tc_after();
                     for (int i = 0; i < nk; ++i, ++it) {
                         const int s = it % kGradStages;
-                        if (abort_flag || !mbar_wait(saddr(&full_bar[s]), (uint32_t)((it / kGradStages) & 1), kWaitNs)) {
+                        if (abort_flag || !mbar_wait(saddr(&full_bar[s]), (uint32_t)((it / kGradStages) & 1), wlim)) {
                             ok = false;
                             break;
                         }
@@ -1075,7 +1119,7 @@ __global__ void __launch_bounds__(64 + 32 * kGradEpi, 1) k_grad_update(const __g
 #pragma unroll 1
             for (int z = 0; z < G.S[j]; ++z, ++sl) {
                 const int acc = sl % kGradAcc;
-                const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((sl / kGradAcc) & 1), kWaitNs);
+                const bool got = mbar_wait(saddr(&accf_bar[acc]), (uint32_t)((sl / kGradAcc) & 1), wlim);
                 if (!__all_sync(0xffffffffu, got) || abort_flag) {
                     ok = false;
                     break;
@@ -1355,13 +1399,15 @@ bool hidden_launch(const HiddenSet& h, int M, int* err, cudaStream_t s)
 
 }  // namespace
 
+int gemm_hidden_clusters(int N) { return N == 256 ? hidden_clusters<2>() : N == 512 ? hidden_clusters<4>() : 0; }
+
 bool gemm_hidden_fits(int M, int N, int K0)
 {
-    if ((N != 256 && N != 512) || M < 1 || K0 < kBK || K0 > kHidMaxK || K0 % kBK) return false;
+    if (M < 1 || K0 < kBK || K0 > kHidMaxK || K0 % kBK) return false;
     // With fewer row tiles than 0.6 of the clusters the smaller tiles of k_gemm_bf16 spread better over the SMs
     // (4 x 512: 5000 rows 53.7 us here, 53.1 there; 9000 rows 58 and 63; 18 000 rows 74 and 89; 4 x 256: 9500
     // rows 50 and 47, 12 000 rows 59 and 62; the whole inference each time).
-    const int clusters = N == 256 ? hidden_clusters<2>() : hidden_clusters<4>();
+    const int clusters = gemm_hidden_clusters(N);
     return clusters > 0 && 5LL * ((M + 2 * kBM - 1) / (2 * kBM)) >= 3LL * clusters;
 }
 

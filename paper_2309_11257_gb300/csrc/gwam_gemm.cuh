@@ -94,6 +94,8 @@ struct GradSet {
     int end[kGradMax];                        // tiles of jobs 0 .. j (filled in by the launch)
     int n;
     Adam adam;
+    unsigned long long wait_ns;   // as in GemmEpi
+    int skip_copies;              // self-test of the give-up path only: the producer issues no copies
 };
 bool gemm_bf16_grad_launch(GradSet& set, int K, int* err, cudaStream_t s);
 
@@ -116,8 +118,12 @@ struct HiddenSet {
     const float* bias[kHiddenMax];
     int nk[kHiddenMax];
     int n;
+    unsigned long long wait_ns;   // as in GemmEpi
+    int skip_copies;              // self-test of the give-up path only: bit r -- CTA r of each pair issues no copies
 };
 bool gemm_hidden_fits(int M, int N, int K0);
+// clusters of gemm_hidden_launch that are resident at once for N outputs a layer (0: N is not one of its widths)
+int gemm_hidden_clusters(int N);
 bool gemm_hidden_launch(const HiddenSet& h, int M, int N, int* err, cudaStream_t s);
 
 // The tile width gemm_bf16_launch uses when bn = 0 (the caller builds tb with this box): the one with

@@ -385,6 +385,30 @@ int wgrad_split(const gwam_mlp* m, int l, int B)
     return S;
 }
 
+gwam::GradSet grad_set(const gwam_mlp* m, int B, const gwam::Adam& adam)
+{
+    gwam::GradSet g{};
+    for (int l = 1; l <= m->nl; ++l) {
+        const int j = l - 1;
+        g.ta[j] = m->tw_a[l];
+        g.tb[j] = m->tw_b[l];
+        g.g[j] = m->gW[l];
+        g.W[j] = m->W[l];
+        g.m[j] = m->mW[l];
+        g.v[j] = m->vW[l];
+        g.Wb[j] = m->Wb[l];
+        g.WbT[j] = m->WbT[l];
+        g.M[j] = m->D[l];
+        g.N[j] = m->D[l - 1];
+        g.n_o[j] = m->N[l];
+        g.n_i[j] = m->N[l - 1];
+        g.S[j] = wgrad_split(m, l, B);
+    }
+    g.n = m->nl;
+    g.adam = adam;
+    return g;
+}
+
 uint64_t host_splitmix(uint64_t& state)
 {
     uint64_t z = (state += 0x9E3779B97F4A7C15ull);
@@ -720,24 +744,11 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
         const long long t = lr > 0 ? m->t + 1 : std::max(1ll, m->t);
         const gwam::Adam adam{lr, m->b1, m->b2, m->eps, (float)(1.0 - std::pow((double)m->b1, (double)t)),
                               (float)(1.0 - std::pow((double)m->b2, (double)t))};
-        gwam::GradSet g{};
         BiasSet u{};
         int outputs = 0;
         for (int l = 1; l <= L; ++l) {
             const int j = l - 1;
-            g.ta[j] = m->tw_a[l];
-            g.tb[j] = m->tw_b[l];
-            g.g[j] = m->gW[l];
-            g.W[j] = m->W[l];
-            g.m[j] = m->mW[l];
-            g.v[j] = m->vW[l];
-            g.Wb[j] = m->Wb[l];
-            g.WbT[j] = m->WbT[l];
-            g.M[j] = m->D[l];
-            g.N[j] = m->D[l - 1];
-            g.n_o[j] = u.n_o[j] = m->N[l];
-            g.n_i[j] = m->N[l - 1];
-            g.S[j] = wgrad_split(m, l, B);
+            u.n_o[j] = m->N[l];
             u.dzT[j] = m->dzT[l];
             u.gb[j] = m->gb[l];
             u.b[j] = m->b[l];
@@ -745,10 +756,11 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
             u.vb[j] = m->vb[l];
             u.end[j] = outputs += m->D[l];
         }
-        g.n = u.nl = L;
+        u.nl = L;
         u.ld = m->max_batch;
         u.B = B;
-        g.adam = u.adam = adam;
+        u.adam = adam;
+        gwam::GradSet g = grad_set(m, B, adam);
         ok = gwam::gemm_bf16_grad_launch(g, B, m->err, m->s) &&
              launch_pdl(k_bias_update, dim3((outputs + 7) / 8), dim3(256), m->s, true, u);
     }
@@ -845,6 +857,40 @@ int gwam_mlp_status(gwam_mlp* m)
 {
     if (!m) return GWAM_EINVAL;
     return check_err(m);
+}
+
+int gwam_selftest_hidden_plan(const gwam_mlp* m, int rows, int* clusters)
+{
+    if (!m || rows < 1 || rows > m->max_batch) return GWAM_EINVAL;
+    if (clusters) *clusters = gwam::gemm_hidden_clusters(m->D[1]);
+    return m->nl > 1 && gwam::gemm_hidden_fits(rows, m->D[1], m->D[0]);
+}
+
+int gwam_selftest_mlp_timeout(gwam_mlp* m, int kernel, int rows, int skip_copies, unsigned int wait_us)
+{
+    if (!m || kernel < 0 || kernel > 1 || rows < 1 || rows > m->max_batch || wait_us < 1 || wait_us > 2000000u ||
+        skip_copies < 0 || skip_copies > (kernel ? 1 : 3) || (kernel ? rows % 64 != 0 : gwam_selftest_hidden_plan(m, rows, nullptr) != 1))
+        return fail(m, GWAM_EINVAL, "bad arguments");
+    int* err = nullptr;
+    if (cudaMallocAsync((void**)&err, sizeof(int), m->s) != cudaSuccess) return fail(m, GWAM_ENOMEM, "scratch");
+    cudaMemsetAsync(err, 0, sizeof(int), m->s);
+    bool ok;
+    if (kernel) {
+        gwam::GradSet g = grad_set(m, rows, gwam::Adam{});   // lr = 0: gradients only
+        g.wait_ns = 1000ull * wait_us;
+        g.skip_copies = skip_copies;
+        ok = gwam::gemm_bf16_grad_launch(g, rows, err, m->s);
+    } else {
+        gwam::HiddenSet h = m->hidden;
+        h.wait_ns = 1000ull * wait_us;
+        h.skip_copies = skip_copies;
+        ok = gwam::gemm_hidden_launch(h, rows, m->D[1], err, m->s);
+    }
+    int h = 0;
+    cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, m->s);
+    cudaFreeAsync(err, m->s);
+    if (cudaStreamSynchronize(m->s) != cudaSuccess || !ok) return fail(m, GWAM_ECUDA, "kernel launch failed");
+    return h ? fail(m, GWAM_ETIMEOUT, "a bounded wait gave up") : GWAM_OK;
 }
 
 int gwam_mlp_merge_fallback(const int32_t* mask, int64_t ncol, int nlev, const double* dudt_tracer,

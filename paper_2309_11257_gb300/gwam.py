@@ -140,6 +140,8 @@ SIGNATURES = {
     "gwam_mlp_output_host": (C.c_int, [_vp, _vp, C.c_int]),
     "gwam_mlp_infer": (C.c_int, [_vp, _vp, C.c_int64, _vp, _vp, _vp, _vp]),
     "gwam_mlp_status": (C.c_int, [_vp]),
+    "gwam_selftest_hidden_plan": (C.c_int, [_vp, C.c_int, _P(C.c_int)]),
+    "gwam_selftest_mlp_timeout": (C.c_int, [_vp, C.c_int, C.c_int, C.c_int, C.c_uint]),
     "gwam_mlp_profile_enable": (C.c_int, [_vp, C.c_int]),
     "gwam_mlp_profile_read": (C.c_int, [_vp, _vp, _P(C.c_int64)]),
     "gwam_mlp_merge_fallback": (C.c_int, [_vp, C.c_int64, C.c_int, _vp, _vp, _vp, _vp, _vp]),
