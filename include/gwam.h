@@ -384,8 +384,8 @@ typedef struct {
     float beta1, beta2, eps;   /* Adam constants (0.9, 0.999, 1e-8) */
 } gwam_mlp_config;
 
-/* Create / destroy.  Allocates every buffer (weights, Adam state, activations of max_batch rows,
- * split-K scratch) and the TMA tensor maps once.  GWAM_EINVAL, GWAM_ENOMEM, GWAM_ECUDA. */
+/* Create / destroy.  Allocates every buffer (weights, Adam state, activations of max_batch rows)
+ * and the TMA tensor maps once.  GWAM_EINVAL, GWAM_ENOMEM, GWAM_ECUDA. */
 int gwam_mlp_create(gwam_mlp **out, const gwam_mlp_config *cfg, void *stream);
 void gwam_mlp_destroy(gwam_mlp *m);
 const char *gwam_mlp_last_error(const gwam_mlp *m);

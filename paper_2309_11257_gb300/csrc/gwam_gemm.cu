@@ -105,8 +105,7 @@ __device__ __forceinline__ float erf_abs(float z, float& e)
     return fmaf(-(t * poly), e, 1.0f);
 }
 
-// GELU(z) = z Phi(z) = z / 2 + |z| erf(|z| / sqrt 2) / 2
-// GELU of two values, z (1 + erf(z / sqrt 2)) / 2, in packed instructions (half the issue slots); the steps
+// GELU(z) = z Phi(z) = z / 2 + |z| erf(|z| / sqrt 2) / 2 of two values in packed instructions (half the issue slots); the steps
 // of erf_abs, with the polynomial's coefficients negated for its negated value.
 __device__ __forceinline__ float2 gelu2(float2 z)
 {
@@ -166,7 +165,7 @@ __device__ __forceinline__ double sum_squares(const float (&d)[32])
 // and 124 us).  Rows >= M only skip the stores.  zz: the prefetched
 // pre-activations of EPI_BWD.
 template <int MODE>
-__device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, float (&v)[32], const float* sbias,
+__device__ __forceinline__ void epi32(const GemmEpi& e, int row, int nb, float (&v)[32], const float* sbias,
                                       const float (&zz)[32], int rowmask, double& sq, uint32_t stg,
                                       int cc0)
 {
@@ -272,7 +271,7 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int z, int row, int nb, 
     }
     if (!live) return;
     if (MODE == EPI_STORE && e.cf) {
-        float* p = e.cf + (size_t)z * e.cf_slice + (size_t)row * e.ldcf + nb;
+        float* p = e.cf + (size_t)row * e.ldcf + nb;
         if (full && (e.ldcf & 3) == 0) {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
@@ -355,11 +354,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, uint32_t (&rr)[16])
 // tile i into accumulator i % 2; warps 2 .. 2+EPW-1 drain accumulator (i % 2) while the MMAs of tile
 // i + 1 run into the other one.  Epilogue warp w reads TMEM lane quarter w % 4 and, with EPW / 4
 // warps per quarter, its share of the columns.  Tiles t = blockIdx.x, blockIdx.x + gridDim.x, ...
-// over (k slice, m tile, n tile), n fastest.
+// over (m tile, n tile), n fastest.
 template <int BN, int ST, int EPW, int MODE>
 __global__ void __launch_bounds__(64 + 32 * EPW, 1)
     k_gemm_bf16(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-                const __grid_constant__ CUtensorMap tc, int K, int ksplit, GemmEpi e)
+                const __grid_constant__ CUtensorMap tc, int K, GemmEpi e)
 {
     constexpr uint32_t kBBytes = BN * kBK * 2;
     constexpr uint32_t kStage = kABytes + kBBytes;   // a multiple of 1024
@@ -376,9 +375,8 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n_tiles = (e.N + BN - 1) / BN, m_tiles = (e.M + kBM - 1) / kBM;
-    const int per_slice = n_tiles * m_tiles;
-    const int total = per_slice * ksplit;
-    const int nk = K / kBK / ksplit;
+    const int total = n_tiles * m_tiles;
+    const int nk = K / kBK;
     const uint32_t base = (saddr(smem_raw) + 1023u) & ~1023u;
 
     if (warp == 1) {
@@ -436,8 +434,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
             // (self-test of the give-up path: no copy is issued, so the MMA and epilogue warps wait
             // on stages that never fill and give up after wait_ns)
             for (int t = blockIdx.x; t < total && ok && !e.skip_copies; t += gridDim.x) {
-                const int z = t / per_slice, r = t - z * per_slice;
-                const int m0 = (r / n_tiles) * kBM, n0 = (r % n_tiles) * BN;
+                const int m0 = (t / n_tiles) * kBM, n0 = (t % n_tiles) * BN;
                 for (int i = 0; i < nk; ++i, ++it) {
                     const int s = it % ST;
                     if (it >= ST && !mbar_wait(saddr(&empty_bar[s]), (uint32_t)((it / ST - 1) & 1), wlim)) {
@@ -450,7 +447,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
                     }
                     const uint32_t fb = saddr(&full_bar[s]);
                     const uint32_t dA = base + (uint32_t)s * kStage, dB = dA + kABytes;
-                    const int kx = (z * nk + i) * kBK;
+                    const int kx = i * kBK;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(kStage)
                                  : "memory");
                     asm volatile(
@@ -526,8 +523,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
         int tl = 0;
         for (int t = blockIdx.x; t < total; t += gridDim.x, ++tl) {
             const int acc = tl & 1;
-            const int z = t / per_slice, r = t - z * per_slice;
-            const int m0 = (r / n_tiles) * kBM, n0 = (r % n_tiles) * BN;
+            const int m0 = (t / n_tiles) * kBM, n0 = (t % n_tiles) * BN;
             const int row = m0 + q * 32 + lane;
             const int cbeg = n0 + part * kColsPerWarp;
             const int rowmask = ((MODE == EPI_DRAG || MODE == EPI_DRAG_WIDE) && row < e.M) ? e.mask[row] : 0;
@@ -579,7 +575,7 @@ __global__ void __launch_bounds__(64 + 32 * EPW, 1)
                 for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(rr[j]);
                 const uint32_t stg =
                     e.tstore ? stg_warp + (uint32_t)((32 * k) / 64) * 4096u + (uint32_t)lane * 128u : 0u;
-                epi32<MODE>(e, z, row, nb, v, sbias, zz, rowmask, sq, stg, ((32 * k) % 64) / 8);
+                epi32<MODE>(e, row, nb, v, sbias, zz, rowmask, sq, stg, ((32 * k) % 64) / 8);
             }
             tc_before();
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&acce_bar[acc])) : "memory");
@@ -1228,13 +1224,13 @@ struct GemmShape {
 constexpr GemmShape kGemmShapes[] = {{256, 3, 16}, {192, 4, 12}, {128, 5, 8}, {64, 8, 4}};
 
 template <int BN, int ST, int EPW, int MODE>
-bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int K, int ksplit,
-                 const GemmEpi& e, cudaStream_t s)
+bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int K, const GemmEpi& e,
+                 cudaStream_t s)
 {
     static_assert(BN / (EPW / 4) == 64, "a warp's staging box");
     const size_t shm = gemm_smem(BN, ST, EPW, e.N, e.bias ? (MODE == EPI_DRAG ? 3 : 1) : 0, e.tstore);
     if (shm > kGemmMaxSmem)
-        return MODE == EPI_DRAG ? launch_mode<BN, ST, EPW, MODE == EPI_DRAG ? (int)EPI_DRAG_WIDE : MODE>(ta, tb, tc, K, ksplit, e, s)
+        return MODE == EPI_DRAG ? launch_mode<BN, ST, EPW, MODE == EPI_DRAG ? (int)EPI_DRAG_WIDE : MODE>(ta, tb, tc, K, e, s)
                                 : false;
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1247,7 +1243,7 @@ bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap
             return false;
         configured[dev] = shm;
     }
-    const long long tiles = (long long)((e.N + BN - 1) / BN) * ((e.M + kBM - 1) / kBM) * ksplit;
+    const long long tiles = (long long)((e.N + BN - 1) / BN) * ((e.M + kBM - 1) / kBM);
     const int grid = (int)std::min<long long>(tiles, gemm_sm_count());
     // launched with programmatic stream serialisation: the set-up of this GEMM (barriers, tensor
     // memory) overlaps the tail of the kernel before it, which it waits for before its first read
@@ -1261,21 +1257,20 @@ bool launch_mode(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gemm_bf16<BN, ST, EPW, MODE>, ta, tb, tc, K, ksplit, e) == cudaSuccess;
+    return cudaLaunchKernelEx(&cfg, k_gemm_bf16<BN, ST, EPW, MODE>, ta, tb, tc, K, e) == cudaSuccess;
 }
 
 // one kernel per epilogue mode: each holds only its own epilogue code (a smaller instruction
 // footprint for the epilogue warps, whose instruction fetch otherwise stalls them)
 template <int SHAPE>
-bool launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int K, int ksplit, const GemmEpi& e,
-            cudaStream_t s)
+bool launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, int K, const GemmEpi& e, cudaStream_t s)
 {
     constexpr GemmShape g = kGemmShapes[SHAPE];
     switch (e.mode) {
-    case EPI_STORE: return launch_mode<g.bn, g.stages, g.warps, EPI_STORE>(ta, tb, tc, K, ksplit, e, s);
-    case EPI_BWD: return launch_mode<g.bn, g.stages, g.warps, EPI_BWD>(ta, tb, tc, K, ksplit, e, s);
-    case EPI_LOSS: return launch_mode<g.bn, g.stages, g.warps, EPI_LOSS>(ta, tb, tc, K, ksplit, e, s);
-    case EPI_DRAG: return launch_mode<g.bn, g.stages, g.warps, EPI_DRAG>(ta, tb, tc, K, ksplit, e, s);
+    case EPI_STORE: return launch_mode<g.bn, g.stages, g.warps, EPI_STORE>(ta, tb, tc, K, e, s);
+    case EPI_BWD: return launch_mode<g.bn, g.stages, g.warps, EPI_BWD>(ta, tb, tc, K, e, s);
+    case EPI_LOSS: return launch_mode<g.bn, g.stages, g.warps, EPI_LOSS>(ta, tb, tc, K, e, s);
+    case EPI_DRAG: return launch_mode<g.bn, g.stages, g.warps, EPI_DRAG>(ta, tb, tc, K, e, s);
     default: return false;
     }
 }
@@ -1449,12 +1444,10 @@ bool gemm_bf16_grad_launch(GradSet& g, int K, int* err, cudaStream_t s)
     return cudaLaunchKernelEx(&cfg, k_grad_update, g, K, err) == cudaSuccess;
 }
 
-bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ksplit,
+bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn,
                       const GemmEpi& e_in, cudaStream_t s)
 {
-    if (e_in.M < 1 || e_in.N < 1 || K < kBK || K % kBK || ksplit < 1 || (K / kBK) % ksplit || ksplit > 65535)
-        return false;
-    if (ksplit > 1 && e_in.mode != EPI_STORE) return false;
+    if (e_in.M < 1 || e_in.N < 1 || K < kBK || K % kBK) return false;
     GemmEpi e = e_in;
     e.tstore = (tc && e.cb) ? 1 : 0;
     static const CUtensorMap none{};
@@ -1462,10 +1455,10 @@ bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtens
     if (bn == 0) bn = gemm_pick_bn(e.M, e.N, e.bias != nullptr, e.tstore != 0);
     static_assert(kGemmShapes[0].bn == 256 && kGemmShapes[1].bn == 192 && kGemmShapes[2].bn == 128 && kGemmShapes[3].bn == 64);
     switch (bn) {
-    case 256: return launch<0>(ta, tb, tcm, K, ksplit, e, s);
-    case 192: return launch<1>(ta, tb, tcm, K, ksplit, e, s);
-    case 128: return launch<2>(ta, tb, tcm, K, ksplit, e, s);
-    case 64: return launch<3>(ta, tb, tcm, K, ksplit, e, s);
+    case 256: return launch<0>(ta, tb, tcm, K, e, s);
+    case 192: return launch<1>(ta, tb, tcm, K, e, s);
+    case 128: return launch<2>(ta, tb, tcm, K, e, s);
+    case 64: return launch<3>(ta, tb, tcm, K, e, s);
     default: return false;
     }
 }
@@ -1506,7 +1499,7 @@ int gemm_selftest(const void* A, const void* B, int M, int N, int K, const float
     e.err = err;
     e.wait_ns = wait_ns;
     e.skip_copies = skip_copies;
-    const bool launched = gwam::gemm_bf16_launch(ta, tb, have_tc ? &tc : nullptr, K, use_bn, 1, e, s);
+    const bool launched = gwam::gemm_bf16_launch(ta, tb, have_tc ? &tc : nullptr, K, use_bn, e, s);
     int h = 0;
     cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaFreeAsync(err, s);

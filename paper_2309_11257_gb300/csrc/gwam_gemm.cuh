@@ -36,9 +36,8 @@ struct GemmEpi {
     int act;                  // EPI_STORE: apply GELU
     int M, N;                 // valid rows and columns of C
     const float* bias;        // [N] or null
-    float* cf;                // FP32 [M][ldcf] (+ blockIdx.z * cf_slice for split-K partials)
+    float* cf;                // FP32 [M][ldcf]
     int ldcf;
-    long long cf_slice;
     __nv_bfloat16* cb;        // BF16 [M][ldcb]
     int ldcb;
     __nv_bfloat16* ct;        // BF16 transposed [N][ldct]
@@ -99,12 +98,11 @@ struct GradSet {
 };
 bool gemm_bf16_grad_launch(GradSet& set, int K, int* err, cudaStream_t s);
 
-// Launch: A described by ta (box rows 128), B by tb (box rows bn); K a multiple of 64, split into
-// ksplit slices along K (K / 64 must be divisible by ksplit).  tc (or null): tensor map of the BF16
-// output cb (box 64 columns x 32 rows) -- the epilogue then stages each warp's rows in shared memory
+// Launch: A described by ta (box rows 128), B by tb (box rows bn); K a multiple of 64.  tc (or null): tensor map
+// of the BF16 output cb (box 64 columns x 32 rows) -- the epilogue then stages each warp's rows in shared memory
 // and writes them with TMA stores.  bn = 0 picks the tile width (gemm_pick_bn).  false on an unsupported
 // shape.
-bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ksplit,
+bool gemm_bf16_launch(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn,
                       const GemmEpi& e, cudaStream_t s);
 
 // All hidden layers of the inference, act_l = GELU(act_(l-1) . W_l^T + bias_l) in BF16, in one kernel with the

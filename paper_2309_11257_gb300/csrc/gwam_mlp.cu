@@ -443,11 +443,11 @@ int check_err(gwam_mlp* m)
     return GWAM_OK;
 }
 
-bool gemm(gwam_mlp* m, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn, int ks,
+bool gemm(gwam_mlp* m, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap* tc, int K, int bn,
           gwam::GemmEpi e)
 {
     e.err = m->err;
-    return gwam::gemm_bf16_launch(ta, tb, tc, K, bn, ks, e, m->s);
+    return gwam::gemm_bf16_launch(ta, tb, tc, K, bn, e, m->s);
 }
 
 // forward through every layer for B rows of act[0]; last layer per `last`
@@ -473,7 +473,7 @@ bool forward(gwam_mlp* m, int B, bool train, const gwam::GemmEpi& last)
             e.ldct = m->max_batch;
         }
         const int bn = gwam::gemm_pick_bn(B, m->D[l], true, true);
-        if (!gemm(m, m->tf_a[l], m->tf_b[l][bn / 64 - 1], &m->to_act[l], m->D[l - 1], bn, 1, e)) return false;
+        if (!gemm(m, m->tf_a[l], m->tf_b[l][bn / 64 - 1], &m->to_act[l], m->D[l - 1], bn, e)) return false;
     }
     gwam::GemmEpi e = last;
     e.M = B;
@@ -481,7 +481,7 @@ bool forward(gwam_mlp* m, int B, bool train, const gwam::GemmEpi& last)
     e.bias = m->b[m->nl];
     const int bn = gwam::gemm_pick_bn(B, e.N, true, e.cb != nullptr);
     return gemm(m, m->tf_a[m->nl], m->tf_b[m->nl][bn / 64 - 1], e.cb ? &m->to_dz[m->nl] : nullptr, m->D[m->nl - 1],
-                bn, 1, e);
+                bn, e);
 }
 
 }  // namespace
@@ -736,7 +736,7 @@ int gwam_mlp_train_step(gwam_mlp* m, const float* X, const float* Y, int64_t n, 
         x.ct = m->dzT[l - 1];
         x.ldct = m->max_batch;
         const int bn = gwam::gemm_pick_bn(B, x.N, false, true);
-        ok = gemm(m, m->tx_a[l], m->tx_b[l][bn / 64 - 1], &m->to_dz[l - 1], m->D[l], bn, 1, x);
+        ok = gemm(m, m->tx_a[l], m->tx_b[l][bn / 64 - 1], &m->to_dz[l - 1], m->D[l], bn, x);
     }
     // then the weight gradients of all layers, dW_l = dz_l^T act_{l-1}, with the weight updates in one
     // launch and the biases in one: with a GEMM, a row sum and two updates per layer a step was 33 launches
