@@ -131,28 +131,30 @@ __device__ __forceinline__ float gelu_grad(float z)
 
 // Sum of the squares of 32 errors, as accurate as the FP64 sum and over its whole range.  FP64 additions and
 // conversions of every element (1/64 of the FP32 rate) had made this kernel 55 us: the exact products
-// (hi, lo) go into an unevaluated sum of three FP32 numbers, the errors of the two larger ones carried into the
-// next, and only the three results are added in FP64 (relative error about 2^-53; a double-float sum, 48 bits, was
-// 1e-14 off after 64 elements).  Products that FP32 cannot hold exactly -- a non-zero error outside 2^-50 .. 2^60,
-// infinities -- take FP64 throughout.
+// (hi, lo) go into unevaluated sums of three FP32 numbers, even and odd columns in the halves of packed pairs, the
+// errors of the two larger ones carried into the next, and only the results are added in FP64 (relative error about
+// 2^-53; a double-float sum, 48 bits, was 1e-14 off after 64 elements).  Where FP32 cannot hold the products to that
+// -- an error beyond 2^60, a sum below 2^-90, infinities -- every one is formed in FP64.
 __device__ __forceinline__ double sum_squares(const float (&d)[32])
 {
-    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, most = 0.0f, least = 1.0f;
-    auto two_sum = [](float& s, float x) {
-        const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+    float2 s0 = dup2(0.0f), s1 = s0, s2 = s0;
+    float most = 0.0f;
+    auto two_sum = [](float2& s, float2 x) {
+        const float2 t = add2(s, x), b = sub2(t, s);
+        const float2 e = add2(sub2(s, sub2(t, b)), sub2(x, b));
         s = t;
         return e;
     };
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const DF p = df_prod(d[j], d[j]);
-        const float e0 = two_sum(s0, p.hi);
-        s2 = __fadd_rn(s2, __fadd_rn(two_sum(s1, e0), two_sum(s1, p.lo)));
-        most = fmaxf(most, fabsf(d[j]));
-        least = fminf(least, d[j] == 0.0f ? 1.0f : fabsf(d[j]));
+    for (int j = 0; j < 32; j += 2) {
+        const DF p = df_prod(d[j], d[j]), q = df_prod(d[j + 1], d[j + 1]);
+        const float2 e = two_sum(s0, make_float2(p.hi, q.hi));
+        const float2 f = two_sum(s1, e);
+        s2 = add2(s2, add2(f, two_sum(s1, make_float2(p.lo, q.lo))));
+        most = fmaxf(most, fmaxf(fabsf(d[j]), fabsf(d[j + 1])));
     }
-    if (most <= 0x1p60f && least >= 0x1p-50f) return widen(s0) + (widen(s1) + widen(s2));
+    if (most <= 0x1p60f && (s0.x + s0.y >= 0x1p-90f || most == 0.0f))
+        return (widen(s0.x) + widen(s0.y)) + ((widen(s1.x) + widen(s1.y)) + widen(s2.x + s2.y));
     double q = 0.0;
 #pragma unroll
     for (int j = 0; j < 32; ++j) q = fma((double)d[j], (double)d[j], q);
