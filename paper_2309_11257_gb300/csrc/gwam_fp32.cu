@@ -48,7 +48,7 @@ void convert_background32(Context& c, int member)
 
 // ---------------------------------------------------------------------------- FP32 grid phase
 // The precision form keeps the projection sums (and the saturation sums and the budget) in FP64;
-// smoothing and divergence run in FP32: GB300's FP64 rate is 1/64 of its FP32 rate, and these
+// smoothing and divergence run in FP32: GB300's FP64 rate is 1/72 of its FP32 rate, and these
 // stencils would otherwise be bound by it.  The smoothing reads the projected FP64 fields and
 // narrows them as it loads (no FP32 copy of the raw fields is written and read back); without
 // smoothing the fields are narrowed once by k_narrow.  du/dt, dv/dt are widened to the caller's

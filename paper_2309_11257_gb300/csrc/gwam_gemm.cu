@@ -130,7 +130,7 @@ __device__ __forceinline__ float gelu_grad(float z)
 }
 
 // Sum of the squares of 32 errors, as accurate as the FP64 sum and over its whole range.  FP64 additions and
-// conversions of every element (1/64 of the FP32 rate) had made this kernel 55 us: the exact products
+// conversions of every element (1/72 of the FP32 rate) had made this kernel 55 us: the exact products
 // (hi, lo) go into unevaluated sums of three FP32 numbers, even and odd columns in the halves of packed pairs, the
 // errors of the two larger ones carried into the next, and only the results are added in FP64 (relative error about
 // 2^-53; a double-float sum, 48 bits, was 1e-14 off after 64 elements).  Where FP32 cannot hold the products to that
@@ -193,7 +193,7 @@ __device__ __forceinline__ void epi32(const GemmEpi& e, int row, int nb, float (
             const int npad = (e.N + 31) & ~31;
             // de-normalised in FP32 (one FMA, relative error 6e-8, far below the BF16 network's) and
             // widened exactly by integer operations: FP64 arithmetic and float -> double conversions
-            // run at 1/64 of the FP32 rate on GB300
+            // run at 1/72 of the FP32 rate on GB300
             if (!live || rowmask != 0) return;
 #pragma unroll
             for (int j = 0; j < 32; j += 4) {
